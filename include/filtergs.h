@@ -137,11 +137,12 @@ typedef struct fgs_stats {
     uint64_t n_pairs;         /* N_P: Gaussian-tile pairs (may exceed capacity on error) */
     uint32_t n_launches;      /* kernels this call enqueued */
     int32_t device_status;    /* latched device status (FGS_OK if none) */
-    uint64_t blend_entries;   /* FGS_RENDER_COUNT: lockstep warp steps of the blend's list walk
-                                 (a step tests one list entry in each half of a warp) */
+    uint64_t blend_entries;   /* FGS_RENDER_COUNT: steps of the blend's list walk (32 pixel
+                                 evaluations each: one list entry of each of a warp's 4x4 blocks, at
+                                 one pixel of each lane) */
     uint64_t blend_evals;     /* FGS_RENDER_COUNT: pixel-Gaussian evaluations (pixels not stopped) */
     uint64_t blend_hits;      /* FGS_RENDER_COUNT: evaluations that reached alpha / T (exp taken) */
-    uint64_t blend_active;    /* FGS_RENDER_COUNT: lockstep steps where some pixel reached it */
+    uint64_t blend_active;    /* FGS_RENDER_COUNT: steps where some pixel reached it */
     uint64_t filter_in_frustum;  /* FGS_RENDER_COUNT: nodes whose centre passes the frustum test */
     uint64_t filter_cov_nodes;   /* FGS_RENDER_COUNT: in-frustum internal nodes, the only ones whose
                                     covariance the R&L filter must read (a leaf passes on the

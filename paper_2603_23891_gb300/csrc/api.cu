@@ -85,6 +85,7 @@ struct fgs_ctx {
     uint32_t* tile_cnt = nullptr;   // pairs per tile, then the tile's scatter cursor
     uint32_t* large = nullptr;      // tiles whose pairs one block sorts
     unsigned long long* lb_scan = nullptr;   // the tile scan's look-back entries
+    uint32_t* heavy = nullptr;      // tiles the blend splits (kSplitTiles)
     float* G = nullptr;
     // image staging for host outputs: rgb planes + T
     size_t img_cap = 0;
@@ -133,7 +134,7 @@ struct fgs_ctx {
         unsigned long long *items = nullptr, *keys = nullptr, *lb_compact = nullptr, *lb_scan = nullptr;
         uint32_t* vals = nullptr;
         uint2* ranges = nullptr;
-        uint32_t *tile_cnt = nullptr, *large = nullptr;
+        uint32_t *tile_cnt = nullptr, *large = nullptr, *heavy = nullptr;
         FrameState* st = nullptr;
         cudaGraphExec_t graph = nullptr;
         float* graph_rgb = nullptr;
@@ -362,7 +363,7 @@ int enqueue_front(fgs_ctx* c, const DevCamera& dc, cudaStream_t s, cudaEvent_t* 
     if (ev) cudaEventRecord(ev[4], s);
     launch_scatter(dc, c->foot, c->tile_cnt, c->keys0, c->pair_cap, c->st, c->sms * c->occ_scatter, s);
     if (ev) cudaEventRecord(ev[5], s);
-    launch_segsort(c->ranges, tiles, c->large, c->keys0, c->keys1, c->vals1, c->st,
+    launch_segsort(c->ranges, tiles, c->large, c->keys0, c->keys1, c->vals1, c->heavy, c->st,
                    c->sms * c->occ_segsort, s);
     if (ev) cudaEventRecord(ev[6], s);
     return 8;
@@ -435,6 +436,7 @@ int fgs_create(fgs_ctx** out, int device)
         cudaMemset(c->st, 0, sizeof(FrameState)) != cudaSuccess ||
         cudaMallocHost((void**)&c->st_host, sizeof(FrameState)) != cudaSuccess)
         r = FGS_ERR_NOMEM;
+    if (r == FGS_OK) r = grow(c, (void**)&c->heavy, 4 * kSplitTiles);
     if (r == FGS_OK) r = ensure_pairs(c, kDefaultPairCap);
     if (r != FGS_OK) {
         fgs_destroy(c);
@@ -453,7 +455,7 @@ int fgs_destroy(fgs_ctx* c)
     void* bufs[] = {c->child_start, c->children, c->frontier0, c->frontier1, c->d_counter,
                     c->tree_mem, c->pbits, c->selbits, c->sel, c->splat, c->lb_compact, c->sel_cnt, c->foot,
                     c->keys0, c->keys1, c->vals0, c->vals1, c->kpc, c->ranges, c->tile_cnt, c->large, c->lb_scan,
-                    c->G, c->img, c->keep, c->st, c->gsplat};
+                    c->G, c->img, c->keep, c->st, c->gsplat, c->heavy};
     for (void* p : bufs) free_ptr(p);
     for (float* p : c->ring) free_ptr(p);
     for (int i = 0; i < 2; ++i) {
@@ -465,7 +467,7 @@ int fgs_destroy(fgs_ctx* c)
         auto& b = c->batch;
         void* bb[] = {b.d_cams, b.d_tile_base, b.d_img_off, b.pbits, b.selbits, b.sel, b.splat,
                       b.foot, b.items, b.keys, b.vals, b.lb_compact, b.lb_scan, b.ranges, b.tile_cnt, b.large,
-                      b.st};
+                      b.heavy, b.st};
         for (void* p : bb) free_ptr(p);
         if (b.h_cams) cudaFreeHost(b.h_cams);
         if (b.graph) cudaGraphExecDestroy(b.graph);
@@ -864,7 +866,7 @@ int fgs_render(fgs_ctx* c, void* stream, float* rgb_out, float* T_out, int out_i
     if (count) flags |= FGS_RENDER_STATS;
     // the image two frames back must have reached the host before it is overwritten
     if (pipelined && c->ring_busy[slot]) FGS_CUDA(c, cudaStreamWaitEvent(s, c->ev_copied[slot], 0));
-    launch_blend(dc, c->ranges, c->vals1, c->splat, rgb_dst, T_dst, keep ? c->keep : nullptr, c->st, count, s);
+    launch_blend(dc, c->ranges, c->heavy, c->vals1, c->splat, rgb_dst, T_dst, keep ? c->keep : nullptr, c->st, count, s);
     ++launches;
     if (ev) cudaEventRecord(ev[kStages], s);
     FGS_CUDA(c, cudaGetLastError());
@@ -1159,7 +1161,7 @@ int fgs_backward(fgs_ctx* c, void* stream, const float* dL_drgb, const fgs_gauss
     cudaStream_t s = (cudaStream_t)stream;
     const float* params[5] = {p->mu, p->log_scale, p->quat, p->logit, p->sh};
     float* grads[5] = {gr->mu, gr->log_scale, gr->quat, gr->logit, gr->sh};
-    launch_backward(c->tree, dc, c->ranges, c->vals1, c->splat, c->keep, c->frame_kept, c->sel,
+    launch_backward(c->tree, dc, c->ranges, c->heavy, c->vals1, c->splat, c->keep, c->frame_kept, c->sel,
                     dL_drgb, c->gsplat, params, grads, (flags & FGS_BACKWARD_ACCUMULATE) != 0, c->sms, c->st,
                     s);
     FGS_CUDA(c, cudaGetLastError());
@@ -1242,6 +1244,7 @@ int fgs_batch_setup(fgs_ctx* c, const fgs_camera* views, int n_views, const int3
     if ((r = grow(c, (void**)&b.large, 4 * b.total_tiles))) return r;
     if (!b.st) {
         if ((r = grow(c, (void**)&b.st, sizeof(FrameState)))) return r;
+        if ((r = grow(c, (void**)&b.heavy, 4 * kSplitTiles))) return r;
     }
     FGS_CUDA(c, cudaMemcpy(b.d_tile_base, b.tile_base.data(), 4 * (n_views + 1), cudaMemcpyHostToDevice));
     FGS_CUDA(c, cudaMemcpy(b.d_img_off, b.img_off.data(), 8 * (n_views + 1), cudaMemcpyHostToDevice));
@@ -1278,9 +1281,9 @@ void enqueue_batch(fgs_ctx* c, float* rgb, float* T, cudaStream_t s)
 {
     auto& b = c->batch;
     launch_batch_front(c->tree, b.d_cams, b.V, b.total_tiles, b.d_tile_base, b.pbits, b.selbits, b.sel,
-                       (uint32_t)b.sel_cap, b.splat, b.foot, b.tile_cnt, b.large, b.items, b.keys, b.vals,
+                       (uint32_t)b.sel_cap, b.splat, b.foot, b.tile_cnt, b.large, b.heavy, b.items, b.keys, b.vals,
                        b.pair_cap, b.lb_compact, b.lb_scan, b.ranges, b.st, c->sms, s);
-    launch_batch_blend(b.d_cams, b.V, b.total_tiles, b.d_tile_base, b.d_img_off, b.ranges, b.vals, b.splat,
+    launch_batch_blend(b.d_cams, b.V, b.total_tiles, b.d_tile_base, b.d_img_off, b.ranges, b.heavy, b.vals, b.splat,
                        rgb, T, b.st, s);
 }
 

@@ -17,7 +17,6 @@
 // applies the chain rule to the parameters.
 #include "blend_impl.cuh"
 
-#include <type_traits>
 #include "project_impl.cuh"
 
 namespace fgs {
@@ -145,9 +144,7 @@ __global__ void __launch_bounds__(256) prep_sh_kernel(DevTree t, const float* __
 // ---------------------------------------------------------------------------
 // blend backward
 // ---------------------------------------------------------------------------
-// Shared memory of the blend backward: the forward's half-block walk (used to
-// recompute each pixel's final T and stop position) and the back-to-front
-// gradient walk over half-block lists, one after the other.
+// Shared memory of the back-to-front gradient walk over half-block lists.
 struct BwdWalkSmem {
     uint32_t vals[blendk::kValsSlots];
     float4 g0[blendk::kChunk];                  // u, v, A', B'
@@ -160,13 +157,6 @@ struct BwdWalkSmem {
     uint64_t bar;
     int timed_out;
 };
-union BwdSmem {
-    blendk::HalfSmem fwd;
-    BwdWalkSmem bwd;
-};
-__device__ __forceinline__ BwdWalkSmem& walk_smem(BwdSmem& b) { return b.bwd; }
-__device__ __forceinline__ BwdWalkSmem& walk_smem(BwdWalkSmem& b) { return b; }
-
 // Sum over each half-warp (16 lanes) of v[0..8], scattered: on return the lane
 // given by half_component() holds its half's sum of that component.  Recursive
 // halving within the half (xor 8, 4, 2, 1 split the value set): 11 shuffles.
@@ -203,31 +193,21 @@ __device__ __forceinline__ int half_component(uint32_t lane)
     return (pb < 3 && pa < 5 && comp < 9) ? comp : -1;
 }
 
-// kKept: the forward kept {final T, stop} per pixel (FGS_RENDER_KEEP) in keep.
-// Otherwise the forward's own half-block walk runs first, without colour, and
-// writes them there.  Then the tile is walked back to front over half-block
-// lists (a 4x4 half-warp tests only the Gaussians whose threshold box meets
-// it, as in the forward), the two halves of a warp in lockstep, each from its
-// list's last entry before its last stop.
-template <bool kKept>
+// keep holds each pixel's {final T, stop} (kept by a FGS_RENDER_KEEP forward, or
+// recomputed by the forward's walk without an image just before).  The tile is
+// walked back to front over half-block lists (a 4x4 half-warp tests only the
+// Gaussians whose threshold box meets it), the two halves of a warp in lockstep,
+// each from its list's last entry before its last stop.
 __global__ void __launch_bounds__(256) blend_bwd_kernel(DevCamera cam, const uint2* __restrict__ ranges,
                                                         const uint32_t* __restrict__ vals,
                                                         const float* __restrict__ splat,
-                                                        uint2* __restrict__ keep,
+                                                        const uint2* __restrict__ keep,
                                                         const float* __restrict__ dL_drgb,
                                                         float* __restrict__ gsplat, FrameState* st)
 {
-    // (with kept state the forward walk's shared memory is not needed)
-    __shared__ __align__(128) typename std::conditional<kKept, BwdWalkSmem, BwdSmem>::type B;
+    __shared__ __align__(128) BwdWalkSmem S;
     const uint32_t tile = blockIdx.x;
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    if constexpr (!kKept) {
-        blendk::blend_tile_half<false, true>(cam, tile, tile, B.fwd, ranges, vals, splat, nullptr, nullptr,
-                                            keep, st);
-        __syncthreads();
-        if (B.fwd.timed_out) return;
-    }
-    BwdWalkSmem& S = walk_smem(B);
     const int32_t tx0 = (int32_t)(tile % (uint32_t)cam.tiles_x) * cam.tile_w;
     const int32_t ty0 = (int32_t)(tile / (uint32_t)cam.tiles_x) * cam.tile_h;
     int32_t wx0, wy0;
@@ -685,19 +665,16 @@ static void launch_project_bwd(const DevTree& t, const DevCamera& cam, const Par
         project_bwd_kernel<kDeg, false><<<blocks, kPbWarps * 32, 0, s>>>(t, cam, p, sel, gsplat, gr, st);
 }
 
-void launch_backward(const DevTree& t, const DevCamera& cam, const uint2* ranges, const uint32_t* vals,
+void launch_backward(const DevTree& t, const DevCamera& cam, const uint2* ranges, const uint32_t* heavy,
+                     const uint32_t* vals,
                      const float* splat, uint2* keep, bool kept, const uint32_t* sel, const float* dL_drgb,
                      float* gsplat, const float* const params[5], float* const grads[5], bool accumulate,
                      int sms, FrameState* st, cudaStream_t s)
 {
     // gsplat rows of the selected Gaussians start at zero: the blend backward adds into them
     zero_rows_kernel<<<sms * 8, 128, 0, s>>>(reinterpret_cast<float4*>(gsplat), st);
-    if (kept)
-        blend_bwd_kernel<true><<<cam.tiles_x * cam.tiles_y, 256, 0, s>>>(cam, ranges, vals, splat, keep, dL_drgb,
-                                                                     gsplat, st);
-    else
-        blend_bwd_kernel<false><<<cam.tiles_x * cam.tiles_y, 256, 0, s>>>(cam, ranges, vals, splat, keep,
-                                                                      dL_drgb, gsplat, st);
+    if (!kept) launch_blend(cam, ranges, heavy, vals, splat, nullptr, nullptr, keep, st, false, s);
+    blend_bwd_kernel<<<cam.tiles_x * cam.tiles_y, 256, 0, s>>>(cam, ranges, vals, splat, keep, dL_drgb, gsplat, st);
     const ParamPtrs p{params[0], params[1], params[2], params[3], params[4], t.n};
     const GradPtrs gr{grads[0], grads[1], grads[2], grads[3], grads[4]};
     if (!accumulate) {

@@ -201,32 +201,43 @@ __global__ void __launch_bounds__(kProjThreads) bproject_kernel(
     }
 }
 
-// Blend every tile of every view; the CTA's view is found by binary search.
-__global__ void __launch_bounds__(256) bblend_kernel(const DevCamera* __restrict__ cams, int V,
-                                                     const uint32_t* __restrict__ tile_base,
-                                                     const unsigned long long* __restrict__ img_off,
-                                                     const uint2* __restrict__ ranges,
-                                                     const uint32_t* __restrict__ vals,
-                                                     const float* __restrict__ splat,
-                                                     float* __restrict__ rgb, float* __restrict__ Tout,
-                                                     FrameState* st)
+// Blend every tile of every view; the tile's view is found by binary search.
+__global__ void __launch_bounds__(blendk::kWalkChunk) bblend_kernel(
+    const DevCamera* __restrict__ cams, int V, uint32_t total_tiles, const uint32_t* __restrict__ tile_base,
+    const unsigned long long* __restrict__ img_off, const uint2* __restrict__ ranges,
+    const uint32_t* __restrict__ heavy, const uint32_t* __restrict__ vals, const float* __restrict__ splat,
+    float* __restrict__ rgb, float* __restrict__ Tout, FrameState* st)
 {
-    __shared__ __align__(128) blendk::HalfSmem H;
+    __shared__ __align__(128) blendk::WalkSmem<false> S;
     __shared__ DevCamera s_cam;
-    const uint32_t gtile = blockIdx.x;
-    int lo = 0, hi = V;                            // largest v with tile_base[v] <= gtile
-    while (hi - lo > 1) {
-        const int mid = (lo + hi) >> 1;
-        if (__ldg(tile_base + mid) <= gtile) lo = mid;
-        else hi = mid;
-    }
-    const int v = lo;
-    for (int i = threadIdx.x; i < (int)(sizeof(DevCamera) / 4); i += blockDim.x)
-        reinterpret_cast<uint32_t*>(&s_cam)[i] = reinterpret_cast<const uint32_t*>(cams + v)[i];
-    __syncthreads();
-    const unsigned long long o = __ldg(img_off + v);
-    blendk::blend_tile_half(s_cam, gtile - __ldg(tile_base + v), gtile, H, ranges, vals, splat, rgb + 3 * o,
-                            Tout ? Tout + o : nullptr, nullptr, st);
+    // the tile's view: its camera to s_cam; first tile and image offset
+    auto locate = [&](uint32_t gtile, uint32_t& base) {
+        int lo = 0, hi = V;                            // largest v with tile_base[v] <= gtile
+        while (hi - lo > 1) {
+            const int mid = (lo + hi) >> 1;
+            if (__ldg(tile_base + mid) <= gtile) lo = mid;
+            else hi = mid;
+        }
+        for (int i = threadIdx.x; i < (int)(sizeof(DevCamera) / 4); i += blockDim.x)
+            reinterpret_cast<uint32_t*>(&s_cam)[i] = reinterpret_cast<const uint32_t*>(cams + lo)[i];
+        __syncthreads();
+        base = __ldg(tile_base + lo);
+        return __ldg(img_off + lo);
+    };
+    blendk::walk_grid(
+        total_tiles, ranges, heavy, st,
+        [&](uint32_t gtile, uint2 rg) {
+            uint32_t base;
+            const unsigned long long o = locate(gtile, base);
+            blendk::blend_walk<8, false, false>(s_cam, gtile - base, 0u, rg, S, vals, splat, rgb + 3 * o,
+                                                Tout ? Tout + o : nullptr, nullptr, st);
+        },
+        [&](uint32_t gtile, uint32_t part, uint2 rg) {
+            uint32_t base;
+            const unsigned long long o = locate(gtile, base);
+            blendk::blend_walk<16, false, false>(s_cam, gtile - base, part, rg, S, vals, splat, rgb + 3 * o,
+                                                 Tout ? Tout + o : nullptr, nullptr, st);
+        });
 }
 
 // ---------------------------------------------------------------------------
@@ -234,7 +245,7 @@ __global__ void __launch_bounds__(256) bblend_kernel(const DevCamera* __restrict
 // ---------------------------------------------------------------------------
 void launch_batch_front(const DevTree& t, const DevCamera* cams, int V, uint32_t total_tiles,
                         const uint32_t* tile_base, uint32_t* pbits, uint32_t* selbits, uint32_t* sel,
-                        uint32_t sel_cap, float* splat, uint4* foot, uint32_t* tile_cnt, uint32_t* large,
+                        uint32_t sel_cap, float* splat, uint4* foot, uint32_t* tile_cnt, uint32_t* large, uint32_t* heavy,
                         unsigned long long* items, unsigned long long* keys, uint32_t* vals,
                         unsigned long long cap, unsigned long long* lb_compact, unsigned long long* lb_scan,
                         uint2* ranges, FrameState* st, int sms, cudaStream_t s)
@@ -254,14 +265,17 @@ void launch_batch_front(const DevTree& t, const DevCamera* cams, int V, uint32_t
                                                                        foot, tile_cnt, st);
     launch_tile_scan(tile_cnt, ranges, total_tiles, large, cap, lb_scan, st, sms * occ_tile_scan(), s);
     launch_scatter_batch(cams, tile_base, t.n_pad, sel, foot, tile_cnt, items, cap, st, sms * occ_scatter(), s);
-    launch_segsort(ranges, total_tiles, large, items, keys, vals, st, sms * occ_segsort(), s);
+    launch_segsort(ranges, total_tiles, large, items, keys, vals, heavy, st, sms * occ_segsort(), s);
 }
 
 void launch_batch_blend(const DevCamera* cams, int V, uint32_t total_tiles, const uint32_t* tile_base,
-                        const unsigned long long* img_off, const uint2* ranges, const uint32_t* vals,
-                        const float* splat, float* rgb, float* T, FrameState* st, cudaStream_t s)
+                        const unsigned long long* img_off, const uint2* ranges, const uint32_t* heavy,
+                        const uint32_t* vals, const float* splat, float* rgb, float* T, FrameState* st,
+                        cudaStream_t s)
 {
-    bblend_kernel<<<total_tiles, 256, 0, s>>>(cams, V, tile_base, img_off, ranges, vals, splat, rgb, T, st);
+    const uint32_t grid = total_tiles + 2u * (uint32_t)split_slots((int)total_tiles);
+    bblend_kernel<<<grid, blendk::kWalkChunk, 0, s>>>(cams, V, total_tiles, tile_base, img_off, ranges, heavy, vals,
+                                                      splat, rgb, T, st);
 }
 
 }  // namespace fgs

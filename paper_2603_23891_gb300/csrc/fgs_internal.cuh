@@ -24,6 +24,7 @@ constexpr int kFilterTile = 4096;         // node arrays are padded to a multipl
 constexpr int kCompactWords = 1024;       // 32-bit selection words per compaction tile (32K nodes)
 constexpr int kSelTileWords = 256;        // words per counted tile (the Ancestor filter's sel_cnt)
 constexpr int kAncCacheWords = 4096;      // P-bit words of the lowest node ids kept in shared memory
+constexpr uint32_t kSplitTiles = 912;      // fewer tiles than that of a blend are split (6 an SM)
 constexpr int kProjThreads = 256;         // selected Gaussians per projection tile
 constexpr uint64_t kSpinLimit = 1ull << 24;   // bounded spin-waits
 
@@ -93,7 +94,7 @@ struct FrameState {
 };
 
 // Ticket slots
-enum : int { kTicketCompact = 0, kTicketSegSort = 2, kTicketScan = 4, kTicketLarge = 5 };
+enum : int { kTicketCompact = 0, kTicketSegSort = 2, kTicketScan = 4, kTicketLarge = 5, kTicketHeavy = 6 };
 
 // ---------------------------------------------------------------------
 // decision-exact binary32 helpers
@@ -262,6 +263,19 @@ __device__ __forceinline__ void ewa_cov2d(const DevCamera& cam, float vz, float 
 // ---------------------------------------------------------------------
 // bounded look-back / spin helpers
 // ---------------------------------------------------------------------
+// Pairs above which a tile is split over two CTAs by the blend (blend_impl.cuh): a
+// tile with more than 1 / kSplitTiles of the frame's pairs, more than the even share of
+// one of the 6 x 152 resident CTAs.  Walked whole its end may be the frame's end.  City
+// flythrough, blend with every tile whole / split above 1/456 / above 1/912 of the pairs:
+// 168 / 133 / 113 us where one tile holds 3,473 of 1.08M pairs, 148 / 152 / 131 us for
+// 2,299 of 1.44M, 111 / 113 / 111 us for 1,834 of 1.12M.  By the definition there are
+// fewer than kSplitTiles of them; in a small frame most tiles with pairs are.
+__device__ __forceinline__ uint32_t split_pairs(unsigned long long n_pairs)
+{
+    return (uint32_t)(n_pairs / kSplitTiles);
+}
+inline int split_slots(int n_tiles) { return n_tiles < (int)kSplitTiles ? n_tiles : (int)kSplitTiles; }
+
 // Look-back entries carry their whole payload (epoch tag, flag, count) in one
 // 64-bit word and publish no other data, so relaxed device-scope accesses
 // suffice (no acquire / release ordering is needed around them).
@@ -431,11 +445,13 @@ void launch_scatter_batch(const DevCamera* cams, const uint32_t* tile_base, uint
                           cudaStream_t s);
 // Sorts every tile's bucket of items[] into keys_out (tile << 32 | depth bits)
 // and vals_out (rank), in place of the bucket's slots.
+// Lists the tiles the blend splits (split_pairs) in heavy[kSplitTiles], their number in
+// FrameState::tickets[kTicketHeavy].
 void launch_segsort(const uint2* ranges, uint32_t n_tiles, const uint32_t* large, unsigned long long* items,
-                    unsigned long long* keys_out, uint32_t* vals_out, FrameState* st, int blocks,
+                    unsigned long long* keys_out, uint32_t* vals_out, uint32_t* heavy, FrameState* st, int blocks,
                     cudaStream_t s);
 // count: use the counting variant (fills FrameState::blend_* work counters)
-void launch_blend(const DevCamera& cam, const uint2* ranges, const uint32_t* vals,
+void launch_blend(const DevCamera& cam, const uint2* ranges, const uint32_t* heavy, const uint32_t* vals,
                   const float* splat, float* rgb, float* T, uint2* keep, FrameState* st, bool count,
                   cudaStream_t s);
 void launch_blend_kpc(const DevCamera& cam, const uint2* ranges, const uint32_t* vals,
@@ -444,18 +460,19 @@ void launch_blend_kpc(const DevCamera& cam, const uint2* ranges, const uint32_t*
 void launch_eval_exp(const float* x, float* y, uint64_t n, cudaStream_t s);
 void launch_batch_front(const DevTree& t, const DevCamera* cams, int V, uint32_t total_tiles,
                         const uint32_t* tile_base, uint32_t* pbits, uint32_t* selbits, uint32_t* sel,
-                        uint32_t sel_cap, float* splat, uint4* foot, uint32_t* tile_cnt, uint32_t* large,
+                        uint32_t sel_cap, float* splat, uint4* foot, uint32_t* tile_cnt, uint32_t* large, uint32_t* heavy,
                         unsigned long long* items, unsigned long long* keys, uint32_t* vals,
                         unsigned long long cap, unsigned long long* lb_compact, unsigned long long* lb_scan, uint2* ranges,
                         FrameState* st, int sms, cudaStream_t s);
 void launch_batch_blend(const DevCamera* cams, int V, uint32_t total_tiles, const uint32_t* tile_base,
-                        const unsigned long long* img_off, const uint2* ranges, const uint32_t* vals,
-                        const float* splat, float* rgb, float* T, FrameState* st, cudaStream_t s);
+                        const unsigned long long* img_off, const uint2* ranges, const uint32_t* heavy,
+                        const uint32_t* vals, const float* splat, float* rgb, float* T, FrameState* st, cudaStream_t s);
 void launch_prep_params(const DevTree& t, const float* mu, const float* log_scale, const float* quat,
                         const float* logit, const float* sh, int blocks, cudaStream_t s);
 // keep: per-pixel {final T, stop} buffer; kept: the last forward filled it
-// (FGS_RENDER_KEEP), otherwise the blend backward recomputes it there.
-void launch_backward(const DevTree& t, const DevCamera& cam, const uint2* ranges, const uint32_t* vals,
+// (FGS_RENDER_KEEP), otherwise the forward's walk runs again and fills it.
+void launch_backward(const DevTree& t, const DevCamera& cam, const uint2* ranges, const uint32_t* heavy,
+                     const uint32_t* vals,
                      const float* splat, uint2* keep, bool kept, const uint32_t* sel, const float* dL_drgb,
                      float* gsplat,
                      const float* const params[5], float* const grads[5], bool accumulate, int proj_blocks,

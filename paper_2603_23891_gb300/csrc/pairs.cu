@@ -889,12 +889,21 @@ __global__ void __launch_bounds__(kProjThreads) scatter_kernel(
 // ---------------------------------------------------------------------------
 // per-tile sort
 // ---------------------------------------------------------------------------
+// A tile of more than `split` pairs into the list of those the blend splits (one
+// thread; fewer than kSplitTiles exist).
+__device__ __forceinline__ void list_heavy(uint32_t n, uint32_t split, uint32_t tile, uint32_t* heavy, FrameState* st)
+{
+    if (n <= split) return;
+    const uint32_t k = atomicAdd(&st->tickets[kTicketHeavy], 1u);
+    if (k < kSplitTiles) heavy[k] = tile;
+}
+
 __global__ void __launch_bounds__(kSegThreads) segsort_kernel(const uint2* __restrict__ ranges,
                                                               uint32_t n_tiles,
                                                               const uint32_t* __restrict__ large,
                                                               unsigned long long* items,
                                                               unsigned long long* keys_out,
-                                                              uint32_t* vals_out, FrameState* st)
+                                                              uint32_t* vals_out, uint32_t* heavy, FrameState* st)
 {
     __shared__ __align__(16) unsigned long long s_items[kSegSmem];
     __shared__ RadixSmem s_radix;
@@ -904,6 +913,7 @@ __global__ void __launch_bounds__(kSegThreads) segsort_kernel(const uint2* __res
     // large buckets first: one block each; a block's first bucket is its index,
     // later ones come from a ticket counter
     const uint32_t n_large = st->tickets[kTicketLarge];
+    const uint32_t split = split_pairs(st->n_pairs);
     bool first = true;
     for (;;) {
         if (threadIdx.x == 0)
@@ -917,6 +927,7 @@ __global__ void __launch_bounds__(kSegThreads) segsort_kernel(const uint2* __res
         const uint2 r = ranges[t];
         const uint32_t n = r.y - r.x;
         unsigned long long* it = items + r.x;
+        if (threadIdx.x == 0) list_heavy(n, split, t, heavy, st);
         if (n <= (uint32_t)kSegSmem) {
             uint32_t* sk = reinterpret_cast<uint32_t*>(s_items);
             bool done;
@@ -943,6 +954,7 @@ __global__ void __launch_bounds__(kSegThreads) segsort_kernel(const uint2* __res
         const uint32_t n = r.y - r.x;
         if (n == 0u || n > (uint32_t)kSegSmall) continue;
         const unsigned long long* it = items + r.x;
+        if ((threadIdx.x & 31u) == 0u) list_heavy(n, split, t, heavy, st);
         bool done = true;
         if (n <= 32u) warp_sort_bucket<1>(it, n, t, keys_out + r.x, vals_out + r.x);
         else if (n <= 64u) done = warp_radix_small<2>(it, n, t, keys_out + r.x, vals_out + r.x, wbuf, whist);
@@ -997,12 +1009,12 @@ void launch_scatter_batch(const DevCamera* cams, const uint32_t* tile_base, uint
 }
 
 void launch_segsort(const uint2* ranges, uint32_t n_tiles, const uint32_t* large, unsigned long long* items,
-                    unsigned long long* keys_out, uint32_t* vals_out, FrameState* st, int blocks,
+                    unsigned long long* keys_out, uint32_t* vals_out, uint32_t* heavy, FrameState* st, int blocks,
                     cudaStream_t s)
 {
     if (blocks < 1) blocks = 1;
     launch_pdl(segsort_kernel, blocks, kSegThreads, 0, s, ranges, n_tiles, large, items, keys_out, vals_out,
-               st);
+               heavy, st);
 }
 
 int occ_scatter()
