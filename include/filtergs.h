@@ -442,12 +442,12 @@ int fgs_update_params(fgs_ctx* ctx, void* stream, const fgs_gauss_params* p);
  * rgb_out).  p: the parameters of that render; g: gradient arrays of the same
  * shapes (device).  Without FGS_BACKWARD_ACCUMULATE every entry of g is
  * written (zero for nodes outside the cut); with it, the selected nodes'
- * gradients are added.  Two kernels: a per-tile blend backward that
- * recomputes each pixel's final transmittance and stop position by a
- * front-to-back walk over its tile (or reads them, if the render used
- * FGS_RENDER_KEEP) and then walks the tile back to front, recovering T before
- * each Gaussian as T / (1 - alpha); and a per-Gaussian chain rule through the
- * conic, the EWA Jacobian, Sigma(q, s), the sigmoid and the SH basis.
+ * gradients are added.  A per-tile blend backward walks the tile back to front
+ * from each pixel's final transmittance and stop position (kept by the render
+ * with FGS_RENDER_KEEP, or recomputed by running the forward's walk once more
+ * without an image), recovering T before each Gaussian as T / (1 - alpha); then
+ * a per-Gaussian chain rule goes through the conic, the EWA Jacobian,
+ * Sigma(q, s), the sigmoid and the SH basis.
  * Asynchronous on `stream`.  Errors: FGS_ERR_STATE (no rendered frame since
  * the last change of tree, camera, parameters or settings), FGS_ERR_ARG,
  * FGS_ERR_NOMEM, FGS_ERR_CUDA. */

@@ -6,15 +6,14 @@
 // mean mu, log-scale s, quaternion q (any norm), opacity logit l, SH
 // coefficients; Sigma = R(q/|q|) diag(e^{2s}) R^T, alpha0 = sigmoid(l).
 //
-// blend_bwd_kernel recomputes each pixel's final transmittance and stop
-// position by a front-to-back walk over its tile with the forward's exact
-// decisions (or, after a FGS_RENDER_KEEP forward, reads the 8 bytes per pixel
-// the forward kept), then walks the tile back to front, recovering T before
-// each Gaussian as T / (1 - alpha) and accumulating the colour behind it;
-// chunks past the last stop of the tile are never loaded.  Gradients with respect to the splat record (u, v,
-// conic A B C, alpha0, colour) are reduced per warp (a transposed reduction:
-// 12 shuffles for 9 values) and added per Gaussian; project_bwd_kernel then
-// applies the chain rule to the parameters.
+// blend_bwd_kernel starts from each pixel's final transmittance and stop position (the
+// 8 bytes per pixel that a FGS_RENDER_KEEP forward kept, or that the forward's walk,
+// run once more without an image, leaves) and walks the tile back to front,
+// recovering T before each Gaussian as T / (1 - alpha); chunks past the last stop of
+// the tile are never loaded.  The gradients with respect to the splat record (u, v,
+// conic A B C, alpha0, colour) of a Gaussian are summed over a 4x4 block of pixels by one lane
+// and added per Gaussian; project_bwd_kernel then applies the chain rule to the
+// parameters.
 #include "blend_impl.cuh"
 
 #include "project_impl.cuh"
@@ -144,204 +143,333 @@ __global__ void __launch_bounds__(256) prep_sh_kernel(DevTree t, const float* __
 // ---------------------------------------------------------------------------
 // blend backward
 // ---------------------------------------------------------------------------
-// Shared memory of the back-to-front gradient walk over half-block lists.
-struct BwdWalkSmem {
-    uint32_t vals[blendk::kValsSlots];
-    float4 g0[blendk::kChunk];                  // u, v, A', B'
-    float4 g1[blendk::kChunk];                  // C', lthr, alpha0, depth
-    float4 g2[blendk::kChunk];                  // r, g, b, radius
-    uint32_t m[blendk::kChunk];                 // selected rank of each chunk entry
-    uint16_t hmask[blendk::kChunk];
-    alignas(16) uint8_t hl[blendk::kHalfBlocks][blendk::kChunk];
-    uint32_t hlim[blendk::kHalfBlocks];         // last stop position of each half-block
-    uint64_t bar;
-    int timed_out;
+// Shared memory of the back-to-front gradient walk.
+struct BwdWarp {                                                  // one warp's: 32 entries at a time
+    float n[32][blendk::kParkStride];                             // -power at a block's 16 pixels
+    float w[32][blendk::kParkStride];                             // alpha T, 0 where the entry is not applied
+    float g[32][blendk::kParkStride];                             // dL/dpower, 0 likewise
+    float4 col[32];                                               // alpha0, r, g, b
+    uint8_t list[4][blendk::kWalkChunk];                          // per block: the chunk's records it may meet
 };
-// Sum over each half-warp (16 lanes) of v[0..8], scattered: on return the lane
-// given by half_component() holds its half's sum of that component.  Recursive
-// halving within the half (xor 8, 4, 2, 1 split the value set): 11 shuffles.
-__device__ __forceinline__ float half_reduce9(const float v[9], uint32_t lane)
+struct BwdSmem {
+    float4 r0[blendk::kWalkChunk];                                // u, v, A, B
+    float4 r1[blendk::kWalkChunk];                                // C, lthr, alpha0, depth
+    float4 r2[blendk::kWalkChunk];                                // r, g, b, radius
+    uint16_t mask[blendk::kWalkChunk];
+    float dC[3][256];                                             // dL/dC by block, in the parked order
+    uint32_t last[blendk::kWalkWarps];
+    BwdWarp w[blendk::kWalkWarps];
+};
+
+// 1 / x for x in [0.01, 1]: the approximate reciprocal and one Newton step.
+__device__ __forceinline__ float rcp1(float x)
 {
-    const bool b3 = lane & 8, b2 = lane & 4, b1 = lane & 2, b0 = lane & 1;
-    float a[5];
-#pragma unroll
-    for (int i = 0; i < 5; ++i) {
-        const float lo = v[i], hi = (5 + i < 9) ? v[5 + i] : 0.0f;
-        a[i] = (b3 ? hi : lo) + __shfl_xor_sync(0xffffffffu, b3 ? lo : hi, 8);
-    }
-    float b[3];
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-        const float lo = a[i], hi = (3 + i < 5) ? a[3 + i] : 0.0f;
-        b[i] = (b2 ? hi : lo) + __shfl_xor_sync(0xffffffffu, b2 ? lo : hi, 4);
-    }
-    float c[2];
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {
-        const float lo = b[i], hi = (2 + i < 3) ? b[2 + i] : 0.0f;
-        c[i] = (b1 ? hi : lo) + __shfl_xor_sync(0xffffffffu, b1 ? lo : hi, 2);
-    }
-    return (b0 ? c[1] : c[0]) + __shfl_xor_sync(0xffffffffu, b0 ? c[0] : c[1], 1);
+    float r;
+    asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return fmaf(r, fmaf(-x, r, 1.0f), r);
 }
 
-// Component whose half sum half_reduce9 leaves in this lane (-1: padding).
-__device__ __forceinline__ int half_component(uint32_t lane)
+// Gradient walk of a tile (kLanes = 8) or its half `part` (kLanes = 16), laid out as the
+// forward's walk (blend_walk): lanes, blocks, chunks, lists and the test are the same,
+// the chunks and the lists' groups of kLanes entries taken from the last to the first.
+// keep holds each pixel's {final T, stop}; a pixel takes part in the list entries
+// before its stop.  Per group of entries:
+//  * test: a lane an entry, as in the forward;
+//  * apply: a lane its own pixels' hits, back to front: T before the entry is
+//    T / (1 - alpha), D = dL/dC . (colour behind) follows, and w = alpha T and
+//    dL/dpower are parked for (entry, pixel);
+//  * gather: a lane an entry again: the sums over the block's 16 pixels of w dL/dC and
+//    of dL/dpower times 1, dx, dy, dx^2, dx dy, dy^2, two pixels to an instruction, from
+//    which the splat's nine gradients follow, added with three reductions (two of four
+//    floats).  (With a lane a pixel throughout, every list entry cost 9 products, 11
+//    shuffles and 9 reductions for 32 pixels, hit or not: about 130 instructions.)
+// Bound: instruction issue.
+template <int kLanes>
+__device__ __forceinline__ void blend_bwd_walk(const DevCamera& cam, uint32_t tile, uint32_t part, uint2 rg,
+                                               BwdSmem& S, const uint32_t* __restrict__ vals,
+                                               const float* __restrict__ splat, const uint2* __restrict__ keep,
+                                               const float* __restrict__ dL_drgb, float* __restrict__ gsplat,
+                                               const FrameState* st)
 {
-    const int pb = 2 * ((lane >> 1) & 1) + (lane & 1);
-    const int pa = 3 * ((lane >> 2) & 1) + pb;
-    const int comp = 5 * ((lane >> 3) & 1) + pa;
-    return (pb < 3 && pa < 5 && comp < 9) ? comp : -1;
+    using namespace blendk;
+    constexpr bool kTwo = kLanes == 8;                             // pixels a lane
+    constexpr uint32_t kC = kWalkChunk, kBlocks = 32 / kLanes;
+    constexpr uint32_t kPx0 = kTwo ? 0xAAAAu : 0xFFFFu, kPx1 = kTwo ? 0x5555u : 0u;      // mask bits a pixel
+    const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint32_t b = lane / kLanes, i = lane % kLanes;
+    const uint32_t M = st->M;
+    BwdWarp& W = S.w[warp];
+    const int32_t tx0 = (int32_t)(tile % (uint32_t)cam.tiles_x) * cam.tile_w;
+    const int32_t ty0 = (int32_t)(tile / (uint32_t)cam.tiles_x) * cam.tile_h;
+    const uint32_t fb = kTwo ? 4u * warp : 8u * part + 2u * warp;
+    int32_t ox, oy;
+    uint32_t bsh;
+    walk_origin(cam, fb >> 2, ox, oy, bsh);
+    const uint32_t bb = (fb & 3u) + b;
+    const int32_t bx0 = tx0 + ox + (int32_t)((bb & ((1u << bsh) - 1u)) << 2);
+    const int32_t by0 = ty0 + oy + (int32_t)((bb >> bsh) << 2);
+    const uint32_t pp = kTwo ? i : i >> 1;
+    const int32_t x = bx0 + (int32_t)(pp & 3u);
+    const int32_t y = by0 + (int32_t)(pp >> 2 << 1) + (kTwo ? 0 : 1 - (int32_t)(i & 1u));
+    const uint32_t park = kTwo ? 2u * i : i ^ 1u;                  // the first pixel's place in the parked order
+
+    // the pixels' forward outcome: final T, stop position; dL/dC
+    f32x2 T, dC0, dC1, dC2;
+    uint32_t lim[2] = {rg.x, rg.x};
+    {
+        float t[2] = {1.0f, 1.0f}, d[3][2] = {};
+        const size_t hw = (size_t)cam.width * cam.height;
+#pragma unroll
+        for (int k = 0; k < (kTwo ? 2 : 1); ++k) {
+            if (x < cam.width && y + k < cam.height) {
+                const size_t pix = (size_t)(y + k) * cam.width + x;
+                const uint2 kp = __ldg(keep + pix);
+                t[k] = __uint_as_float(kp.x);
+                lim[k] = kp.y;
+#pragma unroll
+                for (int c = 0; c < 3; ++c) d[c][k] = __ldg(dL_drgb + c * hw + pix);
+            }
+#pragma unroll
+            for (int c = 0; c < 3; ++c) S.dC[c][32u * kBlocks / 2u * warp + 16u * b + park + k] = d[c][k];
+        }
+        T = pack2(t[0], t[1]);
+        dC0 = pack2(d[0][0], d[0][1]);
+        dC1 = pack2(d[1][0], d[1][1]);
+        dC2 = pack2(d[2][0], d[2][1]);
+    }
+    // dL/dC . colour behind
+    f32x2 D = mul2(mul2(dC0, dup2(cam.bg[0])), T);
+    D = fma2(mul2(dC1, dup2(cam.bg[1])), T, D);
+    D = fma2(mul2(dC2, dup2(cam.bg[2])), T, D);
+
+    // the blocks' last stops, and the walk's
+    uint32_t blim = max(lim[0], lim[1]);
+#pragma unroll
+    for (int o = kLanes / 2; o > 0; o >>= 1) blim = max(blim, __shfl_xor_sync(kFull, blim, o));
+    uint32_t bl[kBlocks];
+#pragma unroll
+    for (uint32_t k = 0; k < kBlocks; ++k) bl[k] = __shfl_sync(kFull, blim, k * kLanes);
+    uint32_t e = bl[0];
+#pragma unroll
+    for (uint32_t k = 1; k < kBlocks; ++k) e = max(e, bl[k]);
+    if (lane == 0) S.last[warp] = e;
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < kWalkWarps; ++k) e = max(e, S.last[k]);
+    e = min(e, rg.y);                    // no pixel of the tile (half) reaches past e
+    if (e <= rg.x) return;
+
+    f32x2 npx[4], npy[2];                                          // minus the block's pixel centres
+#pragma unroll
+    for (int k = 0; k < 4; ++k) npx[k] = dup2(-fa((float)(bx0 + k), 0.5f));
+#pragma unroll
+    for (int k = 0; k < 2; ++k)
+        npy[k] = pack2(-fa((float)(by0 + 2 * k), 0.5f), -fa((float)(by0 + 2 * k + 1), 0.5f));
+
+    const uint32_t n_chunks = (e - rg.x + kC - 1u) / kC;
+    uint32_t m = 0u;
+    {
+        const uint32_t at = rg.x + (n_chunks - 1u) * kC + tid;
+        if (at < e) m = __ldg(vals + at);
+    }
+    for (uint32_t c = n_chunks; c-- > 0u;) {
+        const uint32_t s0 = rg.x + c * kC;
+        const uint32_t cnt = e - s0 < kC ? e - s0 : kC;
+        // ---- stage
+        if (tid < cnt) {
+            if (m >= M) m = 0;      // only after a failed sort (status already latched)
+            const float4* g = reinterpret_cast<const float4*>(splat + (size_t)m * kSplatStride);
+            const float4 g0 = __ldg(g), g1 = __ldg(g + 1), g2 = __ldg(g + 2);
+            S.r0[tid] = g0;
+            S.r1[tid] = g1;
+            S.r2[tid] = g2;
+            S.mask[tid] = (uint16_t)walk_mask(cam, tx0, ty0, g0.x, g0.y, g0.z, g0.w, g1.x, g1.y);
+        }
+        if (c > 0u) m = __ldg(vals + s0 - kC + tid);
+        __syncthreads();
+        // ---- list: the block's records before its last stop; how many before each pixel's own
+        uint32_t len[kBlocks] = {}, own[2] = {0u, 0u};
+        const uint32_t lt = (1u << lane) - 1u;
+        for (uint32_t j0 = 0; j0 < cnt; j0 += 32) {
+            const uint32_t j = j0 + lane;
+            const uint32_t bm = j < cnt ? (uint32_t)S.mask[j] >> fb : 0u;
+            uint32_t mine = 0u;
+#pragma unroll
+            for (uint32_t k = 0; k < kBlocks; ++k) {
+                const bool in = (bm & (1u << k)) && s0 + j < bl[k];
+                const uint32_t v = __ballot_sync(kFull, in);
+                if (in) W.list[k][len[k] + __popc(v & lt)] = (uint8_t)j;
+                len[k] += __popc(v);
+                mine = b == k ? v : mine;
+            }
+#pragma unroll
+            for (int k = 0; k < (kTwo ? 2 : 1); ++k) {
+                const uint32_t r = lim[k] > s0 + j0 ? lim[k] - s0 - j0 : 0u;   // the pixel's records of these 32
+                own[k] += __popc(mine & ~(r < 32u ? kFull << r : 0u));
+            }
+        }
+        __syncwarp();
+        uint32_t left = len[0];
+#pragma unroll
+        for (uint32_t k = 1; k < kBlocks; ++k) left = b == k ? len[k] : left;
+        const uint32_t en = (uint32_t)kLanes - 1u - i;             // (the transposition leaves entry 0 on top)
+        while (__any_sync(kFull, left != 0u)) {
+            // ---- test: one entry a lane at its block's 16 pixels; entry 0 is the list's last
+            const bool valid = en < left;
+            const uint32_t rs = valid ? W.list[b][left - 1u - en] : 0u;
+            const uint32_t sl = b * kLanes + en;
+            uint32_t hits = 0u;
+            {
+                const float4 a = S.r0[rs], cc = S.r1[rs], q = S.r2[rs];
+                W.col[sl] = make_float4(cc.z, q.x, q.y, q.z);
+                f32x2 dx[4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) dx[k] = add2(dup2(a.x), npx[k]);
+                const f32x2 hA = dup2(fm(0.5f, a.z)), B2 = dup2(a.w), hC = dup2(fm(0.5f, cc.x)), K = dup2(-cc.y);
+#pragma unroll
+                for (int rp = 1; rp >= 0; --rp) {
+                    const f32x2 dy = add2(dup2(a.y), npy[rp]);
+                    const f32x2 bdy = mul2(B2, dy), cdy = mul2(mul2(hC, dy), dy);
+                    f32x2 n[4];
+#pragma unroll
+                    for (int k = 3; k >= 0; --k) {
+                        n[k] = fma2(fma2(hA, dx[k], bdy), dx[k], cdy);
+                        const float2 p = unpack2(mul2(n[k], fma2(n[k], dup2(-1.0f), K)));
+                        hits = __funnelshift_l(__float_as_uint(p.x), hits, 1);
+                        hits = __funnelshift_l(__float_as_uint(p.y), hits, 1);
+                    }
+                    float* pn = &W.n[sl][8 * rp];
+                    *reinterpret_cast<ulonglong2*>(pn) = make_ulonglong2(n[0], n[1]);
+                    *reinterpret_cast<ulonglong2*>(pn + 4) = make_ulonglong2(n[2], n[3]);
+                }
+                hits = valid ? ~hits & 0xFFFFu : 0u;
+            }
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                *reinterpret_cast<float4*>(&W.w[sl][4 * k]) = make_float4(0.f, 0.f, 0.f, 0.f);
+                *reinterpret_cast<float4*>(&W.g[sl][4 * k]) = make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+            // the first left - own entries lie behind the pixel's stop
+            const uint32_t d0 = left > own[0] ? left - own[0] : 0u, d1 = left > own[1] ? left - own[1] : 0u;
+            uint32_t mask = transpose_bits<kLanes>(hits, i) &
+                            ((kPx0 & shr0(0xFFFFu, (kTwo ? 2u : 1u) * d0)) | (kPx1 & shr0(0xFFFFu, 2u * d1)));
+            mask <<= 16;
+            __syncwarp();
+            // ---- apply
+            while (__any_sync(kFull, mask != 0u)) {
+                uint32_t sh = clz_or_ones(mask);
+                if (kTwo) sh &= ~1u;
+                const uint32_t h = mask & shr0(kTwo ? 0xC0000000u : 0x80000000u, sh);
+                const bool h0 = (h & (kPx0 << 16)) != 0u, h1 = (h & (kPx1 << 16)) != 0u;
+                mask ^= h;
+                const uint32_t at = b * kLanes + ((kTwo ? sh >> 1 : sh) & (kLanes - 1u));
+                const float4 cv = W.col[at];
+                auto alpha1 = [&](float n) {                       // before the clamp
+                    uint32_t t;
+                    const float p = exp_poly_neg(n, t);
+                    return fm(cv.x, fm(p, __uint_as_float((t << 23) + (127u << 23))));
+                };
+                const f32x2 qd = fma2(dC2, dup2(cv.w), fma2(dC1, dup2(cv.z), mul2(dC0, dup2(cv.y))));
+                if constexpr (kTwo) {
+                    const float2 n = *reinterpret_cast<const float2*>(&W.n[at][park]);
+                    const float r0 = alpha1(n.x), r1 = alpha1(n.y);
+                    const f32x2 al = pack2(h0 ? fminf(r0, 0.99f) : 0.0f, h1 ? fminf(r1, 0.99f) : 0.0f);
+                    const float2 om = unpack2(fma2(al, dup2(-1.0f), dup2(1.0f)));
+                    const f32x2 iom = pack2(rcp1(om.x), rcp1(om.y));
+                    T = mul2(T, iom);                              // before the entry
+                    const f32x2 w = mul2(al, T);
+                    const float2 gp = unpack2(mul2(fma2(mul2(iom, D), dup2(-1.0f), mul2(T, qd)), al));
+                    D = fma2(w, qd, D);
+                    if (h) {
+                        *reinterpret_cast<f32x2*>(&W.w[at][park]) = w;
+                        // a clamped alpha does not move
+                        *reinterpret_cast<float2*>(&W.g[at][park]) =
+                            make_float2(r0 < 0.99f ? gp.x : 0.0f, r1 < 0.99f ? gp.y : 0.0f);
+                    }
+                } else {
+                    const float r0 = alpha1(W.n[at][park]);
+                    const float al = h0 ? fminf(r0, 0.99f) : 0.0f;
+                    const float iom = rcp1(1.0f - al), q0 = unpack2(qd).x, d = unpack2(D).x;
+                    const float t = unpack2(T).x * iom, w = al * t;
+                    if (h0) {
+                        W.w[at][park] = w;
+                        W.g[at][park] = r0 < 0.99f ? (t * q0 - iom * d) * al : 0.0f;
+                    }
+                    T = pack2(t, 0.0f);
+                    D = pack2(fmaf(w, q0, d), 0.0f);
+                }
+            }
+            __syncwarp();
+            // ---- gather: the entry's sums over the block's pixels
+            if (hits) {
+                f32x2 R = 0ull, G = 0ull, Bs = 0ull, S0 = 0ull, Sx = 0ull, Sy = 0ull, Sxx = 0ull, Sxy = 0ull, Syy = 0ull;
+                const uint32_t dc = 32u * kBlocks / 2u * warp + 16u * b;
+                const float4 a = S.r0[rs], cc = S.r1[rs];
+                f32x2 dx[4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) dx[k] = add2(dup2(a.x), npx[k]);
+#pragma unroll
+                for (int rp = 0; rp < 2; ++rp) {
+                    f32x2 sr = 0ull, rx = 0ull;
+#pragma unroll
+                    for (int k = 0; k < 4; k += 2) {
+                        const int o = 8 * rp + 2 * k;
+                        const ulonglong2 w = *reinterpret_cast<const ulonglong2*>(&W.w[sl][o]);
+                        const ulonglong2 g = *reinterpret_cast<const ulonglong2*>(&W.g[sl][o]);
+                        const ulonglong2 c0 = *reinterpret_cast<const ulonglong2*>(&S.dC[0][dc + o]);
+                        const ulonglong2 c1 = *reinterpret_cast<const ulonglong2*>(&S.dC[1][dc + o]);
+                        const ulonglong2 c2 = *reinterpret_cast<const ulonglong2*>(&S.dC[2][dc + o]);
+                        R = fma2(w.y, c0.y, fma2(w.x, c0.x, R));
+                        G = fma2(w.y, c1.y, fma2(w.x, c1.x, G));
+                        Bs = fma2(w.y, c2.y, fma2(w.x, c2.x, Bs));
+                        sr = add2(g.y, add2(g.x, sr));
+                        const f32x2 x0 = mul2(g.x, dx[k]), x1 = mul2(g.y, dx[k + 1]);
+                        rx = add2(x1, add2(x0, rx));
+                        Sxx = fma2(x1, dx[k + 1], fma2(x0, dx[k], Sxx));
+                    }
+                    S0 = add2(S0, sr);
+                    Sx = add2(Sx, rx);
+                    const f32x2 dy = add2(dup2(a.y), npy[rp]), ry = mul2(sr, dy);
+                    Sxy = fma2(rx, dy, Sxy);
+                    Sy = add2(Sy, ry);
+                    Syy = fma2(ry, dy, Syy);
+                }
+                auto total = [](f32x2 v) {
+                    const float2 f = unpack2(v);
+                    return f.x + f.y;
+                };
+                const float sx = total(Sx), sy = total(Sy);
+                float* out = gsplat + (size_t)min(__ldg(vals + s0 + rs), M - 1u) * kGS;
+                // d power / du = -(A dx + B dy), likewise for v; d alpha / d alpha0 = alpha / alpha0
+                atomicAdd(reinterpret_cast<float4*>(out),
+                          make_float4(-(a.z * sx + a.w * sy), -(cc.x * sy + a.w * sx), -0.5f * total(Sxx), -total(Sxy)));
+                atomicAdd(reinterpret_cast<float4*>(out) + 1,
+                          make_float4(-0.5f * total(Syy), total(S0) / cc.z, total(R), total(G)));
+                atomicAdd(out + 8, total(Bs));
+            }
+            __syncwarp();
+            left -= min(left, (uint32_t)kLanes);
+        }
+        __syncthreads();
+    }
 }
 
 // keep holds each pixel's {final T, stop} (kept by a FGS_RENDER_KEEP forward, or
-// recomputed by the forward's walk without an image just before).  The tile is
-// walked back to front over half-block lists (a 4x4 half-warp tests only the
-// Gaussians whose threshold box meets it), the two halves of a warp in lockstep,
-// each from its list's last entry before its last stop.
-__global__ void __launch_bounds__(256) blend_bwd_kernel(DevCamera cam, const uint2* __restrict__ ranges,
-                                                        const uint32_t* __restrict__ vals,
-                                                        const float* __restrict__ splat,
-                                                        const uint2* __restrict__ keep,
-                                                        const float* __restrict__ dL_drgb,
-                                                        float* __restrict__ gsplat, FrameState* st)
+// recomputed by the forward's walk without an image just before).
+__global__ void __launch_bounds__(blendk::kWalkChunk) blend_bwd_kernel(
+    DevCamera cam, const uint2* __restrict__ ranges, const uint32_t* __restrict__ heavy,
+    const uint32_t* __restrict__ vals, const float* __restrict__ splat, const uint2* __restrict__ keep,
+    const float* __restrict__ dL_drgb, float* __restrict__ gsplat, const FrameState* st)
 {
-    __shared__ __align__(128) BwdWalkSmem S;
-    const uint32_t tile = blockIdx.x;
-    const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int32_t tx0 = (int32_t)(tile % (uint32_t)cam.tiles_x) * cam.tile_w;
-    const int32_t ty0 = (int32_t)(tile / (uint32_t)cam.tiles_x) * cam.tile_h;
-    int32_t wx0, wy0;
-    blendk::warp_origin(cam, tx0, ty0, warp, wx0, wy0);
-    const uint32_t half = lane >> 4, q = lane & 15u;
-    const bool wide = cam.warp_shift == 3;
-    const int32_t x = wx0 + (int32_t)(q & 3u) + (wide ? 4 * (int32_t)half : 0);
-    const int32_t y = wy0 + (int32_t)(q >> 2) + (wide ? 0 : 4 * (int32_t)half);
-    const uint32_t hb = ((uint32_t)(y - ty0) >> 2 << (cam.tile_shift_x - 2)) | ((uint32_t)(x - tx0) >> 2);
-    const uint32_t hb0 = __shfl_sync(0xffffffffu, hb, 0), hb1 = __shfl_sync(0xffffffffu, hb, 16);
-    const bool inside = x < cam.width && y < cam.height;
-    const float px = fa((float)x, 0.5f), py = fa((float)y, 0.5f);
-    const uint2 rg = ranges[tile];
-    const uint32_t M = st->M;
-    const uint32_t s = rg.x;
-    const int comp = half_component(lane);
-    const uint32_t lt = (1u << lane) - 1u;
-
-    // this pixel's forward outcome: final T, stop position, and dL/dC
-    float T = 1.0f;
-    uint32_t lim = s;
-    float dC[3] = {0.0f, 0.0f, 0.0f};
-    if (inside) {
-        const size_t hw = (size_t)cam.width * cam.height, pix = (size_t)y * cam.width + x;
-        const uint2 kp = keep[pix];
-        T = __uint_as_float(kp.x);
-        lim = kp.y;
-        dC[0] = __ldg(dL_drgb + pix);
-        dC[1] = __ldg(dL_drgb + hw + pix);
-        dC[2] = __ldg(dL_drgb + 2 * hw + pix);
-    }
-    // each half-block's last stop position; the tile's bounds the chunks
-    const uint32_t hmax = max(lim, __shfl_xor_sync(0xffffffffu, lim, 8));
-    const uint32_t hmax2 = max(hmax, __shfl_xor_sync(0xffffffffu, hmax, 4));
-    const uint32_t hmax3 = max(hmax2, __shfl_xor_sync(0xffffffffu, hmax2, 2));
-    const uint32_t hlim = max(hmax3, __shfl_xor_sync(0xffffffffu, hmax3, 1));
-    if (q == 0) S.hlim[hb] = hlim;
-    if (tid == 0) {
-        blendk::mbar_init(&S.bar, 1);
-        S.timed_out = 0;
-    }
-    __syncthreads();
-    uint32_t e = S.hlim[0];
-#pragma unroll
-    for (int h = 1; h < blendk::kHalfBlocks; ++h) e = max(e, S.hlim[h]);
-    e = min(e, rg.y);                    // no pixel of the tile reaches past e
-    const uint32_t hlim0 = S.hlim[hb0], hlim1 = S.hlim[hb1];
-
-    float Bk[3] = {cam.bg[0] * T, cam.bg[1] * T, cam.bg[2] * T};   // colour behind, absolute
-    float Tc = T;                                                    // transmittance after
-    if (e <= s) return;
-    uint32_t phase = 0;
-    const uint32_t n_chunks = (e - s + blendk::kChunk - 1) / blendk::kChunk;
-    for (int c = (int)n_chunks - 1; c >= 0; --c) {
-        const uint32_t s0 = s + (uint32_t)c * blendk::kChunk, e0 = min(e, s0 + blendk::kChunk);
-        const uint32_t cnt = e0 - s0;
-        const uint32_t off = blendk::stage_vals(S.vals, &S.bar, &S.timed_out, vals, s0, e0, phase, st);
-        if (S.timed_out) return;
-        if (tid < cnt) {
-            uint32_t m = S.vals[off + tid];
-            if (m >= M) m = 0;
-            const float4* g = reinterpret_cast<const float4*>(splat + (size_t)m * kSplatStride);
-            const float4 a = __ldg(g), b = __ldg(g + 1);
-            blendk::put_coeffs(S.g0[tid], S.g1[tid], a, b);
-            S.g2[tid] = __ldg(g + 2);
-            S.hmask[tid] = (uint16_t)blendk::half_mask(cam, tx0, ty0, a.x, a.y, a.z, a.w, b.x, b.y);
-            S.m[tid] = m;
-        }
-        __syncthreads();
-        // this warp's two half-block lists of the chunk entries before their last stops
-        uint32_t n0 = 0, n1 = 0;
-        for (uint32_t j0 = 0; j0 < cnt; j0 += 32) {
-            const uint32_t j = j0 + lane;
-            const uint32_t hm = j < cnt ? (uint32_t)S.hmask[j] : 0u;
-            const bool in0 = ((hm >> hb0) & 1u) && s0 + j < hlim0;
-            const bool in1 = ((hm >> hb1) & 1u) && s0 + j < hlim1;
-            const uint32_t b0 = __ballot_sync(0xffffffffu, in0);
-            const uint32_t b1 = __ballot_sync(0xffffffffu, in1);
-            if (in0) S.hl[hb0][n0 + __popc(b0 & lt)] = (uint8_t)j;
-            if (in1) S.hl[hb1][n1 + __popc(b1 & lt)] = (uint8_t)j;
-            n0 += __popc(b0);
-            n1 += __popc(b1);
-        }
-        __syncwarp();
-        const uint32_t nmax = max(n0, n1);
-        const uint32_t nh = half ? n1 : n0;
-        const uint8_t* myl = S.hl[hb];
-        // step k: each half takes its entry k - (nmax - nh), the lists' ends aligned
-        for (int k = (int)nmax - 1; k >= 0; --k) {
-            const int i = k - (int)(nmax - nh);
-            const bool valid = i >= 0;
-            const uint32_t j = valid ? myl[i] : 0u;
-            // branch-free: every lane evaluates; the lanes whose pixel applied the
-            // Gaussian in the forward (same decisions) contribute, the others add 0
-            const float4 g0 = S.g0[j];
-            const float4 g1 = S.g1[j];
-            const float dx = fs(g0.x, px), dy = fs(g0.y, py);
-            const float power = blendk::power_of(g0.z, g0.w, g1.x, dx, dy);
-            const bool hit = valid && s0 + j < lim && !(power > 0.0f || power < g1.y);
-            const uint32_t hb_any = __ballot_sync(0xffffffffu, hit);
-            if (!hb_any) continue;
-            const float ex = exp_nonpos(fminf(power, 0.0f));
-            const float raw = fm(g1.z, ex);
-            const bool clamped = !(raw < 0.99f);
-            const float alpha = hit ? (clamped ? 0.99f : raw) : 0.0f;
-            const float4 g2 = S.g2[j];
-            const float iom = __frcp_rn(1.0f - alpha);              // decides nothing
-            const float Tb = Tc * iom;                               // transmittance before
-            const float w = alpha * Tb;
-            const float galpha = hit ? dC[0] * (g2.x * Tb - Bk[0] * iom) + dC[1] * (g2.y * Tb - Bk[1] * iom) +
-                                       dC[2] * (g2.z * Tb - Bk[2] * iom)
-                                     : 0.0f;
-            Bk[0] += g2.x * w;
-            Bk[1] += g2.y * w;
-            Bk[2] += g2.z * w;
-            Tc = Tb;
-            float g[9];
-            g[6] = w * dC[0];
-            g[7] = w * dC[1];
-            g[8] = w * dC[2];
-            const float gpow = clamped ? 0.0f : galpha * alpha;     // d alpha / d power = alpha
-            g[5] = clamped ? 0.0f : galpha * ex;                   // d alpha / d alpha0 = e^power
-            g[2] = -0.5f * dx * dx * gpow;                         // A
-            g[3] = -dx * dy * gpow;                                // B
-            g[4] = -0.5f * dy * dy * gpow;                         // C
-            // d power / du = -(A dx + B dy) = 2 A' dx + B' dy, likewise for v
-            g[0] = gpow * (2.0f * g0.z * dx + g0.w * dy);          // u
-            g[1] = gpow * (2.0f * g1.x * dy + g0.w * dx);          // v
-            const float v = half_reduce9(g, lane);
-            const bool my_half_hit = ((hb_any >> (half << 4)) & 0xFFFFu) != 0u;
-            if (comp >= 0 && my_half_hit) atomicAdd(gsplat + (size_t)S.m[j] * kGS + comp, v);
-        }
-        __syncthreads();
-    }
+    __shared__ __align__(128) BwdSmem S;
+    blendk::walk_grid(
+        (uint32_t)(cam.tiles_x * cam.tiles_y), ranges, heavy, st,
+        [&](uint32_t tile, uint2 rg) {
+            blend_bwd_walk<8>(cam, tile, 0u, rg, S, vals, splat, keep, dL_drgb, gsplat, st);
+        },
+        [&](uint32_t tile, uint32_t part, uint2 rg) {
+            blend_bwd_walk<16>(cam, tile, part, rg, S, vals, splat, keep, dL_drgb, gsplat, st);
+        });
 }
 
 // ---------------------------------------------------------------------------
@@ -674,7 +802,9 @@ void launch_backward(const DevTree& t, const DevCamera& cam, const uint2* ranges
     // gsplat rows of the selected Gaussians start at zero: the blend backward adds into them
     zero_rows_kernel<<<sms * 8, 128, 0, s>>>(reinterpret_cast<float4*>(gsplat), st);
     if (!kept) launch_blend(cam, ranges, heavy, vals, splat, nullptr, nullptr, keep, st, false, s);
-    blend_bwd_kernel<<<cam.tiles_x * cam.tiles_y, 256, 0, s>>>(cam, ranges, vals, splat, keep, dL_drgb, gsplat, st);
+    const int n_tiles = cam.tiles_x * cam.tiles_y;
+    blend_bwd_kernel<<<n_tiles + 2 * split_slots(n_tiles), blendk::kWalkChunk, 0, s>>>(cam, ranges, heavy, vals, splat,
+                                                                                     keep, dL_drgb, gsplat, st);
     const ParamPtrs p{params[0], params[1], params[2], params[3], params[4], t.n};
     const GradPtrs gr{grads[0], grads[1], grads[2], grads[3], grads[4]};
     if (!accumulate) {

@@ -291,35 +291,6 @@ __device__ __forceinline__ void blend_tile_kpc(const DevCamera& cam, uint32_t ti
     }
 }
 
-constexpr int kHalfBlocks = 16;
-
-// Half-blocks of the tile (grid of tile_w / 4 x tile_h / 4, row-major bits) that
-// the Gaussian's threshold box meets; the box and its margins are warp_mask's.
-__device__ __forceinline__ uint32_t half_mask(const DevCamera& cam, int32_t tx0, int32_t ty0, float u,
-                                              float v, float A, float B, float C, float lthr)
-{
-    if (!(lthr <= 0.0f)) return 0u;
-    const float det = A * C - B * B;
-    const float tr = A + C;
-    if (!(det > 0.0f) || tr * tr > 1e4f * det) return 0xFFFFu;
-    const float sq = fmaf(-2.1f, lthr, 1e-4f);
-    const float ex = fmaf(sqrtf(sq * C / det), 1.001f, 0.01f);
-    const float ey = fmaf(sqrtf(sq * A / det), 1.001f, 0.01f);
-    const int32_t sh = cam.tile_shift_x - 2;                 // log2(half-block columns)
-    const int32_t ncol = 1 << sh, nrow = kHalfBlocks >> sh;
-    const float ux = u - (float)tx0, vy = v - (float)ty0;
-    const int32_t c_lo = max(0, (int32_t)ceilf((ux - ex - 3.5f) * 0.25f));
-    const int32_t c_hi = min(ncol - 1, (int32_t)floorf((ux + ex - 0.5f) * 0.25f));
-    const int32_t r_lo = max(0, (int32_t)ceilf((vy - ey - 3.5f) * 0.25f));
-    const int32_t r_hi = min(nrow - 1, (int32_t)floorf((vy + ey - 0.5f) * 0.25f));
-    if (c_lo > c_hi || r_lo > r_hi) return 0u;
-    const uint32_t cols = ((2u << c_hi) - 1u) & ~((1u << c_lo) - 1u);
-    uint32_t mask = 0;
-    for (int32_t r = r_lo; r <= r_hi; ++r) mask |= cols << (r << sh);
-    return mask;
-}
-
-
 // ---------------------------------------------------------------------------
 // The forward's walk
 // ---------------------------------------------------------------------------

@@ -6,7 +6,7 @@ import pytest
 
 from paper_2603_23891_gb300 import synth
 
-from gpu_util import assert_frame_parity, gpu_frame, oracle_frame
+from gpu_util import assert_frame_parity, gpu_frame, grad_parity_case, oracle_frame
 
 pytestmark = pytest.mark.gpu
 
@@ -94,3 +94,25 @@ def test_infinite_colour_stays_where_it_is_applied(renderer, size):
     big = np.abs(c).max(axis=0) > 1e30
     assert np.array_equal(big | ~np.isfinite(c).all(axis=0), touched)
     assert np.array_equal(a[:, ~touched].view(np.uint32), c[:, ~touched].view(np.uint32))
+
+
+@pytest.mark.parametrize("size", [(90, 70), (1920, 1080)])
+@pytest.mark.parametrize("tile", [(16, 16), (32, 8), (8, 32), (64, 4)])
+def test_gradients_on_every_tile_shape(renderer, tile, size):
+    """The gradient walk on a scene with tiles of up to hundreds of pairs, opaque enough
+    that pixels stop inside the lists, against the oracle: split tiles (small image, every
+    pixel), whole ones (1080p, a thousand pixels)."""
+    rng = np.random.default_rng(12)
+    n = 400
+    mu = np.stack([rng.uniform(-7, 7, n), rng.uniform(8, 14, n), rng.uniform(-5, 5, n)], 1)
+    logs = rng.uniform(-1.5, 0.8, (n, 3))
+    quat = rng.normal(size=(n, 4))
+    sh = rng.normal(0, 0.1, (n, 4, 3))
+    tree = synth.tree_from_gaussians(mu, logs, quat / np.linalg.norm(quat, axis=1, keepdims=True),
+                                     rng.normal(0.0, 1.5, n), sh, 1)
+    cam = synth.look_at_camera([0, 0, 0], [0, 1, 0], *size, 70.0)
+    small = size[0] < 1000
+    pix = None if small else np.sort(rng.choice(size[0] * size[1], 1000, replace=False))
+    g, _, _ = grad_parity_case(renderer, tree, cam, -1.0, 3, tile=tile, pix=pix)
+    split = np.bincount((g["keys"] >> np.uint64(32)).astype(np.int64)) > g["NP"] // SPLIT
+    assert split.all() if small else np.count_nonzero(~split) > 5000
