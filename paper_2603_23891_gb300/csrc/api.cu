@@ -997,7 +997,6 @@ int kpc_view(fgs_ctx* c, void* stream, bool force_3sigma, double* gbar_out, floa
     cudaStream_t s = (cudaStream_t)stream;
     const DevCamera dc = make_devcam(c, force_3sigma);
     enqueue_front(c, dc, s, nullptr);
-    FGS_CUDA(c, cudaMemsetAsync(c->kpc, 0, c->pair_cap * 4, s));
     launch_blend_kpc(dc, c->ranges, c->vals1, c->splat, c->kpc, c->G, c->st, s);
     FGS_CUDA(c, cudaGetLastError());
     c->have_frame = true;

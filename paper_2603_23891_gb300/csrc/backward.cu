@@ -551,7 +551,7 @@ struct GradPtrs {
 // bank (l (3 K + 1) + k) mod 32, a different bank for every lane.
 __device__ __forceinline__ void cp_async4(float* smem, const float* gmem)
 {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(blendk::smem_addr(smem)), "l"(gmem)
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(smem)), "l"(gmem)
                  : "memory");
 }
 

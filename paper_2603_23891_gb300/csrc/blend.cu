@@ -6,13 +6,8 @@
 // at a time and each warp walks it for its own blocks of pixels (blend_walk in
 // blend_impl.cuh).
 //
-// The KPC pass: one thread per pixel (tile_w * tile_h = 256); each warp covers an
-// 8 x 4 (or 4 x 8) pixel block.  The slice is brought into shared memory in chunks
-// of 256 by a TMA bulk copy (cp.async.bulk, completion on an mbarrier; the copy
-// starts at the 16-byte boundary at or below the slice and the index is offset
-// accordingly); each thread then gathers one splat record and computes which warps
-// it can reach, and each warp walks its own ordered list one entry at a time,
-// reducing alpha * T across the warp.
+// The KPC pass: the same walk of whole tiles without an image, with the applied
+// alpha * T summed for every pair (blend_walk_kpc).
 //
 // Blend decisions are exact: power, the log-domain skip test, alpha, the
 // opacity clamp and the transmittance update use explicitly rounded binary32
@@ -23,8 +18,6 @@
 #include "blend_impl.cuh"
 
 namespace fgs {
-
-using blendk::BlendSmem;
 
 template <bool kCount, bool kKeep>
 __global__ void __launch_bounds__(blendk::kWalkChunk) blend_kernel(
@@ -45,16 +38,14 @@ __global__ void __launch_bounds__(blendk::kWalkChunk) blend_kernel(
         });
 }
 
-__global__ void __launch_bounds__(256) blend_kpc_kernel(DevCamera cam, const uint2* __restrict__ ranges,
-                                                        const uint32_t* __restrict__ vals,
-                                                        const float* __restrict__ splat, float* __restrict__ kpc_out,
-                                                        float* __restrict__ G_out, FrameState* st)
+__global__ void __launch_bounds__(blendk::kWalkChunk) blend_kpc_kernel(
+    DevCamera cam, const uint2* __restrict__ ranges, const uint32_t* __restrict__ vals,
+    const float* __restrict__ splat, float* __restrict__ kpc_out, float* __restrict__ G_out, FrameState* st)
 {
-    __shared__ __align__(128) BlendSmem<true> S;
-    __shared__ double s_red[8];
+    __shared__ __align__(128) blendk::KpcSmem S;
     grid_dep_wait();
     grid_dep_trigger();
-    blendk::blend_tile_kpc(cam, blockIdx.x, S, s_red, ranges, vals, splat, kpc_out, G_out, st);
+    blendk::blend_walk_kpc(cam, blockIdx.x, ranges[blockIdx.x], S, vals, splat, kpc_out, G_out, st);
 }
 
 void launch_blend(const DevCamera& cam, const uint2* ranges, const uint32_t* heavy, const uint32_t* vals,
@@ -76,7 +67,7 @@ void launch_blend_kpc(const DevCamera& cam, const uint2* ranges, const uint32_t*
                       const float* splat, float* kpc, float* G, FrameState* st, cudaStream_t s)
 {
     const int n_tiles = cam.tiles_x * cam.tiles_y;
-    launch_pdl(blend_kpc_kernel, n_tiles, 256, 0, s, cam, ranges, vals, splat, kpc, G, st);
+    launch_pdl(blend_kpc_kernel, n_tiles, blendk::kWalkChunk, 0, s, cam, ranges, vals, splat, kpc, G, st);
 }
 
 __global__ void eval_exp_kernel(const float* __restrict__ x, float* __restrict__ y, uint64_t n)

@@ -9,288 +9,6 @@
 namespace fgs {
 namespace blendk {
 
-
-
-
-constexpr int kChunk = 256;
-constexpr int kValsSlots = kChunk + 8;     // aligned superset of one chunk
-
-__device__ __forceinline__ uint32_t smem_addr(const void* p)
-{
-    return (uint32_t)__cvta_generic_to_shared(p);
-}
-
-__device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count)
-{
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(bar)), "r"(count) : "memory");
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-}
-
-__device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t* bar, uint32_t bytes)
-{
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(bar)),
-                 "r"(bytes)
-                 : "memory");
-}
-
-__device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t phase)
-{
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(smem_addr(bar)), "r"(phase)
-        : "memory");
-    return ok != 0;
-}
-
-// 1D bulk copy global -> shared; src, dst 16-byte aligned, bytes a multiple of 16.
-__device__ __forceinline__ void tma_bulk_g2s(void* dst, const void* src, uint32_t bytes, uint64_t* bar)
-{
-    asm volatile(
-        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-            smem_addr(dst)),
-        "l"(src), "r"(bytes), "r"(smem_addr(bar))
-        : "memory");
-}
-
-__device__ __forceinline__ void fence_proxy_async_smem()
-{
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-}
-
-template <bool kKpc>
-struct BlendSmem {
-    uint32_t vals[kValsSlots];
-    float4 g0[kChunk];          // u, v, A', B'  (power coefficients, see power_of)
-    float4 g1[kChunk];          // C', lthr, alpha0, depth
-    float4 g2[kChunk];          // r, g, b, radius
-    uint32_t wmask[kChunk];     // bit w: warp w's pixels can reach the skip threshold
-    alignas(16) uint16_t wlist[8][kChunk];  // per-warp list of chunk entries, in order
-    float kpc_w[kKpc ? 8 : 1][kKpc ? kChunk : 1];   // per-warp partial KPC (Eq. 5)
-    uint64_t bar;
-    int timed_out;
-};
-
-// The Gaussian's exponent at offset (dx, dy) = (u - px, v - py):
-// -1/2 (A dx^2 + 2 B dx dy + C dy^2) = (A' dx + B' dy) dx + (C' dy) dy with the
-// per-Gaussian coefficients A' = -A/2, B' = -B, C' = -C/2, evaluated with two
-// fused multiply-adds in this order (the reading both sides share).
-__device__ __forceinline__ float power_of(float Ah, float Bn, float Ch, float dx, float dy)
-{
-    return ff(ff(Ah, dx, fm(Bn, dy)), dx, fm(fm(Ch, dy), dy));
-}
-
-// Shared-memory copy of a splat record's first two float4 (u, v, A, B),
-// (C, lthr, alpha0, depth) with the conic replaced by the power coefficients.
-__device__ __forceinline__ void put_coeffs(float4& d0, float4& d1, float4 a, float4 b)
-{
-    d0 = make_float4(a.x, a.y, fm(-0.5f, a.z), -a.w);
-    d1 = make_float4(fm(-0.5f, b.x), b.y, b.z, b.w);
-}
-
-// Bring chunk [s0, e0) of the sorted values into shared memory with one TMA bulk
-// copy of the 16-byte aligned superset [s0 & ~3, (e0 + 3) & ~3).  Returns the
-// offset of s0 inside the staged copy.  Called by all threads; thread 0 issues
-// the copy and waits on the mbarrier (bounded).  If the wait gives up, the
-// status FGS_ERR_TIMEOUT is latched and the callers leave the tile; the copy may
-// still be in flight into the block's shared memory as the block exits, so
-// after such a timeout neither the frame's output nor the context can be
-// trusted (the caller must destroy the context).
-__device__ __forceinline__ uint32_t stage_vals(uint32_t* dst, uint64_t* bar, int* timed_out,
-                                               const uint32_t* vals, uint32_t s0, uint32_t e0,
-                                               uint32_t& phase, FrameState* st)
-{
-    const uint32_t a0 = s0 & ~3u;
-    const uint32_t a1 = (e0 + 3u) & ~3u;
-    const uint32_t bytes = (a1 - a0) * 4u;
-    if (threadIdx.x == 0) {
-        fence_proxy_async_smem();
-        mbar_arrive_expect_tx(bar, bytes);
-        tma_bulk_g2s(dst, vals + a0, bytes, bar);
-        uint64_t spins = 0;
-        while (!mbar_try_wait(bar, phase)) {
-            if (++spins > kSpinLimit) {
-                *timed_out = 1;
-                set_status(st, kErrTimeout, 0x500u);
-                break;
-            }
-        }
-    }
-    phase ^= 1u;
-    __syncthreads();
-    return s0 - a0;
-}
-
-// Warps of a CTA cover ww x wh pixel blocks of the tile, ww = 1 << warp_shift
-// (8 or 4), wh = 32 / ww, tile_w / ww of them across; (tx0, ty0) is the tile's
-// first pixel.
-__device__ __forceinline__ void warp_origin(const DevCamera& cam, int32_t tx0, int32_t ty0, uint32_t w,
-                                            int32_t& x0, int32_t& y0)
-{
-    const uint32_t sh = (uint32_t)(cam.tile_shift_x - cam.warp_shift);   // log2(warps per row)
-    x0 = tx0 + (int32_t)((w & ((1u << sh) - 1u)) << cam.warp_shift);
-    y0 = ty0 + (int32_t)((w >> sh) << (5 - cam.warp_shift));
-}
-
-// Which warps of the tile may hold a pixel whose binary32 power reaches the
-// Gaussian's skip threshold lthr.  Exactly, power >= lthr is the ellipse
-// d^T Q d <= s with Q = [[A, B], [B, C]] and s = -2 lthr, whose bounding box has
-// half-widths sqrt(s C / det Q) and sqrt(s A / det Q).  Margins, for
-// cond(Q) < 1e4 (cond(Q) <= tr^2 / det; beyond that, or for a singular Q, every
-// warp keeps the Gaussian):
-//  * the binary32 power (offsets rounded, three products, two fused
-//    multiply-adds) is within 11 * 2^-24 * cond(Q) < 0.7% of the exact form at
-//    the exact offsets, so a pixel passing the test lies in the ellipse of
-//    s' = 1.05 s + 1e-4;
-//  * det Q computed in binary32 loses at most 2^-24 cond(Q) / 2 < 3e-4
-//    relative, so the computed half-widths are within 2e-4 relative of the
-//    exact ones for s' (the 5% in s leaves 2% of the half-width spare);
-//  * the box is further widened by 0.1% and 0.01 px for the roundings of
-//    u - tx0, v - ty0 and of the bounds below.
-// A warp left out of the mask would have skipped the Gaussian at every one of
-// its pixels.  Warp column c spans pixel centres tx0 + ww c + [0.5, ww - 0.5],
-// row r spans ty0 + wh r + [0.5, wh - 0.5]; the mask is the block of columns x
-// rows the box meets.  (A one-pixel margin here listed 28% more entries for the
-// few-pixel Gaussians of far LoD levels; an exact ellipse-rectangle test per
-// warp removed only 4% more and cost more than it saved.)
-__device__ __forceinline__ uint32_t warp_mask(const DevCamera& cam, int32_t tx0, int32_t ty0, float u,
-                                              float v, float A, float B, float C, float lthr)
-{
-    if (!(lthr <= 0.0f)) return 0u;             // alpha0 < 1/255: no pixel can pass
-    const float det = A * C - B * B;
-    const float tr = A + C;
-    if (!(det > 0.0f) || tr * tr > 1e4f * det) return 0xFFu;
-    const float sq = fmaf(-2.1f, lthr, 1e-4f);  // 1.05 * (-2 lthr) + 1e-4
-    const float ex = fmaf(sqrtf(sq * C / det), 1.001f, 0.01f);
-    const float ey = fmaf(sqrtf(sq * A / det), 1.001f, 0.01f);
-    const int32_t sh = cam.tile_shift_x - cam.warp_shift;   // log2(warps per tile row)
-    const int32_t ncol = 1 << sh, nrow = 8 >> sh;
-    const float ww = (float)(1 << cam.warp_shift), wh = (float)(32 >> cam.warp_shift);
-    const float iww = 1.0f / ww, iwh = 1.0f / wh;            // exact: powers of two
-    const float ux = u - (float)tx0, vy = v - (float)ty0;
-    const int32_t c_lo = max(0, (int32_t)ceilf((ux - ex - (ww - 0.5f)) * iww));
-    const int32_t c_hi = min(ncol - 1, (int32_t)floorf((ux + ex - 0.5f) * iww));
-    const int32_t r_lo = max(0, (int32_t)ceilf((vy - ey - (wh - 0.5f)) * iwh));
-    const int32_t r_hi = min(nrow - 1, (int32_t)floorf((vy + ey - 0.5f) * iwh));
-    if (c_lo > c_hi || r_lo > r_hi) return 0u;
-    const uint32_t cols = ((2u << c_hi) - 1u) & ~((1u << c_lo) - 1u);
-    uint32_t mask = 0;
-    for (int32_t r = r_lo; r <= r_hi; ++r) mask |= cols << (r << sh);
-    return mask;
-}
-
-
-// The KPC pre-render of one tile (the CTA's; Eq. 5-6): the forward walk with
-// per-warp lists, one entry at a time, every lane computing power and (when any
-// lane of the warp can apply the Gaussian) alpha and T', selected per lane; the
-// applied alpha * T is reduced across the warp per entry and over the warps per
-// pair.  Writes kpc_out[pair] and the tile's mean KPC G_out[tile] (NaN for a
-// tile without pairs).  No image is written.
-__device__ __forceinline__ void blend_tile_kpc(const DevCamera& cam, uint32_t tile, BlendSmem<true>& S,
-                                               double* s_red, const uint2* __restrict__ ranges,
-                                               const uint32_t* __restrict__ vals,
-                                               const float* __restrict__ splat,
-                                               float* __restrict__ kpc_out, float* __restrict__ G_out,
-                                               FrameState* st)
-{
-    const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int32_t tx0 = (int32_t)(tile % (uint32_t)cam.tiles_x) * cam.tile_w;
-    const int32_t ty0 = (int32_t)(tile / (uint32_t)cam.tiles_x) * cam.tile_h;
-    int32_t wx0, wy0;
-    warp_origin(cam, tx0, ty0, warp, wx0, wy0);
-    const int32_t x = wx0 + (int32_t)(lane & ((1u << cam.warp_shift) - 1u));
-    const int32_t y = wy0 + (int32_t)(lane >> cam.warp_shift);
-    const bool inside = x < cam.width && y < cam.height;
-    const float px = fa((float)x, 0.5f), py = fa((float)y, 0.5f);
-    const uint2 rg = ranges[tile];
-    const uint32_t M = st->M;
-    const uint32_t s = rg.x, e = rg.y;
-
-    if (tid == 0) {
-        mbar_init(&S.bar, 1);
-        S.timed_out = 0;
-    }
-    __syncthreads();
-
-    float T = 1.0f;
-    bool done = !inside;
-    uint32_t phase = 0;
-    double kpc_acc = 0.0;      // this thread's share of the tile's KPC sum (fixed order)
-
-    for (uint32_t s0 = s; s0 < e; s0 += kChunk) {
-        const uint32_t e0 = min(e, s0 + kChunk);
-        const uint32_t cnt = e0 - s0;
-        const uint32_t off = stage_vals(S.vals, &S.bar, &S.timed_out, vals, s0, e0, phase, st);
-        if (S.timed_out) break;
-        if (tid < cnt) {
-            uint32_t m = S.vals[off + tid];
-            if (m >= M) m = 0;      // only after a failed sort (status already latched)
-            const float4* g = reinterpret_cast<const float4*>(splat + (size_t)m * kSplatStride);
-            const float4 a = __ldg(g), b = __ldg(g + 1);
-            put_coeffs(S.g0[tid], S.g1[tid], a, b);
-            S.wmask[tid] = warp_mask(cam, tx0, ty0, a.x, a.y, a.z, a.w, b.x, b.y);
-        }
-        __syncthreads();
-        // this warp's ordered list of the chunk entries that can reach its pixels
-        uint32_t wcnt = 0;
-        for (uint32_t j0 = 0; j0 < cnt; j0 += 32) {
-            const uint32_t j = j0 + lane;
-            const bool mine = j < cnt && ((S.wmask[j] >> warp) & 1u);
-            const uint32_t b = __ballot_sync(0xffffffffu, mine);
-            if (mine) S.wlist[warp][wcnt + __popc(b & ((1u << lane) - 1u))] = (uint16_t)j;
-            wcnt += __popc(b);
-        }
-        __syncwarp();
-        for (uint32_t i = 0; i < wcnt; ++i) {
-            const uint32_t j = S.wlist[warp][i];
-            float w = 0.0f;
-            const float4 g0 = S.g0[j];
-            const float4 g1 = S.g1[j];
-            const float power = power_of(g0.z, g0.w, g1.x, fs(g0.x, px), fs(g0.y, py));
-            const bool hit = !done && !(power > 0.0f || power < g1.y);
-            if (__any_sync(0xffffffffu, hit)) {
-                float alpha = fm(g1.z, exp_nonpos(fminf(power, 0.0f)));
-                alpha = alpha < 0.99f ? alpha : 0.99f;
-                const float Tn = fm(T, fs(1.0f, alpha));
-                const bool stop = hit && Tn < 0.0001f;     // stop before adding this Gaussian
-                const bool apply = hit && !stop;
-                w = apply ? alpha * T : 0.0f;
-                T = apply ? Tn : T;
-                done = done || stop;
-            }
-            // Eq. 5: sum of alpha * T over the warp's pixels for this pair
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
-            if (lane == 0) S.kpc_w[warp][j] = w;
-        }
-        __syncthreads();
-        if (tid < cnt) {
-            const uint32_t msk = S.wmask[tid];
-            float k = 0.0f;
-#pragma unroll
-            for (int w8 = 0; w8 < 8; ++w8)
-                if ((msk >> w8) & 1u) k += S.kpc_w[w8][tid];
-            kpc_out[s0 + tid] = k;
-            kpc_acc += (double)k;
-        }
-        __syncthreads();
-    }
-    // Eq. 6: G = mean KPC over the tile's pairs; fixed-order block reduction
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) kpc_acc += __shfl_xor_sync(0xffffffffu, kpc_acc, o);
-    if (lane == 0) s_red[warp] = kpc_acc;
-    __syncthreads();
-    if (tid == 0) {
-        const uint32_t n = e - s;
-        double sum = 0.0;
-        for (int w8 = 0; w8 < 8; ++w8) sum += s_red[w8];
-        G_out[tile] = n > 0 ? (float)(sum / (double)n) : __int_as_float(0x7fc00000);
-    }
-}
-
 // ---------------------------------------------------------------------------
 // The forward's walk
 // ---------------------------------------------------------------------------
@@ -298,7 +16,7 @@ __device__ __forceinline__ void blend_tile_kpc(const DevCamera& cam, uint32_t ti
 // tile is 16 blocks of 4x4 pixels; a warp has 32 / kLanes blocks, kLanes lanes each:
 // four blocks with two pixels a lane, or two blocks with one.
 //  * Stage: 128 records at a time, one a thread, into shared memory; the thread boxes
-//    its record against the tile's blocks (margins as warp_mask's).
+//    its record against the tile's blocks (walk_mask).
 //  * List: each warp gives every block of its own an ordered list of the records it
 //    may meet.
 //  * Test, kLanes entries of each block at a time: a lane takes ONE ENTRY and computes
@@ -423,10 +141,25 @@ __device__ __forceinline__ void walk_origin(const DevCamera& cam, uint32_t w, in
     oy = (int32_t)((w >> wsh) << (4u - bsh));
 }
 
-// Bit 4 w + b: block b of the w-th four (walk_origin's layout) may hold a pixel that
-// reaches the threshold: the box and the margins of warp_mask (the approximate
-// quotient and roots are within 1e-6, a thousandth of the 0.1% by which the box is
-// widened).
+// Which blocks of the tile may hold a pixel whose binary32 power reaches the
+// Gaussian's skip threshold lthr; bit 4 w + b: block b of the w-th four (walk_origin's
+// layout).  Exactly, power >= lthr is the ellipse d^T Q d <= s with Q = [[A, B], [B, C]]
+// and s = -2 lthr, whose bounding box has half-widths sqrt(s C / det Q) and
+// sqrt(s A / det Q).  Margins, for cond(Q) < 1e4 (cond(Q) <= tr^2 / det; beyond that, or
+// for a singular Q, every block keeps the Gaussian):
+//  * the binary32 power (offsets rounded, three products, two fused
+//    multiply-adds) is within 11 * 2^-24 * cond(Q) < 0.7% of the exact form at
+//    the exact offsets, so a pixel passing the test lies in the ellipse of
+//    s' = 1.05 s + 1e-4;
+//  * det Q computed in binary32 loses at most 2^-24 cond(Q) / 2 < 3e-4
+//    relative, and the approximate quotient and roots 1e-6, so the computed
+//    half-widths are within 2e-4 relative of the exact ones for s' (the 5% in s leaves
+//    2% of the half-width spare);
+//  * the box is further widened by 0.1% and 0.01 px for the roundings of
+//    u - tx0, v - ty0 and of the bounds below.
+// A block left out of the mask would have skipped the Gaussian at every one of
+// its pixels.  Block column c spans pixel centres tx0 + 4 c + [0.5, 3.5], row r
+// ty0 + 4 r + [0.5, 3.5]; the mask is the block of columns x rows the box meets.
 __device__ __forceinline__ uint32_t walk_mask(const DevCamera& cam, int32_t tx0, int32_t ty0, float u, float v,
                                               float A, float B, float C, float lthr)
 {
@@ -802,6 +535,194 @@ __device__ __forceinline__ void blend_walk(const DevCamera& cam, uint32_t tile, 
         if (Tout) Tout[pix] = tk;
         // a live pixel did not stop
         if (kKeep && (live & (k ? kPx1 : kPx0))) keep_out[pix] = make_uint2(__float_as_uint(tk), e);
+    }
+}
+
+// ---------------------------------------------------------------------------
+// The KPC pre-render of a tile (Eq. 5-6)
+// ---------------------------------------------------------------------------
+struct KpcWarp {                                  // one warp's: 32 entries at a time
+    float n[32][kParkStride];                     // -power at a block's 16 pixels
+    float w[32][kParkStride];                     // alpha T, 0 where the entry is not applied
+    float a0[32];
+    uint8_t list[4][kWalkChunk];                  // per block: the chunk's records it may meet
+};
+struct KpcSmem {
+    float4 r0[kWalkChunk];                        // u, v, A, B
+    float4 r1[kWalkChunk];                        // C, lthr, alpha0, depth
+    uint16_t mask[kWalkChunk];                    // walk_mask
+    float part[16][kWalkChunk];                   // a record's sum over each block
+    double red[kWalkWarps];
+    KpcWarp w[kWalkWarps];
+};
+
+// blend_walk<8> without an image: after each group of 8 entries of each block a lane
+// an entry sums the applied alpha T over its block's pixels, and after each chunk a
+// thread a record adds up its blocks in their order.  Writes kpc_out of every pair of
+// the tile and the tile's mean G_out[tile] (NaN for a tile without pairs).
+__device__ __forceinline__ void blend_walk_kpc(const DevCamera& cam, uint32_t tile, uint2 rg, KpcSmem& S,
+                                               const uint32_t* __restrict__ vals, const float* __restrict__ splat,
+                                               float* __restrict__ kpc_out, float* __restrict__ G_out,
+                                               const FrameState* st)
+{
+    constexpr uint32_t kC = kWalkChunk;
+    const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint32_t b = lane >> 3, i = lane & 7u;
+    const uint32_t M = st->M;
+    const uint32_t e = rg.y;
+    KpcWarp& W = S.w[warp];
+    uint32_t m = rg.x + tid < e ? __ldg(vals + rg.x + tid) : 0u;
+    const int32_t tx0 = (int32_t)(tile % (uint32_t)cam.tiles_x) * cam.tile_w;
+    const int32_t ty0 = (int32_t)(tile / (uint32_t)cam.tiles_x) * cam.tile_h;
+    int32_t ox, oy;
+    uint32_t bsh;
+    walk_origin(cam, warp, ox, oy, bsh);
+    const int32_t bx0 = tx0 + ox + (int32_t)((b & ((1u << bsh) - 1u)) << 2);
+    const int32_t by0 = ty0 + oy + (int32_t)((b >> bsh) << 2);
+    const int32_t x = bx0 + (int32_t)(i & 3u), y = by0 + (int32_t)(i >> 2 << 1);
+    uint32_t live = x < cam.width ? (y < cam.height ? 0xAAAAAAAAu : 0u) | (y + 1 < cam.height ? 0x55555555u : 0u) : 0u;
+    f32x2 T = dup2(1.0f);
+    f32x2 npx[4], npy[2];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) npx[k] = dup2(-fa((float)(bx0 + k), 0.5f));
+#pragma unroll
+    for (int k = 0; k < 2; ++k)
+        npy[k] = pack2(-fa((float)(by0 + 2 * k), 0.5f), -fa((float)(by0 + 2 * k + 1), 0.5f));
+    double acc = 0.0;                             // this thread's share of the tile's sum (fixed order)
+
+    for (uint32_t s0 = rg.x; s0 < e; s0 += kC) {
+        const uint32_t cnt = e - s0 < kC ? e - s0 : kC;
+        uint32_t my_mask = 0u;
+        if (tid < cnt) {
+            if (m >= M) m = 0;      // only after a failed sort (status already latched)
+            const float4* g = reinterpret_cast<const float4*>(splat + (size_t)m * kSplatStride);
+            const float4 g0 = __ldg(g), g1 = __ldg(g + 1);
+            S.r0[tid] = g0;
+            S.r1[tid] = g1;
+            my_mask = walk_mask(cam, tx0, ty0, g0.x, g0.y, g0.z, g0.w, g1.x, g1.y);
+            S.mask[tid] = (uint16_t)my_mask;
+#pragma unroll
+            for (int k = 0; k < 16; ++k) S.part[k][tid] = 0.0f;
+        }
+        if (s0 + kC + tid < e) m = __ldg(vals + s0 + kC + tid);
+        __syncthreads();
+        if (__any_sync(kFull, live != 0u)) {
+            uint32_t len[4] = {};
+            const uint32_t lt = (1u << lane) - 1u;
+            for (uint32_t j = lane; j < cnt + lane; j += 32) {
+                const uint32_t bm = j < cnt ? (uint32_t)S.mask[j] >> (4u * warp) : 0u;
+#pragma unroll
+                for (uint32_t k = 0; k < 4; ++k) {
+                    const uint32_t v = __ballot_sync(kFull, bm & (1u << k));
+                    if (bm & (1u << k)) W.list[k][len[k] + __popc(v & lt)] = (uint8_t)j;
+                    len[k] += __popc(v);
+                }
+            }
+            __syncwarp();
+            uint32_t left = b == 0 ? len[0] : b == 1 ? len[1] : b == 2 ? len[2] : len[3];
+            const uint32_t en = 7u - i, sl = b * 8u + en;
+            const uint8_t* next = &W.list[b][en];
+            while (__any_sync(kFull, left != 0u)) {
+                // ---- test: one entry a lane at its block's 16 pixels
+                const bool valid = en < left;
+                const uint32_t rs = valid ? *next : 0u;
+                const float4 a = S.r0[rs], c = S.r1[rs];
+                W.a0[sl] = c.z;
+                const f32x2 hA = dup2(fm(0.5f, a.z)), B2 = dup2(a.w), hC = dup2(fm(0.5f, c.x)), K = dup2(-c.y);
+                f32x2 dx[4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) dx[k] = add2(dup2(a.x), npx[k]);
+                uint32_t hits = 0u;
+#pragma unroll
+                for (int rp = 1; rp >= 0; --rp) {
+                    const f32x2 dy = add2(dup2(a.y), npy[rp]);
+                    const f32x2 bdy = mul2(B2, dy), cdy = mul2(mul2(hC, dy), dy);
+                    f32x2 n[4];
+#pragma unroll
+                    for (int k = 3; k >= 0; --k) {
+                        n[k] = fma2(fma2(hA, dx[k], bdy), dx[k], cdy);
+                        const float2 p = unpack2(mul2(n[k], fma2(n[k], dup2(-1.0f), K)));
+                        hits = __funnelshift_l(__float_as_uint(p.x), hits, 1);
+                        hits = __funnelshift_l(__float_as_uint(p.y), hits, 1);
+                    }
+                    float* pn = &W.n[sl][8 * rp];
+                    *reinterpret_cast<ulonglong2*>(pn) = make_ulonglong2(n[0], n[1]);
+                    *reinterpret_cast<ulonglong2*>(pn + 4) = make_ulonglong2(n[2], n[3]);
+                }
+                hits = valid ? ~hits & 0xFFFFu : 0u;
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                    *reinterpret_cast<float4*>(&W.w[sl][4 * k]) = make_float4(0.f, 0.f, 0.f, 0.f);
+                uint32_t mask = (transpose_bits<8>(hits, i) & live) << 16;
+                __syncwarp();
+                // ---- apply
+                while (__any_sync(kFull, mask != 0u)) {
+                    const uint32_t sh = clz_or_ones(mask) & ~1u;
+                    const uint32_t h = mask & shr0(0xC0000000u, sh);
+                    const bool h0 = (h & 0xAAAAAAAAu) != 0u, h1 = (h & 0x55555555u) != 0u;
+                    mask ^= h;
+                    const uint32_t at = b * 8u + ((sh >> 1) & 7u);
+                    const float a0 = W.a0[at];
+                    const float2 n = *reinterpret_cast<const float2*>(&W.n[at][2 * i]);
+                    auto alpha1 = [&](float nn, bool on) {
+                        uint32_t t;
+                        const float p = exp_poly_neg(nn, t);
+                        const float al = fm(a0, fm(p, __uint_as_float((t << 23) + (127u << 23))));
+                        return on ? fminf(al, 0.99f) : 0.0f;
+                    };
+                    const f32x2 al = pack2(alpha1(n.x, h0), alpha1(n.y, h1));
+                    const f32x2 Tn = mul2(T, fma2(al, dup2(-1.0f), dup2(1.0f)));
+                    float2 w = unpack2(mul2(al, T)), tn = unpack2(Tn);
+                    if (fminf(tn.x, tn.y) < 0.0001f) {             // stops before this Gaussian
+                        const float2 to = unpack2(T);
+                        const bool q0 = tn.x < 0.0001f, q1 = tn.y < 0.0001f;
+                        w = make_float2(q0 ? 0.0f : w.x, q1 ? 0.0f : w.y);
+                        tn = make_float2(q0 ? to.x : tn.x, q1 ? to.y : tn.y);
+                        live &= (q0 ? 0x55555555u : kFull) & (q1 ? 0xAAAAAAAAu : kFull);
+                        mask &= live;
+                    }
+                    T = pack2(tn.x, tn.y);
+                    if (h) *reinterpret_cast<float2*>(&W.w[at][2 * i]) = w;
+                }
+                __syncwarp();
+                // ---- gather
+                if (hits) {
+                    f32x2 s2 = 0ull;
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(&W.w[sl][4 * k]);
+                        s2 = add2(v.y, add2(v.x, s2));
+                    }
+                    const float2 f = unpack2(s2);
+                    S.part[4u * warp + b][rs] = f.x + f.y;
+                }
+                __syncwarp();
+                left -= min(left, 8u);
+                next += 8;
+                if (__all_sync(kFull, live == 0u)) break;
+            }
+        }
+        __syncthreads();
+        if (tid < cnt) {
+            float k = 0.0f;
+#pragma unroll
+            for (int h = 0; h < 16; ++h)
+                if ((my_mask >> h) & 1u) k += S.part[h][tid];
+            kpc_out[s0 + tid] = k;
+            acc += (double)k;
+        }
+        __syncthreads();
+    }
+    // Eq. 6: G = mean KPC over the tile's pairs; fixed-order block reduction
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(kFull, acc, o);
+    if (lane == 0) S.red[warp] = acc;
+    __syncthreads();
+    if (tid == 0) {
+        const uint32_t n = e - rg.x;
+        double sum = 0.0;
+        for (int k = 0; k < kWalkWarps; ++k) sum += S.red[k];
+        G_out[tile] = n > 0 ? (float)(sum / (double)n) : __int_as_float(0x7fc00000);
     }
 }
 
