@@ -16,14 +16,16 @@
 //  * segsort_kernel: each bucket is sorted by item.  (depth, rank) is unique
 //    within a tile, so the result does not depend on the scatter order.  Four
 //    forms by bucket size: a warp sorts up to 32 items in registers (bitonic
-//    network, lanes exchange through shuffles) and up to kSegSmall by depth
-//    radix passes through its slice of shared memory (with the fix of
-//    equal-depth runs below; a longer run: the network); a block sorts up to
-//    kSegSmem items by depth with a stable LSD radix sort in shared memory
-//    (and, if two depths are equal, with the bitonic network by (depth, rank)
-//    instead); a block sorts a larger bucket with an LSD radix sort over every
-//    byte in which the items differ, in chunks, between the bucket and the
-//    tile's slots of the key output.  The sorted bucket is written as keys
+//    network, lanes exchange through shuffles) and up to kSegSmall by radix passes
+//    through its slice of shared memory; a block sorts up to kSegSmem items by
+//    radix passes in shared memory, and a larger bucket in chunks between the
+//    bucket and the tile's slots of the key output.  The radix passes cover the
+//    leading 16 bits of the depths' offsets from the bucket's nearest (two passes
+//    instead of up to four: 49 -> 37 us for 1.2M pairs of 1M blobs at 1080p, 75 ->
+//    45 us for a city frame with buckets above kSegSmem; issue and barrier bound),
+//    and the runs of equal ones, which keep the scatter's order, are ordered
+//    where they lie; a bucket with a run longer than kTieRun is sorted by every bit.
+//    The sorted bucket is written as keys
 //    (tile << 32 | depth bits) and values (rank).
 #include "pairs_impl.cuh"
 
@@ -208,6 +210,7 @@ struct RadixSmem {
     uint32_t dcnt[256];                      // a chunk's count of each digit
     uint32_t tmp[kSegThreads / 32];
     unsigned long long vor, vand;            // OR and AND of the bucket's items
+    uint32_t lo, hi;                         // smallest and largest depth of the bucket
 };
 
 __device__ __forceinline__ uint32_t block_excl_scan(uint32_t v, uint32_t* tmp)
@@ -291,38 +294,70 @@ __device__ __forceinline__ void block_or_and(unsigned long long vor, unsigned lo
     __syncthreads();
 }
 
-// Equal depths found after a depth-only sort: the run of equal keys starting at
-// i (keys[i - 1] differs, keys[i + 1] is equal) is put in rank order by
-// insertion sort of its values, if it is at most kTieRun long; returns false,
-// changing nothing, for a longer run.  Only this thread writes the run, and the
-// keys (which other threads read) do not change.
-constexpr uint32_t kTieRun = 32;
-__device__ __forceinline__ bool sort_tie_run(const uint32_t* keys, uint32_t* vals, uint32_t i, uint32_t n)
+// Block-wide minimum and maximum of the depths (every thread passes its own).
+__device__ __forceinline__ void block_min_max(uint32_t lo, uint32_t hi, RadixSmem& R)
 {
+    if (threadIdx.x == 0) {
+        R.lo = 0xFFFFFFFFu;
+        R.hi = 0u;
+    }
+    __syncthreads();
+    lo = __reduce_min_sync(0xffffffffu, lo);
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    if ((threadIdx.x & 31) == 0) {
+        atomicMin(&R.lo, lo);
+        atomicMax(&R.hi, hi);
+    }
+    __syncthreads();
+}
+
+// The depth sorts order a bucket by bits [s0, bl) of the depths' offsets from the
+// bucket's smallest, bl the bits of the largest offset: all of them (s0 = 0), or the
+// leading kCoarseBits, which takes two passes of 8 bits instead of up to four and
+// leaves short runs of equal leading bits (the depths of a tile fill a few octaves of
+// binary32 values, so 65,536 steps between its nearest and farthest put one to a few
+// Gaussians in each).  A run of equal sorted bits keeps the scatter's order; it is put
+// in (depth, rank) order where it lies by the thread holding its first element, by
+// insertion, if it is at most kTieRun long; a longer one sends the bucket to the next
+// slower sort.
+constexpr uint32_t kTieRun = 32;
+constexpr uint32_t kCoarseBits = 16;
+
+__device__ __forceinline__ uint32_t coarse_shift(uint32_t bl) { return bl > kCoarseBits ? bl - kCoarseBits : 0u; }
+
+// Order the run that starts at i (the element before it has other leading bits);
+// false, changing nothing, for a run longer than kTieRun.  Only this thread writes the
+// run, and the leading bits that other threads compare do not change.
+__device__ __forceinline__ bool sort_run(uint32_t* keys, uint32_t* vals, uint32_t base, uint32_t s0, uint32_t i,
+                                         uint32_t n)
+{
+    const uint32_t k = (keys[i] - base) >> s0;
     uint32_t j = i + 1;
-    while (j < n && keys[j] == keys[i]) {
+    while (j < n && (keys[j] - base) >> s0 == k) {
         if (j - i >= kTieRun) return false;
         ++j;
     }
     for (uint32_t a = i + 1; a < j; ++a) {
-        const uint32_t x = vals[a];
+        const uint32_t x = keys[a], v = vals[a];
         uint32_t b = a;
-        while (b > i && vals[b - 1] > x) {
+        while (b > i && (keys[b - 1] > x || (keys[b - 1] == x && vals[b - 1] > v))) {
+            keys[b] = keys[b - 1];
             vals[b] = vals[b - 1];
             --b;
         }
-        vals[b] = x;
+        keys[b] = x;
+        vals[b] = v;
     }
     return true;
 }
 
-// The same for 64-bit items (depth bits << 32 | rank): a run of equal depths
-// sorted by item is sorted by rank.
-__device__ __forceinline__ bool sort_tie_run64(unsigned long long* items, uint32_t i, uint32_t n)
+// The same for 64-bit items (depth bits << 32 | rank).
+__device__ __forceinline__ bool sort_run64(unsigned long long* items, uint32_t base, uint32_t s0, uint32_t i,
+                                           uint32_t n)
 {
-    const uint32_t d = (uint32_t)(items[i] >> 32);
+    const uint32_t k = ((uint32_t)(items[i] >> 32) - base) >> s0;
     uint32_t j = i + 1;
-    while (j < n && (uint32_t)(items[j] >> 32) == d) {
+    while (j < n && ((uint32_t)(items[j] >> 32) - base) >> s0 == k) {
         if (j - i >= kTieRun) return false;
         ++j;
     }
@@ -338,23 +373,20 @@ __device__ __forceinline__ bool sort_tie_run64(unsigned long long* items, uint32
     return true;
 }
 
-// A block sorts n <= 256 I items of one tile by depth with a stable LSD radix
-// sort over the depth bytes in which the items differ, items held in registers
-// and exchanged through shared memory (skeys / svals) after every pass.  Item i
-// of the input order is item it, lane L of warp w with i = (w I + it) 32 + L.
-// Equal depths keep that order, which is the scatter's and not the rank order,
-// so each run of equal depths is then put in rank order where it lies (by the
-// thread holding its first element).  If a run is longer than kTieRun, false is
-// returned and nothing is written (the caller sorts the bucket by (depth, rank)
-// instead); otherwise the sorted pairs are written and true is returned.
+// A block sorts n <= 256 I items of one tile by depth (its leading bits if coarse)
+// with a stable LSD radix sort, items held in registers and exchanged through shared
+// memory (skeys / svals) after every pass.  Item i of the input order is item it, lane
+// L of warp w with i = (w I + it) 32 + L.  Then each run of equal sorted bits is put
+// in order where it lies.  If a run is longer than kTieRun, false is returned and
+// nothing is written; otherwise the sorted pairs are written and true is returned.
 template <int I>
 __device__ bool block_radix_bucket(const unsigned long long* items, uint32_t n, uint32_t tile,
                                    unsigned long long* keys_out, uint32_t* vals_out, uint32_t* skeys,
-                                   uint32_t* svals, RadixSmem& R)
+                                   uint32_t* svals, RadixSmem& R, bool coarse)
 {
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     uint32_t key[I], val[I];
-    unsigned long long vor = 0ull, vand = ~0ull;
+    uint32_t lo = 0xFFFFFFFFu, hi = 0u;
 #pragma unroll
     for (int it = 0; it < I; ++it) {
         const uint32_t i = (warp * I + it) * 32 + lane;
@@ -362,17 +394,17 @@ __device__ bool block_radix_bucket(const unsigned long long* items, uint32_t n, 
         key[it] = (uint32_t)(x >> 32);
         val[it] = (uint32_t)x;
         if (i < n) {
-            vor |= x;
-            vand &= x;
+            lo = min(lo, key[it]);
+            hi = max(hi, key[it]);
         }
     }
-    block_or_and(vor, vand, R);
-    const uint32_t diff = (uint32_t)((R.vor & ~R.vand) >> 32);
-    for (uint32_t shift = 0; shift < 32; shift += 8) {
-        if (((diff >> shift) & 0xFFu) == 0u) continue;
+    block_min_max(lo, hi, R);
+    const uint32_t base = R.lo, bl = 32u - (uint32_t)__clz((int)(R.hi - R.lo));
+    const uint32_t s0 = coarse ? coarse_shift(bl) : 0u;
+    for (uint32_t shift = s0; shift < bl; shift += 8) {
         uint32_t d[I], rank[I];
 #pragma unroll
-        for (int it = 0; it < I; ++it) d[it] = (key[it] >> shift) & 0xFFu;
+        for (int it = 0; it < I; ++it) d[it] = ((key[it] - base) >> shift) & 0xFFu;
         rank_chunk<I>(d, n, R, rank);
         R.dbase[tid] = block_excl_scan(R.dcnt[tid], R.tmp);
         __syncthreads();
@@ -395,7 +427,7 @@ __device__ bool block_radix_bucket(const unsigned long long* items, uint32_t n, 
         }
         __syncthreads();
     }
-    // the depth order into shared memory, then each run of equal depths in rank order
+    // the order into shared memory, then each run in order
 #pragma unroll
     for (int it = 0; it < I; ++it) {
         const uint32_t i = (warp * I + it) * 32 + lane;
@@ -407,8 +439,9 @@ __device__ bool block_radix_bucket(const unsigned long long* items, uint32_t n, 
     __syncthreads();
     bool long_run = false;
     for (uint32_t i = tid; i + 1 < n; i += kSegThreads) {
-        if (skeys[i + 1] == skeys[i] && (i == 0 || skeys[i - 1] != skeys[i]))
-            long_run |= !sort_tie_run(skeys, svals, i, n);
+        const uint32_t k = (skeys[i] - base) >> s0;
+        if ((skeys[i + 1] - base) >> s0 == k && (i == 0 || (skeys[i - 1] - base) >> s0 != k))
+            long_run |= !sort_run(skeys, svals, base, s0, i, n);
     }
     if (__syncthreads_or(long_run)) return false;
     for (uint32_t i = tid; i < n; i += kSegThreads) {
@@ -419,65 +452,48 @@ __device__ bool block_radix_bucket(const unsigned long long* items, uint32_t n, 
     return true;
 }
 
-// A block sorts a bucket of any size by (depth, rank) with stable LSD radix
-// passes over bytes of the 64-bit items, each pass a histogram sweep and a
-// scatter sweep over chunks of 256 I items, between the bucket (a) and the
-// tile's slots of the key output (b) as scratch.  First only the depth bytes in
-// which the items differ: equal depths then keep the scatter's order, so each
-// run of equal depths is put in rank order where it lies; if a run is longer
-// than kTieRun the sort is repeated over every byte in which the items differ
-// (rank bytes first, so equal depths end in rank order; the input order does
-// not matter, (depth, rank) being unique).  The sorted pairs are written
-// to keys_out (which is b) and vals_out.
+// A block sorts a bucket of any size by (depth, rank) with stable LSD radix passes
+// over 8-bit digits of the 64-bit items, each pass a histogram sweep and a scatter
+// sweep over chunks of 256 I items, between the bucket (a) and the tile's slots of the
+// key output (b) as scratch.  First only the leading bits of the depths (two passes),
+// and each run of equal ones put in order where it lies; if a run is longer than
+// kTieRun the sort is repeated over every byte in which the items differ (rank bytes
+// first; the input order does not matter, (depth, rank) being unique).  The sorted
+// pairs are written to keys_out (which is b) and vals_out.
 constexpr int kRadixGlobalItems = 8;
-__device__ void radix_global_passes(unsigned long long*& src, unsigned long long*& dst, uint32_t n,
-                                    unsigned long long diff, RadixSmem& R)
+// One pass over bits [shift, shift + 8) of the items less `base`.
+__device__ void radix_global_pass(const unsigned long long* src, unsigned long long* dst, uint32_t n,
+                                  unsigned long long base, uint32_t shift, RadixSmem& R)
 {
     constexpr int I = kRadixGlobalItems;
     constexpr uint32_t kChunk = 256u * I;
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    for (uint32_t shift = 0; shift < 64; shift += 8) {
-        if (((diff >> shift) & 0xFFull) == 0ull) continue;
-        // histogram of the digit over the bucket, then each digit's first slot
-        uint32_t total = 0;
-        for (uint32_t c0 = 0; c0 < n; c0 += kChunk) {
-            const uint32_t nv = n - c0 < kChunk ? n - c0 : kChunk;
-            uint32_t d[I], rank[I];
+    // histogram of the digit over the bucket, then each digit's first slot
+    R.dcnt[tid] = 0u;
+    __syncthreads();
+    for (uint32_t i = tid; i < n; i += kSegThreads) atomicAdd(&R.dcnt[(uint32_t)((src[i] - base) >> shift) & 0xFFu], 1u);
+    __syncthreads();
+    R.dbase[tid] = block_excl_scan(R.dcnt[tid], R.tmp);
+    __syncthreads();
+    // stable scatter, chunk by chunk in order
+    for (uint32_t c0 = 0; c0 < n; c0 += kChunk) {
+        const uint32_t nv = n - c0 < kChunk ? n - c0 : kChunk;
+        unsigned long long x[I];
+        uint32_t d[I], rank[I];
 #pragma unroll
-            for (int it = 0; it < I; ++it) {
-                const uint32_t i = (warp * I + it) * 32 + lane;
-                d[it] = i < nv ? (uint32_t)(src[c0 + i] >> shift) & 0xFFu : 0u;
-            }
-            rank_chunk<I>(d, nv, R, rank);
-            total += R.dcnt[tid];
-            __syncthreads();
+        for (int it = 0; it < I; ++it) {
+            const uint32_t i = (warp * I + it) * 32 + lane;
+            x[it] = i < nv ? src[c0 + i] : base;
+            d[it] = (uint32_t)((x[it] - base) >> shift) & 0xFFu;
         }
-        R.dbase[tid] = block_excl_scan(total, R.tmp);
+        rank_chunk<I>(d, nv, R, rank);
+#pragma unroll
+        for (int it = 0; it < I; ++it) {
+            if ((warp * I + it) * 32 + lane < nv) dst[R.dbase[d[it]] + R.whist[warp][d[it]] + rank[it]] = x[it];
+        }
         __syncthreads();
-        // stable scatter, chunk by chunk in order
-        for (uint32_t c0 = 0; c0 < n; c0 += kChunk) {
-            const uint32_t nv = n - c0 < kChunk ? n - c0 : kChunk;
-            unsigned long long x[I];
-            uint32_t d[I], rank[I];
-#pragma unroll
-            for (int it = 0; it < I; ++it) {
-                const uint32_t i = (warp * I + it) * 32 + lane;
-                x[it] = i < nv ? src[c0 + i] : 0ull;
-                d[it] = (uint32_t)(x[it] >> shift) & 0xFFu;
-            }
-            rank_chunk<I>(d, nv, R, rank);
-#pragma unroll
-            for (int it = 0; it < I; ++it) {
-                if ((warp * I + it) * 32 + lane < nv)
-                    dst[R.dbase[d[it]] + R.whist[warp][d[it]] + rank[it]] = x[it];
-            }
-            __syncthreads();
-            R.dbase[tid] += R.dcnt[tid];
-            __syncthreads();
-        }
-        unsigned long long* t = src;
-        src = dst;
-        dst = t;
+        R.dbase[tid] += R.dcnt[tid];
+        __syncthreads();
     }
 }
 
@@ -485,26 +501,42 @@ __device__ void block_radix_global(unsigned long long* a, unsigned long long* b,
                                    unsigned long long* keys_out, uint32_t* vals_out, RadixSmem& R)
 {
     const uint32_t tid = threadIdx.x;
-    unsigned long long vor = 0ull, vand = ~0ull;
+    uint32_t lo = 0xFFFFFFFFu, hi = 0u;
     for (uint32_t i = tid; i < n; i += kSegThreads) {
-        const unsigned long long x = a[i];
-        vor |= x;
-        vand &= x;
+        const uint32_t d = (uint32_t)(a[i] >> 32);
+        lo = min(lo, d);
+        hi = max(hi, d);
     }
-    block_or_and(vor, vand, R);
-    const unsigned long long diff = R.vor & ~R.vand;
+    block_min_max(lo, hi, R);
+    const uint32_t base = R.lo, bl = 32u - (uint32_t)__clz((int)(R.hi - R.lo)), s0 = coarse_shift(bl);
     unsigned long long* src = a;
     unsigned long long* dst = b;
-    radix_global_passes(src, dst, n, diff & 0xFFFFFFFF00000000ull, R);
-    // each run of equal depths in rank order where it lies; a run longer than
-    // kTieRun: the full sort instead
+    auto pass = [&](unsigned long long from, uint32_t shift) {
+        radix_global_pass(src, dst, n, from, shift, R);
+        unsigned long long* t = src;
+        src = dst;
+        dst = t;
+    };
+    for (uint32_t shift = s0; shift < bl; shift += 8) pass((unsigned long long)base << 32, 32u + shift);
+    // each run in order where it lies; a run longer than kTieRun: the full sort instead
     bool long_run = false;
     for (uint32_t i = tid; i + 1 < n; i += kSegThreads) {
-        const uint32_t d = (uint32_t)(src[i] >> 32);
-        if ((uint32_t)(src[i + 1] >> 32) == d && (i == 0 || (uint32_t)(src[i - 1] >> 32) != d))
-            long_run |= !sort_tie_run64(src, i, n);
+        const uint32_t k = ((uint32_t)(src[i] >> 32) - base) >> s0;
+        if (((uint32_t)(src[i + 1] >> 32) - base) >> s0 == k &&
+            (i == 0 || ((uint32_t)(src[i - 1] >> 32) - base) >> s0 != k))
+            long_run |= !sort_run64(src, base, s0, i, n);
     }
-    if (__syncthreads_or(long_run)) radix_global_passes(src, dst, n, diff, R);
+    if (__syncthreads_or(long_run)) {
+        unsigned long long vor = 0ull, vand = ~0ull;
+        for (uint32_t i = tid; i < n; i += kSegThreads) {
+            vor |= src[i];
+            vand &= src[i];
+        }
+        block_or_and(vor, vand, R);
+        const unsigned long long diff = R.vor & ~R.vand;
+        for (uint32_t shift = 0; shift < 64; shift += 8)
+            if (((diff >> shift) & 0xFFull) != 0ull) pass(0ull, shift);
+    }
     // src holds the sorted items; a slot of keys_out (= b) is read and then
     // rewritten by the same thread
     for (uint32_t i = tid; i < n; i += kSegThreads) put_pair(src[i], tile, keys_out, vals_out, i);
@@ -512,13 +544,12 @@ __device__ void block_radix_global(unsigned long long* a, unsigned long long* b,
 }
 
 // A warp sorts n <= 32 I items of one tile by (depth, rank), items in registers
-// (item it of lane L is element 32 it + L): stable LSD radix passes over the
-// depth bytes in which the items differ, each ranking the digits with one ballot
-// per digit bit and the warp's 256 counters (hist), the items exchanged through
-// the warp's buffer buf (32 I slots); then each run of equal depths in rank
-// order where it lies, and the pairs written.  Returns false, writing nothing,
-// if a run is longer than kTieRun (the caller sorts the bucket by the bitonic
-// network instead).
+// (item it of lane L is element 32 it + L): stable LSD radix passes over the leading
+// bits of the depths, each ranking the digits with one ballot per digit bit and the
+// warp's 256 counters (hist), the items exchanged through the warp's buffer buf (32 I
+// slots); then each run of equal leading bits in order where it lies, and the pairs
+// written.  Returns false, writing nothing, if a run is longer than kTieRun (the
+// caller sorts the bucket by the bitonic network instead).
 template <int I>
 __device__ bool warp_radix_small(const unsigned long long* items, uint32_t n, uint32_t tile,
                                  unsigned long long* keys_out, uint32_t* vals_out, unsigned long long* buf,
@@ -526,19 +557,20 @@ __device__ bool warp_radix_small(const unsigned long long* items, uint32_t n, ui
 {
     const uint32_t lane = threadIdx.x & 31, lt = (1u << lane) - 1u;
     unsigned long long x[I];
-    uint32_t vor = 0u, vand = ~0u;
+    uint32_t lo = 0xFFFFFFFFu, hi = 0u;
 #pragma unroll
     for (int it = 0; it < I; ++it) {
         const uint32_t i = ((uint32_t)it << 5) + lane;
         x[it] = i < n ? items[i] : ~0ull;
         if (i < n) {
-            vor |= (uint32_t)(x[it] >> 32);
-            vand &= (uint32_t)(x[it] >> 32);
+            lo = min(lo, (uint32_t)(x[it] >> 32));
+            hi = max(hi, (uint32_t)(x[it] >> 32));
         }
     }
-    const uint32_t diff = __reduce_or_sync(0xffffffffu, vor) & ~__reduce_and_sync(0xffffffffu, vand);
-    for (uint32_t shift = 32; shift < 64; shift += 8) {
-        if (((diff >> (shift - 32)) & 0xFFu) == 0u) continue;
+    const uint32_t base = __reduce_min_sync(0xffffffffu, lo);
+    const uint32_t bl = 32u - (uint32_t)__clz((int)(__reduce_max_sync(0xffffffffu, hi) - base));
+    const uint32_t s0 = coarse_shift(bl);
+    for (uint32_t shift = s0; shift < bl; shift += 8) {
 #pragma unroll
         for (int j = 0; j < 8; ++j) hist[lane * 8 + j] = 0u;
         __syncwarp();
@@ -546,7 +578,7 @@ __device__ bool warp_radix_small(const unsigned long long* items, uint32_t n, ui
 #pragma unroll
         for (int it = 0; it < I; ++it) {
             const bool valid = ((uint32_t)it << 5) + lane < n;
-            dg[it] = (uint32_t)(x[it] >> shift) & 0xFFu;
+            dg[it] = (((uint32_t)(x[it] >> 32) - base) >> shift) & 0xFFu;
             uint32_t peers = __ballot_sync(0xffffffffu, valid);
 #pragma unroll
             for (int bit = 0; bit < 8; ++bit) {
@@ -600,9 +632,10 @@ __device__ bool warp_radix_small(const unsigned long long* items, uint32_t n, ui
     __syncwarp();
     bool long_run = false;
     for (uint32_t i = lane; i + 1 < n; i += 32) {
-        const uint32_t d = (uint32_t)(buf[i] >> 32);
-        if ((uint32_t)(buf[i + 1] >> 32) == d && (i == 0 || (uint32_t)(buf[i - 1] >> 32) != d))
-            long_run |= !sort_tie_run64(buf, i, n);
+        const uint32_t k = ((uint32_t)(buf[i] >> 32) - base) >> s0;
+        if (((uint32_t)(buf[i + 1] >> 32) - base) >> s0 == k &&
+            (i == 0 || ((uint32_t)(buf[i - 1] >> 32) - base) >> s0 != k))
+            long_run |= !sort_run64(buf, base, s0, i, n);
     }
     if (__any_sync(0xffffffffu, long_run)) return false;
     __syncwarp();
@@ -898,7 +931,7 @@ __device__ __forceinline__ void list_heavy(uint32_t n, uint32_t split, uint32_t 
     if (k < kSplitTiles) heavy[k] = tile;
 }
 
-__global__ void __launch_bounds__(kSegThreads) segsort_kernel(const uint2* __restrict__ ranges,
+__global__ void __launch_bounds__(kSegThreads, 3) segsort_kernel(const uint2* __restrict__ ranges,
                                                               uint32_t n_tiles,
                                                               const uint32_t* __restrict__ large,
                                                               unsigned long long* items,
@@ -930,10 +963,13 @@ __global__ void __launch_bounds__(kSegThreads) segsort_kernel(const uint2* __res
         if (threadIdx.x == 0) list_heavy(n, split, t, heavy, st);
         if (n <= (uint32_t)kSegSmem) {
             uint32_t* sk = reinterpret_cast<uint32_t*>(s_items);
-            bool done;
-            if (n <= 512u) done = block_radix_bucket<2>(it, n, t, keys_out + r.x, vals_out + r.x, sk, sk + kSegSmem, s_radix);
-            else if (n <= 1024u) done = block_radix_bucket<4>(it, n, t, keys_out + r.x, vals_out + r.x, sk, sk + kSegSmem, s_radix);
-            else done = block_radix_bucket<8>(it, n, t, keys_out + r.x, vals_out + r.x, sk, sk + kSegSmem, s_radix);
+            bool done = false;
+            // by the leading bits of the depth; by all of them; by the network
+            for (int coarse = 1; coarse >= 0 && !done; --coarse) {
+                if (n <= 512u) done = block_radix_bucket<2>(it, n, t, keys_out + r.x, vals_out + r.x, sk, sk + kSegSmem, s_radix, coarse);
+                else if (n <= 1024u) done = block_radix_bucket<4>(it, n, t, keys_out + r.x, vals_out + r.x, sk, sk + kSegSmem, s_radix, coarse);
+                else done = block_radix_bucket<8>(it, n, t, keys_out + r.x, vals_out + r.x, sk, sk + kSegSmem, s_radix, coarse);
+            }
             if (!done) block_bitonic_any(s_items, it, n, t, keys_out + r.x, vals_out + r.x);
         } else {
             block_radix_global(it, keys_out + r.x, n, t, keys_out + r.x, vals_out + r.x, s_radix);
