@@ -87,6 +87,7 @@ struct fgs_ctx {
     unsigned long long* lb_scan = nullptr;   // the tile scan's look-back entries
     uint32_t* heavy = nullptr;      // tiles the blend splits (kSplitTiles)
     float* G = nullptr;
+    float* G_host = nullptr;        // pinned, tile_cap
     // image staging for host outputs: rgb planes + T
     size_t img_cap = 0;
     float* img = nullptr;
@@ -246,6 +247,9 @@ int ensure_tiles(fgs_ctx* c, size_t tiles, size_t pixels)
         if ((r = grow(c, (void**)&c->large, tiles * 4))) return r;
         if ((r = grow(c, (void**)&c->lb_scan, tile_scan_lookback_entries(tiles) * 8))) return r;
         if ((r = grow(c, (void**)&c->G, tiles * 4))) return r;
+        if (c->G_host) cudaFreeHost(c->G_host);
+        c->G_host = nullptr;
+        FGS_CUDA(c, cudaMallocHost((void**)&c->G_host, tiles * 4));
         c->tile_cap = tiles;
     }
     if (pixels > c->img_cap) {
@@ -342,6 +346,11 @@ int check_ready(fgs_ctx* c)
     return FGS_OK;
 }
 
+FrameBegin frame_begin_of(const fgs_ctx* c, const DevCamera& dc)
+{
+    return FrameBegin{c->st, c->tile_cnt, dc.tiles_x * dc.tiles_y, c->sel_cnt, (int)n_sel_tiles(c)};
+}
+
 // Enqueue the frame up to the sorted pair list and its tile ranges.  Returns
 // the number of kernel launches.  Stage events (if ev): filter R&L | ancestor
 // filter + compaction | projection + pair counts | tile ranges | key scatter |
@@ -350,8 +359,9 @@ int enqueue_front(fgs_ctx* c, const DevCamera& dc, cudaStream_t s, cudaEvent_t* 
 {
     const uint32_t tiles = (uint32_t)(dc.tiles_x * dc.tiles_y);
     if (ev) cudaEventRecord(ev[0], s);
-    launch_frame_begin(c->st, c->tile_cnt, (int)tiles, c->sel_cnt, (int)n_sel_tiles(c), s);
-    launch_filter_pred(c->tree, dc, c->pbits, count ? c->st : nullptr, c->sms * c->occ_pred, s);
+    if (count) launch_frame_begin(frame_begin_of(c, dc), s);
+    launch_filter_pred(c->tree, dc, c->pbits, count ? c->st : nullptr, count ? FrameBegin{} : frame_begin_of(c, dc),
+                       c->sms * c->occ_pred, s);
     if (ev) cudaEventRecord(ev[1], s);
     launch_filter_anc(c->tree, c->pbits, c->selbits, c->sel_cnt, c->sms * c->occ_anc, s);
     launch_compact_counted(c->selbits, c->tree.n_pad / 32, c->sel, c->tree.n_pad, c->sel_cnt, c->st, s);
@@ -366,7 +376,7 @@ int enqueue_front(fgs_ctx* c, const DevCamera& dc, cudaStream_t s, cudaEvent_t* 
     launch_segsort(c->ranges, tiles, c->large, c->keys0, c->keys1, c->vals1, c->heavy, c->st,
                    c->sms * c->occ_segsort, s);
     if (ev) cudaEventRecord(ev[6], s);
-    return 8;
+    return count ? 8 : 7;
 }
 
 int read_state(fgs_ctx* c, cudaStream_t s)
@@ -473,6 +483,7 @@ int fgs_destroy(fgs_ctx* c)
         if (b.graph) cudaGraphExecDestroy(b.graph);
     }
     if (c->st_host) cudaFreeHost(c->st_host);
+    if (c->G_host) cudaFreeHost(c->G_host);
     if (c->h_counter) cudaFreeHost(c->h_counter);
     if (c->ev_ready)
         for (int i = 0; i < kEventSlots; ++i)
@@ -754,8 +765,7 @@ int fgs_filter(fgs_ctx* c, void* stream, uint32_t* sel_out, uint32_t cap, uint32
     DeviceGuard g(c->device);
     cudaStream_t s = (cudaStream_t)stream;
     const DevCamera dc = make_devcam(c, false);
-    launch_frame_begin(c->st, c->tile_cnt, dc.tiles_x * dc.tiles_y, c->sel_cnt, (int)n_sel_tiles(c), s);
-    launch_filter_pred(c->tree, dc, c->pbits, nullptr, c->sms * c->occ_pred, s);
+    launch_filter_pred(c->tree, dc, c->pbits, nullptr, frame_begin_of(c, dc), c->sms * c->occ_pred, s);
     launch_filter_anc(c->tree, c->pbits, c->selbits, c->sel_cnt, c->sms * c->occ_anc, s);
     launch_compact_counted(c->selbits, c->tree.n_pad / 32, c->sel, c->tree.n_pad, c->sel_cnt, c->st, s);
     FGS_CUDA(c, cudaGetLastError());
@@ -788,7 +798,7 @@ int fgs_filter_levelwise(fgs_ctx* c, void* stream, uint32_t* sel_out, uint32_t c
     DeviceGuard g(c->device);
     cudaStream_t s = (cudaStream_t)stream;
     const DevCamera dc = make_devcam(c, false);
-    launch_frame_begin(c->st, c->tile_cnt, dc.tiles_x * dc.tiles_y, c->sel_cnt, (int)n_sel_tiles(c), s);
+    launch_frame_begin(frame_begin_of(c, dc), s);
     FGS_CUDA(c, cudaMemsetAsync(c->selbits, 0, c->tree.n_pad / 32 * 4, s));
     c->h_counter[0] = c->root;
     FGS_CUDA(c, cudaMemcpyAsync(c->frontier0, c->h_counter, 4, cudaMemcpyHostToDevice, s));
@@ -1002,20 +1012,23 @@ int kpc_view(fgs_ctx* c, void* stream, bool force_3sigma, double* gbar_out, floa
     c->have_frame = true;
     c->frame_rendered = false;
     c->frame_kept = false;
+    // the state and G with one wait (and G through pinned memory): two waits and two
+    // copies into pageable memory took 40 us of a 1080p view's 320
+    const size_t tiles = (size_t)dc.tiles_x * dc.tiles_y;
+    FGS_CUDA(c, cudaMemcpyAsync(c->G_host, c->G, tiles * 4, cudaMemcpyDeviceToHost, s));
     if ((r = read_state(c, s))) return r;
     if ((r = latched_status(c))) {
         clear_status(c, s);
         return r;
     }
-    const FrameState& h = *c->st_host;
-    const size_t tiles = (size_t)dc.tiles_x * dc.tiles_y;
-    std::vector<float> Gh(tiles);
-    FGS_CUDA(c, cudaMemcpyAsync(Gh.data(), c->G, tiles * 4, cudaMemcpyDeviceToHost, s));
+    const float* Gh = c->G_host;
     const cudaMemcpyKind kind = out_is_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
-    const uint64_t np = std::min<uint64_t>(h.n_pairs, c->pair_cap);
-    if (kpc_out && np) FGS_CUDA(c, cudaMemcpyAsync(kpc_out, c->kpc, std::min(np, kpc_cap) * 4, kind, s));
-    if (G_out) FGS_CUDA(c, cudaMemcpyAsync(G_out, c->G, tiles * 4, kind, s));
-    FGS_CUDA(c, cudaStreamSynchronize(s));
+    const uint64_t np = std::min<uint64_t>(c->st_host->n_pairs, c->pair_cap);
+    const bool copy_kpc = kpc_out && np, copy_G = G_out && out_is_device;
+    if (copy_kpc) FGS_CUDA(c, cudaMemcpyAsync(kpc_out, c->kpc, std::min(np, kpc_cap) * 4, kind, s));
+    if (copy_G) FGS_CUDA(c, cudaMemcpyAsync(G_out, c->G, tiles * 4, kind, s));
+    if (copy_kpc || copy_G) FGS_CUDA(c, cudaStreamSynchronize(s));
+    if (G_out && !out_is_device) std::memcpy(G_out, Gh, tiles * 4);
     // Eq. 7: mean of G over the tiles that have pairs (tile order, float64)
     double sum = 0.0;
     size_t used = 0;

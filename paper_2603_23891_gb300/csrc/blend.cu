@@ -27,7 +27,6 @@ __global__ void __launch_bounds__(blendk::kWalkChunk) blend_kernel(
 {
     __shared__ __align__(128) blendk::WalkSmem<kKeep> S;
     grid_dep_wait();
-    grid_dep_trigger();
     blendk::walk_grid(
         (uint32_t)(cam.tiles_x * cam.tiles_y), ranges, heavy, st,
         [&](uint32_t tile, uint2 rg) {
@@ -44,7 +43,6 @@ __global__ void __launch_bounds__(blendk::kWalkChunk) blend_kpc_kernel(
 {
     __shared__ __align__(128) blendk::KpcSmem S;
     grid_dep_wait();
-    grid_dep_trigger();
     blendk::blend_walk_kpc(cam, blockIdx.x, ranges[blockIdx.x], S, vals, splat, kpc_out, G_out, st);
 }
 

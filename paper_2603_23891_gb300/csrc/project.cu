@@ -17,7 +17,6 @@ __global__ void __launch_bounds__(kProjThreads) project_kernel(
     uint4* __restrict__ foot, uint32_t* __restrict__ tile_cnt, FrameState* st)
 {
     grid_dep_wait();
-    grid_dep_trigger();
     const uint32_t lane = threadIdx.x & 31;
     const uint32_t M = st->M;
     const uint32_t n_groups = (M + kProjThreads - 1) / kProjThreads;
