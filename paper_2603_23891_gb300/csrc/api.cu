@@ -1147,7 +1147,6 @@ int fgs_update_params(fgs_ctx* c, void* stream, const fgs_gauss_params* p)
     const int blocks = (int)std::min<uint64_t>((c->tree.n + 255) / 256, (uint64_t)c->sms * 8);
     launch_prep_params(c->tree, p->mu, p->log_scale, p->quat, p->logit, p->sh, std::max(blocks, 1),
                        (cudaStream_t)stream);
-    launch_chunk_boxes(c->tree, c->sms, (cudaStream_t)stream);     // the centres changed
     FGS_CUDA(c, cudaGetLastError());
     return FGS_OK;
 }

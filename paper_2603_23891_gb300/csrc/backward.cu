@@ -98,15 +98,47 @@ __device__ __forceinline__ float clamp_logit(float l)
 }
 
 // Parameters -> the tree attributes the frame kernels read: mu, Sigma,
-// alpha0 = sigmoid(l), ln alpha0 = -ln(1 + e^{-l}) (l clamped to [-80, 80]), SH.
-__global__ void __launch_bounds__(256) prep_params_kernel(DevTree t, ParamPtrs p)
+// alpha0 = sigmoid(l), ln alpha0 = -ln(1 + e^{-l}) (l clamped to [-80, 80]), the boxes of
+// 128 centres, SH.  Three passes over different data in one launch: the SH rows
+// (coefficients [n][K3] -> rows of sh_stride floats; vec: sh_stride == K3 and the source
+// 16-byte aligned, so one flat copy by 16-byte loads, four in flight a thread), the
+// boxes (a warp a chunk, from the parameters), the attributes (a thread a node).
+// Bound: HBM, 4 (11 + K3) bytes read and 4 (23 + sh_stride) written a node.  1.25M nodes
+// of degree 3: 135 us as three launches with 4-byte SH copies.
+template <int kDeg>
+__global__ void __launch_bounds__(256) prep_kernel(DevTree t, ParamPtrs p, bool vec)
 {
+    grid_dep_wait();
+    const uint32_t tid = blockIdx.x * blockDim.x + threadIdx.x, nt = gridDim.x * blockDim.x;
+    constexpr uint64_t K3 = (kDeg + 1) * (kDeg + 1) * 3;
+    float* sh = const_cast<float*>(t.sh);
+    if (K3 % 4 == 0 && vec) {
+        const uint64_t total = (uint64_t)t.n * K3 / 4;
+        const float4* src = reinterpret_cast<const float4*>(p.sh);
+        float4* dst = reinterpret_cast<float4*>(sh);
+        uint64_t i = tid;
+        for (; i + 3ull * nt < total; i += 4ull * nt) {
+            float4 v[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) v[k] = __ldcs(src + i + (uint64_t)k * nt);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) dst[i + (uint64_t)k * nt] = v[k];
+        }
+        for (; i < total; i += nt) dst[i] = __ldcs(src + i);
+    } else {
+        const uint64_t total = (uint64_t)t.n * K3;
+        for (uint64_t i = tid; i < total; i += nt) {
+            const uint64_t n = i / K3;                              // a multiply: K3 is a constant
+            sh[n * t.sh_stride + (i - n * K3)] = __ldg(p.sh + i);
+        }
+    }
+    chunk_boxes(p.mu, p.n, p.n, t.n_pad >> 7, const_cast<float4*>(t.cbox), tid, nt);
     float* mu = const_cast<float*>(t.mu);
     float* cov = const_cast<float*>(t.cov);
     float* op = const_cast<float*>(t.opacity);
     float* lop = const_cast<float*>(t.ln_opacity);
     const size_t np = t.n_pad, N = p.n;
-    for (uint32_t n = blockIdx.x * blockDim.x + threadIdx.x; n < p.n; n += gridDim.x * blockDim.x) {
+    for (uint32_t n = tid; n < p.n; n += nt) {
 #pragma unroll
         for (int k = 0; k < 3; ++k) mu[k * np + n] = p.mu[k * N + n];
         float c6[6], R[9], s2[3], qh[4], qn;
@@ -121,22 +153,6 @@ __global__ void __launch_bounds__(256) prep_params_kernel(DevTree t, ParamPtrs p
         attr[0] = make_float4(p.mu[n], p.mu[N + n], p.mu[2 * N + n], a0);
         attr[1] = make_float4(c6[0], c6[1], c6[2], c6[3]);
         attr[2] = make_float4(c6[4], c6[5], la0, 0.0f);
-    }
-}
-
-// SH coefficients [n][K3] -> the tree's rows of sh_stride floats, one flat
-// coalesced pass over the source (K3 a compile-time constant: the division is
-// a multiply).
-template <int kDeg>
-__global__ void __launch_bounds__(256) prep_sh_kernel(DevTree t, const float* __restrict__ src)
-{
-    constexpr uint64_t K3 = (kDeg + 1) * (kDeg + 1) * 3;
-    float* sh = const_cast<float*>(t.sh);
-    const uint64_t total = (uint64_t)t.n * K3;
-    for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < total;
-         i += (uint64_t)gridDim.x * blockDim.x) {
-        const uint64_t n = i / K3;
-        sh[n * t.sh_stride + (i - n * K3)] = __ldg(src + i);
     }
 }
 
@@ -454,14 +470,43 @@ __device__ __forceinline__ void blend_bwd_walk(const DevCamera& cam, uint32_t ti
     }
 }
 
+// The parameter gradients to be zeroed (none: n == 0), [per_node[k]][n] floats each.
+struct GradZero {
+    float* p[5];
+    uint32_t per_node[5];
+    uint32_t n;
+};
+
+// This block's share of the zeros, past L2 (nothing reads them soon): 16-byte stores
+// where the array allows.
+__device__ __forceinline__ void zero_share(const GradZero& z)
+{
+    for (int k = 0; k < 5; ++k) {
+        const uint64_t total = (uint64_t)z.per_node[k] * z.n;
+        const uint64_t lo = total * blockIdx.x / gridDim.x, hi = total * (blockIdx.x + 1ull) / gridDim.x;
+        float* p = z.p[k];
+        uint64_t a = lo + ((4ull - (((uint64_t)p / 4ull + lo) & 3ull)) & 3ull);      // the first 16-byte boundary
+        if (a > hi) a = hi;
+        const uint64_t b = a + ((hi - a) & ~3ull);
+        for (uint64_t i = a + 4ull * threadIdx.x; i < b; i += 4ull * blockDim.x)
+            __stcs(reinterpret_cast<float4*>(p + i), make_float4(0.f, 0.f, 0.f, 0.f));
+        if (lo + threadIdx.x < a) p[lo + threadIdx.x] = 0.0f;
+        if (b + threadIdx.x < hi) p[b + threadIdx.x] = 0.0f;
+    }
+}
+
 // keep holds each pixel's {final T, stop} (kept by a FGS_RENDER_KEEP forward, or
-// recomputed by the forward's walk without an image just before).
+// recomputed by the forward's walk without an image just before).  zero: the gradients
+// of nodes outside the selection, written here, where HBM idles (1.25M nodes of degree
+// 3: five memsets of 295 MB in all took 45 us and their launches).
 __global__ void __launch_bounds__(blendk::kWalkChunk) blend_bwd_kernel(
     DevCamera cam, const uint2* __restrict__ ranges, const uint32_t* __restrict__ heavy,
     const uint32_t* __restrict__ vals, const float* __restrict__ splat, const uint2* __restrict__ keep,
-    const float* __restrict__ dL_drgb, float* __restrict__ gsplat, const FrameState* st)
+    const float* __restrict__ dL_drgb, float* __restrict__ gsplat, GradZero zero, const FrameState* st)
 {
     __shared__ __align__(128) BwdSmem S;
+    grid_dep_wait();
+    if (zero.n) zero_share(zero);
     blendk::walk_grid(
         (uint32_t)(cam.tiles_x * cam.tiles_y), ranges, heavy, st,
         [&](uint32_t tile, uint2 rg) {
@@ -547,11 +592,18 @@ struct GradPtrs {
 // Each warp takes 32 consecutive selected Gaussians per iteration, one per
 // lane.  Their SH rows (3 K floats each, contiguous per node) are staged in
 // shared memory with coalesced asynchronous copies, and the SH gradient rows
-// leave the same way; the row stride 3 K + 1 is odd, so lane l reading row l, element k hits
-// bank (l (3 K + 1) + k) mod 32, a different bank for every lane.
+// leave the same way, 16 bytes at a time where the rows are multiples of 16 bytes and
+// the arrays aligned (vec; degrees 1 and 3), else 4.  A lane reads its row four floats
+// at a time: the row stride is a multiple of 4 floats and odd in units of 4, so the 8
+// lanes of a quarter-warp hit different banks.
 __device__ __forceinline__ void cp_async4(float* smem, const float* gmem)
 {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(smem)), "l"(gmem)
+                 : "memory");
+}
+__device__ __forceinline__ void cp_async16(float* smem, const float* gmem)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(smem)), "l"(gmem)
                  : "memory");
 }
 
@@ -563,12 +615,13 @@ template <int kDeg, bool kAccumulate>
 __global__ void __launch_bounds__(kPbWarps * 32, 16 / kPbWarps) project_bwd_kernel(DevTree t, DevCamera cam, ParamPtrs p,
                                                           const uint32_t* __restrict__ sel,
                                                           const float* __restrict__ gsplat,
-                                                          GradPtrs gr, const FrameState* st)
+                                                          GradPtrs gr, bool vec, const FrameState* st)
 {
     constexpr int K = (kDeg + 1) * (kDeg + 1);
-    constexpr int K3 = 3 * K, RS = K3 + 1;
-    __shared__ float s_rows[kPbWarps][32 * RS];
-    __shared__ float s_olds[kAccumulate ? kPbWarps : 1][kAccumulate ? 32 * RS : 1];
+    constexpr int K3 = 3 * K, Q = (K3 + 3) / 4, RS = 4 * (Q | 1);
+    __shared__ __align__(16) float s_rows[kPbWarps][32 * RS];
+    __shared__ __align__(16) float s_olds[kAccumulate ? kPbWarps : 1][kAccumulate ? 32 * RS : 4];
+    grid_dep_wait();
     const uint32_t M = st->M;
     const size_t N = p.n;
     const float* W = cam.R;
@@ -583,12 +636,21 @@ __global__ void __launch_bounds__(kPbWarps * 32, 16 / kPbWarps) project_bwd_kern
         // stage the warp's SH rows (and, accumulating, their current gradient
         // rows) with asynchronous copies: element i * 32 + lane of the 32 x K3
         // block, all in flight at once, no registers held
+        if (K3 % 4 == 0 && vec) {
 #pragma unroll
-        for (int i = 0; i < K3; ++i) {
-            const uint32_t idx = (uint32_t)i * 32u + lane, r = idx / K3, k = idx - r * K3;
-            const uint32_t nr = __shfl_sync(0xffffffffu, n, r);
-            cp_async4(rows + r * RS + k, p.sh + (size_t)nr * K3 + k);
-            if (kAccumulate && base + r < M) cp_async4(olds + r * RS + k, gr.sh + (size_t)nr * K3 + k);
+            for (int i = 0; i < Q; ++i) {
+                const uint32_t idx = (uint32_t)i * 32u + lane, r = idx / Q, k = 4u * (idx - r * Q);
+                const uint32_t nr = __shfl_sync(0xffffffffu, n, r);
+                cp_async16(rows + r * RS + k, p.sh + (size_t)nr * K3 + k);
+                if (kAccumulate && base + r < M) cp_async16(olds + r * RS + k, gr.sh + (size_t)nr * K3 + k);
+            }
+        } else {
+            for (int i = 0; i < K3; ++i) {
+                const uint32_t idx = (uint32_t)i * 32u + lane, r = idx / K3, k = idx - r * K3;
+                const uint32_t nr = __shfl_sync(0xffffffffu, n, r);
+                cp_async4(rows + r * RS + k, p.sh + (size_t)nr * K3 + k);
+                if (kAccumulate && base + r < M) cp_async4(olds + r * RS + k, gr.sh + (size_t)nr * K3 + k);
+            }
         }
         cp_async_wait_all();
         __syncwarp();
@@ -693,30 +755,55 @@ __global__ void __launch_bounds__(kPbWarps * 32, 16 / kPbWarps) project_bwd_kern
         for (int k = 0; k < 3; ++k) d[k] *= idl;
         float Y[16], dY[16][3];
         sh_basis_grad<kDeg>(d[0], d[1], d[2], Y, dY);
-        float gd[3] = {0.0f, 0.0f, 0.0f};
+        float gd[3] = {0.0f, 0.0f, 0.0f}, g3[3] = {0.5f, 0.5f, 0.5f};
+        float4* row4 = reinterpret_cast<float4*>(row);
 #pragma unroll
-        for (int ch = 0; ch < 3; ++ch) {
-            float pre = 0.5f;
+        for (int v = 0; v < Q; ++v) {
+            const float4 f = row4[v];
+            const float e[4] = {f.x, f.y, f.z, f.w};
 #pragma unroll
-            for (int k = 0; k < K; ++k) pre += Y[k] * row[3 * k + ch];
-            const float g = pre > 0.0f ? gcol[ch] : 0.0f;
+            for (int r = 0; r < 4; ++r)
+                if (4 * v + r < K3) g3[(4 * v + r) % 3] += Y[(4 * v + r) / 3] * e[r];
+        }
 #pragma unroll
-            for (int k = 0; k < K; ++k) {
-                const float cg = row[3 * k + ch] * g;
-                gd[0] += cg * dY[k][0];
-                gd[1] += cg * dY[k][1];
-                gd[2] += cg * dY[k][2];
-                row[3 * k + ch] = Y[k] * g;      // the row now holds the SH gradient
-            }
+        for (int ch = 0; ch < 3; ++ch) g3[ch] = g3[ch] > 0.0f ? gcol[ch] : 0.0f;
+#pragma unroll
+        for (int v = 0; v < Q; ++v) {
+            const float4 f = row4[v];
+            float e[4] = {f.x, f.y, f.z, f.w};
+#pragma unroll
+            for (int r = 0; r < 4; ++r)
+                if (4 * v + r < K3) {
+                    const int k = (4 * v + r) / 3, ch = (4 * v + r) % 3;      // compile-time after unrolling
+                    const float cg = e[r] * g3[ch];
+                    gd[0] += cg * dY[k][0];
+                    gd[1] += cg * dY[k][1];
+                    gd[2] += cg * dY[k][2];
+                    e[r] = Y[k] * g3[ch];              // the row now holds the SH gradient
+                }
+            row4[v] = make_float4(e[0], e[1], e[2], e[3]);
         }
         __syncwarp();
         // SH gradient rows out, coalesced
+        if (K3 % 4 == 0 && vec) {
 #pragma unroll
-        for (int i = 0; i < K3; ++i) {
-            const uint32_t idx = (uint32_t)i * 32u + lane, r = idx / K3, k = idx - r * K3;
-            const uint32_t nr = __shfl_sync(0xffffffffu, n, r);
-            const float g = rows[r * RS + k] + (kAccumulate ? olds[r * RS + k] : 0.0f);
-            if (base + r < M) gr.sh[(size_t)nr * K3 + k] = g;
+            for (int i = 0; i < Q; ++i) {
+                const uint32_t idx = (uint32_t)i * 32u + lane, r = idx / Q, k = 4u * (idx - r * Q);
+                const uint32_t nr = __shfl_sync(0xffffffffu, n, r);
+                float4 g = *reinterpret_cast<const float4*>(rows + r * RS + k);
+                if (kAccumulate) {
+                    const float4 o = *reinterpret_cast<const float4*>(olds + r * RS + k);
+                    g = make_float4(g.x + o.x, g.y + o.y, g.z + o.z, g.w + o.w);
+                }
+                if (base + r < M) *reinterpret_cast<float4*>(gr.sh + (size_t)nr * K3 + k) = g;
+            }
+        } else {
+            for (int i = 0; i < K3; ++i) {
+                const uint32_t idx = (uint32_t)i * 32u + lane, r = idx / K3, k = idx - r * K3;
+                const uint32_t nr = __shfl_sync(0xffffffffu, n, r);
+                const float g = rows[r * RS + k] + (kAccumulate ? olds[r * RS + k] : 0.0f);
+                if (base + r < M) gr.sh[(size_t)nr * K3 + k] = g;
+            }
         }
         __syncwarp();
         if (!act) continue;
@@ -761,6 +848,7 @@ __global__ void __launch_bounds__(kPbWarps * 32, 16 / kPbWarps) project_bwd_kern
 
 __global__ void __launch_bounds__(128) zero_rows_kernel(float4* __restrict__ gsplat, const FrameState* st)
 {
+    grid_dep_wait();
     const uint32_t n4 = st->M * (uint32_t)(kGS / 4);
     for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n4; i += gridDim.x * blockDim.x)
         gsplat[i] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
@@ -772,25 +860,28 @@ __global__ void __launch_bounds__(128) zero_rows_kernel(float4* __restrict__ gsp
 void launch_prep_params(const DevTree& t, const float* mu, const float* log_scale, const float* quat,
                         const float* logit, const float* sh, int blocks, cudaStream_t s)
 {
-    ParamPtrs p{mu, log_scale, quat, logit, sh, t.n};
-    prep_params_kernel<<<blocks, 256, 0, s>>>(t, p);
+    const ParamPtrs p{mu, log_scale, quat, logit, sh, t.n};
+    const uint32_t K3 = (t.sh_degree + 1) * (t.sh_degree + 1) * 3;
+    const bool vec = t.sh_stride == K3 && ((uintptr_t)sh & 15u) == 0;
     switch (t.sh_degree) {
-    case 0: prep_sh_kernel<0><<<blocks, 256, 0, s>>>(t, sh); break;
-    case 1: prep_sh_kernel<1><<<blocks, 256, 0, s>>>(t, sh); break;
-    case 2: prep_sh_kernel<2><<<blocks, 256, 0, s>>>(t, sh); break;
-    default: prep_sh_kernel<3><<<blocks, 256, 0, s>>>(t, sh); break;
+    case 0: launch_pdl(prep_kernel<0>, blocks, 256, 0, s, t, p, vec); break;
+    case 1: launch_pdl(prep_kernel<1>, blocks, 256, 0, s, t, p, vec); break;
+    case 2: launch_pdl(prep_kernel<2>, blocks, 256, 0, s, t, p, vec); break;
+    default: launch_pdl(prep_kernel<3>, blocks, 256, 0, s, t, p, vec); break;
     }
 }
 
 template <int kDeg>
 static void launch_project_bwd(const DevTree& t, const DevCamera& cam, const ParamPtrs& p,
                                const uint32_t* sel, const float* gsplat, const GradPtrs& gr,
-                               bool accumulate, int blocks, FrameState* st, cudaStream_t s)
+                               bool accumulate, int blocks, const FrameState* st, cudaStream_t s)
 {
+    constexpr int K3 = 3 * (kDeg + 1) * (kDeg + 1);
+    const bool vec = K3 % 4 == 0 && (((uintptr_t)p.sh | (uintptr_t)gr.sh) & 15u) == 0;
     if (accumulate)
-        project_bwd_kernel<kDeg, true><<<blocks, kPbWarps * 32, 0, s>>>(t, cam, p, sel, gsplat, gr, st);
+        launch_pdl(project_bwd_kernel<kDeg, true>, blocks, kPbWarps * 32, 0, s, t, cam, p, sel, gsplat, gr, vec, st);
     else
-        project_bwd_kernel<kDeg, false><<<blocks, kPbWarps * 32, 0, s>>>(t, cam, p, sel, gsplat, gr, st);
+        launch_pdl(project_bwd_kernel<kDeg, false>, blocks, kPbWarps * 32, 0, s, t, cam, p, sel, gsplat, gr, vec, st);
 }
 
 void launch_backward(const DevTree& t, const DevCamera& cam, const uint2* ranges, const uint32_t* heavy,
@@ -800,22 +891,16 @@ void launch_backward(const DevTree& t, const DevCamera& cam, const uint2* ranges
                      int sms, FrameState* st, cudaStream_t s)
 {
     // gsplat rows of the selected Gaussians start at zero: the blend backward adds into them
-    zero_rows_kernel<<<sms * 8, 128, 0, s>>>(reinterpret_cast<float4*>(gsplat), st);
+    launch_pdl(zero_rows_kernel, sms * 8, 128, 0, s, reinterpret_cast<float4*>(gsplat), st);
     if (!kept) launch_blend(cam, ranges, heavy, vals, splat, nullptr, nullptr, keep, st, false, s);
-    const int n_tiles = cam.tiles_x * cam.tiles_y;
-    blend_bwd_kernel<<<n_tiles + 2 * split_slots(n_tiles), blendk::kWalkChunk, 0, s>>>(cam, ranges, heavy, vals, splat,
-                                                                                     keep, dL_drgb, gsplat, st);
     const ParamPtrs p{params[0], params[1], params[2], params[3], params[4], t.n};
     const GradPtrs gr{grads[0], grads[1], grads[2], grads[3], grads[4]};
-    if (!accumulate) {
-        // nodes outside the selection get zero gradient
-        const size_t K3 = (size_t)(t.sh_degree + 1) * (t.sh_degree + 1) * 3;
-        cudaMemsetAsync(gr.mu, 0, sizeof(float) * 3 * t.n, s);
-        cudaMemsetAsync(gr.log_scale, 0, sizeof(float) * 3 * t.n, s);
-        cudaMemsetAsync(gr.quat, 0, sizeof(float) * 4 * t.n, s);
-        cudaMemsetAsync(gr.logit, 0, sizeof(float) * t.n, s);
-        cudaMemsetAsync(gr.sh, 0, sizeof(float) * K3 * t.n, s);
-    }
+    // nodes outside the selection get zero gradient
+    const uint32_t K3 = (t.sh_degree + 1) * (t.sh_degree + 1) * 3;
+    const GradZero zero{{gr.mu, gr.log_scale, gr.quat, gr.logit, gr.sh}, {3, 3, 4, 1, K3}, accumulate ? 0u : t.n};
+    const int n_tiles = cam.tiles_x * cam.tiles_y;
+    launch_pdl(blend_bwd_kernel, n_tiles + 2 * split_slots(n_tiles), blendk::kWalkChunk, 0, s, cam, ranges, heavy, vals,
+               splat, keep, dL_drgb, gsplat, zero, st);
     const int blocks = sms * (16 / kPbWarps);
     switch (t.sh_degree) {
     case 0: launch_project_bwd<0>(t, cam, p, sel, gsplat, gr, accumulate, blocks, st, s); break;

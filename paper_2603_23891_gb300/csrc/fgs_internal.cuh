@@ -221,6 +221,41 @@ __device__ __forceinline__ bool chunk_outside(const FrustumPlanes& F, float4 lo,
     return out;
 }
 
+// The box of the centres mu[3][stride] (n nodes) of each of n_box chunks of 128
+// consecutive nodes: one warp a chunk, four nodes a lane; thread tid of n_threads (whole
+// warps).  A chunk of padding only gets lo.x > hi.x.  Run after every change of the
+// centres (tree upload, parameter map).
+__device__ __forceinline__ void chunk_boxes(const float* __restrict__ mu, size_t stride, uint32_t n, uint32_t n_box,
+                                            float4* __restrict__ box, uint32_t tid, uint32_t n_threads)
+{
+    const uint32_t lane = tid & 31;
+    for (uint32_t b = tid >> 5; b < n_box; b += n_threads >> 5) {
+        float lo[3] = {1e30f, 1e30f, 1e30f}, hi[3] = {-1e30f, -1e30f, -1e30f};
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const uint32_t i = (b << 7) + (k << 5) + lane;
+            if (i < n)
+#pragma unroll
+                for (int q = 0; q < 3; ++q) {
+                    const float v = mu[(size_t)q * stride + i];
+                    lo[q] = fminf(lo[q], v);
+                    hi[q] = fmaxf(hi[q], v);
+                }
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+            for (int q = 0; q < 3; ++q) {
+                lo[q] = fminf(lo[q], __shfl_xor_sync(0xffffffffu, lo[q], o));
+                hi[q] = fmaxf(hi[q], __shfl_xor_sync(0xffffffffu, hi[q], o));
+            }
+        if (lane == 0) {
+            box[2 * b] = make_float4(lo[0], lo[1], lo[2], 0.0f);
+            box[2 * b + 1] = make_float4(hi[0], hi[1], hi[2], 0.0f);
+        }
+    }
+}
+
 // Sigma_2D and lambda_max for an in-frustum node.  s = {xx, xy, xz, yy, yz, zz}.
 __device__ __forceinline__ void ewa_cov2d(const DevCamera& cam, float vz, float txtz, float tytz,
                                           const float s[6], float& a, float& b, float& c, float& lam)
@@ -475,6 +510,7 @@ void launch_batch_front(const DevTree& t, const DevCamera* cams, int V, uint32_t
 void launch_batch_blend(const DevCamera* cams, int V, uint32_t total_tiles, const uint32_t* tile_base,
                         const unsigned long long* img_off, const uint2* ranges, const uint32_t* heavy,
                         const uint32_t* vals, const float* splat, float* rgb, float* T, FrameState* st, cudaStream_t s);
+// Attributes, chunk boxes and SH of the tree from the parameters.
 void launch_prep_params(const DevTree& t, const float* mu, const float* log_scale, const float* quat,
                         const float* logit, const float* sh, int blocks, cudaStream_t s);
 // keep: per-pixel {final T, stop} buffer; kept: the last forward filled it

@@ -160,40 +160,11 @@ __global__ void __launch_bounds__(256) filter_pred_kernel(DevTree t, DevCamera c
     }
 }
 
-// The box of the centres of each 128 consecutive nodes (one warp a chunk, four
-// nodes a lane); a chunk of padding only gets lo.x > hi.x.  Run after every change
-// of the centres (tree upload, parameter map).
+// The boxes of 128 consecutive centres (chunk_boxes), after a tree upload.
 __global__ void __launch_bounds__(256) chunk_boxes_kernel(DevTree t)
 {
-    const uint32_t lane = threadIdx.x & 31;
-    const uint32_t n_box = t.n_pad >> 7;
-    float4* box = const_cast<float4*>(t.cbox);
-    for (uint32_t b = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; b < n_box;
-         b += (gridDim.x * blockDim.x) >> 5) {
-        float lo[3] = {1e30f, 1e30f, 1e30f}, hi[3] = {-1e30f, -1e30f, -1e30f};
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const uint32_t n = (b << 7) + (lane << 2) + k;
-            if (n < t.n)
-#pragma unroll
-                for (int q = 0; q < 3; ++q) {
-                    const float v = t.mu[(size_t)q * t.n_pad + n];
-                    lo[q] = fminf(lo[q], v);
-                    hi[q] = fmaxf(hi[q], v);
-                }
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-            for (int q = 0; q < 3; ++q) {
-                lo[q] = fminf(lo[q], __shfl_xor_sync(0xffffffffu, lo[q], o));
-                hi[q] = fmaxf(hi[q], __shfl_xor_sync(0xffffffffu, hi[q], o));
-            }
-        if (lane == 0) {
-            box[2 * b] = make_float4(lo[0], lo[1], lo[2], 0.0f);
-            box[2 * b + 1] = make_float4(hi[0], hi[1], hi[2], 0.0f);
-        }
-    }
+    chunk_boxes(t.mu, t.n_pad, t.n, t.n_pad >> 7, const_cast<float4*>(t.cbox), blockIdx.x * blockDim.x + threadIdx.x,
+                gridDim.x * blockDim.x);
 }
 
 void launch_chunk_boxes(const DevTree& t, int sms, cudaStream_t s)
