@@ -475,15 +475,16 @@ struct GradZero {
     float* p[5];
     uint32_t per_node[5];
     uint32_t n;
+    uint32_t blocks;
 };
 
-// This block's share of the zeros, past L2 (nothing reads them soon): 16-byte stores
-// where the array allows.
-__device__ __forceinline__ void zero_share(const GradZero& z)
+// Block `part` of n_parts' share of the zeros, past L2 (nothing reads them soon): 16-byte
+// stores where the array allows.
+__device__ __forceinline__ void zero_share(const GradZero& z, uint32_t part, uint32_t n_parts)
 {
     for (int k = 0; k < 5; ++k) {
         const uint64_t total = (uint64_t)z.per_node[k] * z.n;
-        const uint64_t lo = total * blockIdx.x / gridDim.x, hi = total * (blockIdx.x + 1ull) / gridDim.x;
+        const uint64_t lo = total * part / n_parts, hi = total * (part + 1ull) / n_parts;
         float* p = z.p[k];
         uint64_t a = lo + ((4ull - (((uint64_t)p / 4ull + lo) & 3ull)) & 3ull);      // the first 16-byte boundary
         if (a > hi) a = hi;
@@ -497,8 +498,10 @@ __device__ __forceinline__ void zero_share(const GradZero& z)
 
 // keep holds each pixel's {final T, stop} (kept by a FGS_RENDER_KEEP forward, or
 // recomputed by the forward's walk without an image just before).  zero: the gradients
-// of nodes outside the selection, written here, where HBM idles (1.25M nodes of degree
-// 3: five memsets of 295 MB in all took 45 us and their launches).
+// of nodes outside the selection, written by the first zero.blocks blocks beside the
+// walk, where HBM idles (1.25M nodes of degree 3: five memsets of 295 MB in all took 45 us
+// and their launches; a share of the zeros in every block delayed its walk, 252 us
+// instead of 190).
 __global__ void __launch_bounds__(blendk::kWalkChunk) blend_bwd_kernel(
     DevCamera cam, const uint2* __restrict__ ranges, const uint32_t* __restrict__ heavy,
     const uint32_t* __restrict__ vals, const float* __restrict__ splat, const uint2* __restrict__ keep,
@@ -506,9 +509,12 @@ __global__ void __launch_bounds__(blendk::kWalkChunk) blend_bwd_kernel(
 {
     __shared__ __align__(128) BwdSmem S;
     grid_dep_wait();
-    if (zero.n) zero_share(zero);
+    if (blockIdx.x < zero.blocks) {
+        zero_share(zero, blockIdx.x, zero.blocks);
+        return;
+    }
     blendk::walk_grid(
-        (uint32_t)(cam.tiles_x * cam.tiles_y), ranges, heavy, st,
+        blockIdx.x - zero.blocks, gridDim.x - zero.blocks, (uint32_t)(cam.tiles_x * cam.tiles_y), ranges, heavy, st,
         [&](uint32_t tile, uint2 rg) {
             blend_bwd_walk<8>(cam, tile, 0u, rg, S, vals, splat, keep, dL_drgb, gsplat, st);
         },
@@ -595,7 +601,9 @@ struct GradPtrs {
 // leave the same way, 16 bytes at a time where the rows are multiples of 16 bytes and
 // the arrays aligned (vec; degrees 1 and 3), else 4.  A lane reads its row four floats
 // at a time: the row stride is a multiple of 4 floats and odd in units of 4, so the 8
-// lanes of a quarter-warp hit different banks.
+// lanes of a quarter-warp hit different banks.  Bound: the latency of the rows (8 blocks
+// of 2 warps an SM, by shared memory and registers), so the next group's rows are copied
+// while this one is computed; accumulating, the second buffer holds the old gradients.
 __device__ __forceinline__ void cp_async4(float* smem, const float* gmem)
 {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(smem)), "l"(gmem)
@@ -607,8 +615,6 @@ __device__ __forceinline__ void cp_async16(float* smem, const float* gmem)
                  : "memory");
 }
 
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
-
 constexpr int kPbWarps = 2;   // warps per projection-backward block
 
 template <int kDeg, bool kAccumulate>
@@ -619,40 +625,58 @@ __global__ void __launch_bounds__(kPbWarps * 32, 16 / kPbWarps) project_bwd_kern
 {
     constexpr int K = (kDeg + 1) * (kDeg + 1);
     constexpr int K3 = 3 * K, Q = (K3 + 3) / 4, RS = 4 * (Q | 1);
-    __shared__ __align__(16) float s_rows[kPbWarps][32 * RS];
+    constexpr int kBuf = kAccumulate ? 1 : 2;         // row buffers: the next group's rows land during this one's work
+    __shared__ __align__(16) float s_rows[kPbWarps][kBuf][32 * RS];
     __shared__ __align__(16) float s_olds[kAccumulate ? kPbWarps : 1][kAccumulate ? 32 * RS : 4];
     grid_dep_wait();
     const uint32_t M = st->M;
     const size_t N = p.n;
     const float* W = cam.R;
     const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    float* rows = s_rows[warp];
     float* olds = s_olds[kAccumulate ? warp : 0];
-    float* row = rows + lane * RS;
-    for (uint32_t base = (blockIdx.x * kPbWarps + warp) * 32; base < M; base += gridDim.x * kPbWarps * 32) {
-        const uint32_t m = base + lane;
-        const bool act = m < M;
-        const uint32_t n = act ? sel[m] : sel[base];
-        // stage the warp's SH rows (and, accumulating, their current gradient
-        // rows) with asynchronous copies: element i * 32 + lane of the 32 x K3
-        // block, all in flight at once, no registers held
+    const uint32_t step = gridDim.x * kPbWarps * 32;
+    auto node = [&](uint32_t at) { return at < M ? sel[min(at + lane, M - 1u)] : 0u; };
+    // the SH rows of the group at `at` (nodes nn, one a lane; and, accumulating, their
+    // current gradient rows) with asynchronous copies, all in flight at once
+    auto stage = [&](uint32_t at, uint32_t nn, float* to) {
+        if (at >= M) return;
         if (K3 % 4 == 0 && vec) {
 #pragma unroll
             for (int i = 0; i < Q; ++i) {
                 const uint32_t idx = (uint32_t)i * 32u + lane, r = idx / Q, k = 4u * (idx - r * Q);
-                const uint32_t nr = __shfl_sync(0xffffffffu, n, r);
-                cp_async16(rows + r * RS + k, p.sh + (size_t)nr * K3 + k);
-                if (kAccumulate && base + r < M) cp_async16(olds + r * RS + k, gr.sh + (size_t)nr * K3 + k);
+                const uint32_t nr = __shfl_sync(0xffffffffu, nn, r);
+                cp_async16(to + r * RS + k, p.sh + (size_t)nr * K3 + k);
+                if (kAccumulate && at + r < M) cp_async16(olds + r * RS + k, gr.sh + (size_t)nr * K3 + k);
             }
         } else {
             for (int i = 0; i < K3; ++i) {
                 const uint32_t idx = (uint32_t)i * 32u + lane, r = idx / K3, k = idx - r * K3;
-                const uint32_t nr = __shfl_sync(0xffffffffu, n, r);
-                cp_async4(rows + r * RS + k, p.sh + (size_t)nr * K3 + k);
-                if (kAccumulate && base + r < M) cp_async4(olds + r * RS + k, gr.sh + (size_t)nr * K3 + k);
+                const uint32_t nr = __shfl_sync(0xffffffffu, nn, r);
+                cp_async4(to + r * RS + k, p.sh + (size_t)nr * K3 + k);
+                if (kAccumulate && at + r < M) cp_async4(olds + r * RS + k, gr.sh + (size_t)nr * K3 + k);
             }
         }
-        cp_async_wait_all();
+    };
+    uint32_t base = (blockIdx.x * kPbWarps + warp) * 32;
+    uint32_t n = node(base);
+    if (kBuf == 2) {
+        stage(base, n, s_rows[warp][0]);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    }
+    for (uint32_t buf = 0; base < M; base += step, buf ^= (uint32_t)(kBuf - 1)) {
+        const uint32_t m = base + lane;
+        const bool act = m < M;
+        float* rows = s_rows[warp][buf];
+        float* row = rows + lane * RS;
+        const uint32_t n_next = base + step < M ? node(base + step) : 0u;
+        if (kBuf == 2) {
+            stage(base + step, n_next, s_rows[warp][buf ^ 1u]);
+            asm volatile("cp.async.commit_group;" ::: "memory");
+            asm volatile("cp.async.wait_group 1;" ::: "memory");
+        } else {
+            stage(base, n, rows);
+            asm volatile("cp.async.wait_all;" ::: "memory");
+        }
         __syncwarp();
         const float* gs = gsplat + (size_t)(act ? m : base) * kGS;
         const float gu = gs[0], gv = gs[1], gA = gs[2], gB = gs[3], gC = gs[4], ga0 = gs[5];
@@ -806,6 +830,8 @@ __global__ void __launch_bounds__(kPbWarps * 32, 16 / kPbWarps) project_bwd_kern
             }
         }
         __syncwarp();
+        const uint32_t nn = n;
+        n = n_next;
         if (!act) continue;
         const float dd = gd[0] * d[0] + gd[1] * d[1] + gd[2] * d[2];
 #pragma unroll
@@ -819,29 +845,29 @@ __global__ void __launch_bounds__(kPbWarps * 32, 16 / kPbWarps) project_bwd_kern
             float o_mu[3], o_ls[3], o_q[4];
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
-                o_mu[k] = gr.mu[k * N + n];
-                o_ls[k] = gr.log_scale[k * N + n];
+                o_mu[k] = gr.mu[k * N + nn];
+                o_ls[k] = gr.log_scale[k * N + nn];
             }
 #pragma unroll
-            for (int k = 0; k < 4; ++k) o_q[k] = gr.quat[k * N + n];
-            const float o_l = gr.logit[n];
+            for (int k = 0; k < 4; ++k) o_q[k] = gr.quat[k * N + nn];
+            const float o_l = gr.logit[nn];
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
-                gr.mu[k * N + n] = o_mu[k] + gmu[k];
-                gr.log_scale[k * N + n] = o_ls[k] + gls[k];
+                gr.mu[k * N + nn] = o_mu[k] + gmu[k];
+                gr.log_scale[k * N + nn] = o_ls[k] + gls[k];
             }
 #pragma unroll
-            for (int k = 0; k < 4; ++k) gr.quat[k * N + n] = o_q[k] + gqn[k];
-            gr.logit[n] = o_l + glogit;
+            for (int k = 0; k < 4; ++k) gr.quat[k * N + nn] = o_q[k] + gqn[k];
+            gr.logit[nn] = o_l + glogit;
         } else {
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
-                gr.mu[k * N + n] = gmu[k];
-                gr.log_scale[k * N + n] = gls[k];
+                gr.mu[k * N + nn] = gmu[k];
+                gr.log_scale[k * N + nn] = gls[k];
             }
 #pragma unroll
-            for (int k = 0; k < 4; ++k) gr.quat[k * N + n] = gqn[k];
-            gr.logit[n] = glogit;
+            for (int k = 0; k < 4; ++k) gr.quat[k * N + nn] = gqn[k];
+            gr.logit[nn] = glogit;
         }
     }
 }
@@ -897,10 +923,10 @@ void launch_backward(const DevTree& t, const DevCamera& cam, const uint2* ranges
     const GradPtrs gr{grads[0], grads[1], grads[2], grads[3], grads[4]};
     // nodes outside the selection get zero gradient
     const uint32_t K3 = (t.sh_degree + 1) * (t.sh_degree + 1) * 3;
-    const GradZero zero{{gr.mu, gr.log_scale, gr.quat, gr.logit, gr.sh}, {3, 3, 4, 1, K3}, accumulate ? 0u : t.n};
+    const GradZero zero{{gr.mu, gr.log_scale, gr.quat, gr.logit, gr.sh}, {3, 3, 4, 1, K3}, t.n, accumulate ? 0u : (uint32_t)sms};
     const int n_tiles = cam.tiles_x * cam.tiles_y;
-    launch_pdl(blend_bwd_kernel, n_tiles + 2 * split_slots(n_tiles), blendk::kWalkChunk, 0, s, cam, ranges, heavy, vals,
-               splat, keep, dL_drgb, gsplat, zero, st);
+    launch_pdl(blend_bwd_kernel, n_tiles + 2 * split_slots(n_tiles) + (int)zero.blocks, blendk::kWalkChunk, 0, s, cam,
+               ranges, heavy, vals, splat, keep, dL_drgb, gsplat, zero, st);
     const int blocks = sms * (16 / kPbWarps);
     switch (t.sh_degree) {
     case 0: launch_project_bwd<0>(t, cam, p, sel, gsplat, gr, accumulate, blocks, st, s); break;

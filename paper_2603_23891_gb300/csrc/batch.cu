@@ -225,7 +225,7 @@ __global__ void __launch_bounds__(blendk::kWalkChunk) bblend_kernel(
         return __ldg(img_off + lo);
     };
     blendk::walk_grid(
-        total_tiles, ranges, heavy, st,
+        blockIdx.x, gridDim.x, total_tiles, ranges, heavy, st,
         [&](uint32_t gtile, uint2 rg) {
             uint32_t base;
             const unsigned long long o = locate(gtile, base);

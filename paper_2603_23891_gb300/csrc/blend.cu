@@ -28,7 +28,7 @@ __global__ void __launch_bounds__(blendk::kWalkChunk) blend_kernel(
     __shared__ __align__(128) blendk::WalkSmem<kKeep> S;
     grid_dep_wait();
     blendk::walk_grid(
-        (uint32_t)(cam.tiles_x * cam.tiles_y), ranges, heavy, st,
+        blockIdx.x, gridDim.x, (uint32_t)(cam.tiles_x * cam.tiles_y), ranges, heavy, st,
         [&](uint32_t tile, uint2 rg) {
             blendk::blend_walk<8, kCount, kKeep>(cam, tile, 0u, rg, S, vals, splat, rgb, Tout, keep, st);
         },

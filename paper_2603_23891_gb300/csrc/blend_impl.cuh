@@ -726,15 +726,15 @@ __device__ __forceinline__ void blend_walk_kpc(const DevCamera& cam, uint32_t ti
     }
 }
 
-// A CTA's share of the grid: the halves of the split tiles (heavy[], listed by the
-// sort) first, two CTAs for each of the split_slots there may be, then the n_tiles
+// CTA bid's share of a grid of n_ctas: the halves of the split tiles (heavy[], listed by
+// the sort) first, two CTAs for each of the split_slots there may be, then the n_tiles
 // tiles, those that are not split.
 template <class Whole, class Half>
-__device__ __forceinline__ void walk_grid(uint32_t n_tiles, const uint2* __restrict__ ranges,
+__device__ __forceinline__ void walk_grid(uint32_t bid, uint32_t n_ctas, uint32_t n_tiles, const uint2* __restrict__ ranges,
                                           const uint32_t* __restrict__ heavy, const FrameState* st, Whole whole,
                                           Half half)
 {
-    const uint32_t bid = blockIdx.x, n_half = gridDim.x - n_tiles;
+    const uint32_t n_half = n_ctas - n_tiles;
     if (bid < n_half) {
         if (bid >> 1 >= st->tickets[kTicketHeavy]) return;
         const uint32_t tile = heavy[bid >> 1];
