@@ -132,7 +132,8 @@ struct fgs_ctx {
         uint32_t *pbits = nullptr, *selbits = nullptr, *sel = nullptr;
         float* splat = nullptr;
         uint4* foot = nullptr;
-        unsigned long long *items = nullptr, *keys = nullptr, *lb_compact = nullptr, *lb_scan = nullptr;
+        unsigned long long *items = nullptr, *keys = nullptr, *lb_scan = nullptr;
+        uint32_t* sel_cnt = nullptr;              // selected entries per kBatchSelTileWords words
         uint32_t* vals = nullptr;
         uint2* ranges = nullptr;
         uint32_t *tile_cnt = nullptr, *large = nullptr, *heavy = nullptr;
@@ -476,7 +477,7 @@ int fgs_destroy(fgs_ctx* c)
     {
         auto& b = c->batch;
         void* bb[] = {b.d_cams, b.d_tile_base, b.d_img_off, b.pbits, b.selbits, b.sel, b.splat,
-                      b.foot, b.items, b.keys, b.vals, b.lb_compact, b.lb_scan, b.ranges, b.tile_cnt, b.large,
+                      b.foot, b.items, b.keys, b.vals, b.sel_cnt, b.lb_scan, b.ranges, b.tile_cnt, b.large,
                       b.heavy, b.st};
         for (void* p : bb) free_ptr(p);
         if (b.h_cams) cudaFreeHost(b.h_cams);
@@ -1235,7 +1236,7 @@ int fgs_batch_setup(fgs_ctx* c, const fgs_camera* views, int n_views, const int3
     if ((r = grow(c, (void**)&b.d_img_off, 8 * (n_views + 1)))) return r;
     if ((r = grow(c, (void**)&b.pbits, 4 * n_words * n_views))) return r;
     if ((r = grow(c, (void**)&b.selbits, 4 * n_words * n_views))) return r;
-    if ((r = grow(c, (void**)&b.lb_compact, 8 * (n_words * n_views / kCompactWords + 2)))) return r;
+    if ((r = grow(c, (void**)&b.sel_cnt, 4 * batch_sel_tiles(n_words * n_views)))) return r;
     if ((r = grow(c, (void**)&b.lb_scan, 8 * tile_scan_lookback_entries(b.total_tiles)))) return r;
     if (sel_cap != b.sel_cap) {
         if ((r = grow(c, (void**)&b.sel, 4 * sel_cap))) return r;
@@ -1293,7 +1294,7 @@ void enqueue_batch(fgs_ctx* c, float* rgb, float* T, cudaStream_t s)
     auto& b = c->batch;
     launch_batch_front(c->tree, b.d_cams, b.V, b.total_tiles, b.d_tile_base, b.pbits, b.selbits, b.sel,
                        (uint32_t)b.sel_cap, b.splat, b.foot, b.tile_cnt, b.large, b.heavy, b.items, b.keys, b.vals,
-                       b.pair_cap, b.lb_compact, b.lb_scan, b.ranges, b.st, c->sms, s);
+                       b.pair_cap, b.sel_cnt, b.lb_scan, b.ranges, b.st, c->sms, s);
     launch_batch_blend(b.d_cams, b.V, b.total_tiles, b.d_tile_base, b.d_img_off, b.ranges, b.heavy, b.vals, b.splat,
                        rgb, T, b.st, s);
 }
@@ -1314,7 +1315,7 @@ int fgs_render_batch(fgs_ctx* c, void* stream, float* rgb_out, float* T_out, uin
         b.h_cams[v] = d;
     }
     FGS_CUDA(c, cudaMemcpyAsync(b.d_cams, b.h_cams, sizeof(DevCamera) * b.V, cudaMemcpyHostToDevice, s));
-    const int launches = 9;
+    const int launches = 8;
     if (flags & FGS_BATCH_GRAPH) {
         if (!b.graph || b.graph_rgb != rgb_out || b.graph_T != T_out) {
             if (b.graph) {

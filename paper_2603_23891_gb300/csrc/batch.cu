@@ -3,11 +3,11 @@
 //
 // All views go through one sequence of kernels instead of one sequence per view:
 //  * bpred_kernel    R&L (§3.2) for every view: each node's centre and covariance
-//                    are read once and tested against all V cameras;
+//                    are read once and tested against the views that may see it;
 //  * banc_kernel     Ancestor filter per view: a node's ancestor path AP is read
 //                    once for all views in which the node passed R&L;
 //  * compaction      the per-view selection bits are one concatenated bit array
-//                    [V][words]; the render path's compaction kernel turns it into
+//                    [V][words]; the render path's counted compaction turns it into
 //                    global entries v * n_pad + node (ascending: view, then node);
 //  * bproject        projection and shrink of every entry with its view's camera;
 //                    pairs are counted into global tile ids (the view's first
@@ -25,148 +25,171 @@ namespace fgs {
 
 constexpr int kMaxBatchViews = 64;
 
-__global__ void bframe_begin_kernel(FrameState* st, uint32_t* tile_cnt, uint32_t n_tiles)
-{
-    const uint32_t tid = blockIdx.x * blockDim.x + threadIdx.x;
-    if (tid == 0) {
-        st->epoch = st->epoch + 1;
-        st->M = 0;
-        st->n_pairs = 0;
-    }
-    if (tid < 16) st->tickets[tid] = 0;
-    for (uint32_t i = tid; i < n_tiles; i += gridDim.x * blockDim.x) tile_cnt[i] = 0;
-}
-
-// R&L for V views: 4 consecutive nodes per thread, a warp a 128-node chunk,
-// cameras and their frustum planes in shared memory.  Lane v tests the chunk's
-// box against view v's frustum: the chunk's centres are read only if some view
-// may hold one of them, and evaluated only for those views (a chunk outside a
-// view's frustum has no node with P there: its P bits are written as 0); lane l
-// tests views l and l + 32.
+// R&L for V views: a warp takes chunks of 128 nodes g, g + W, g + 2W, ... (W warps), 32
+// at a time: lane l tests the box of the l-th against every view's frustum planes (in
+// shared memory, as the cameras); a chunk outside a view's frustum has no node with P
+// there and its P bits are written as 0; the others are read by the whole warp, 4 nodes
+// a lane, once for the views that need them, and evaluated for those.  The batch's
+// counters are zeroed here first.  Bound: the box tests' issue and the in-frustum chunks'
+// loads; a box tested by one lane a view, a chunk at a time, left most lanes idle and
+// a round trip a chunk (8 views of 12.5M nodes: 111 us).
 __global__ void __launch_bounds__(256) bpred_kernel(DevTree t, const DevCamera* __restrict__ cams,
-                                                    int V, uint32_t* __restrict__ pbits)
+                                                    int V, uint32_t* __restrict__ pbits, FrameBegin begin)
 {
     __shared__ DevCamera s_cam[kMaxBatchViews];
     __shared__ FrustumPlanes s_planes[kMaxBatchViews];
+    grid_dep_wait();
+    frame_begin(begin, (int)(blockIdx.x * blockDim.x + threadIdx.x), (int)(gridDim.x * blockDim.x));
     for (int i = threadIdx.x; i < V * (int)(sizeof(DevCamera) / 4); i += blockDim.x)
         reinterpret_cast<uint32_t*>(s_cam)[i] = reinterpret_cast<const uint32_t*>(cams)[i];
     __syncthreads();
     if ((int)threadIdx.x < V) frustum_planes(s_cam[threadIdx.x], s_planes[threadIdx.x]);
     __syncthreads();
-    const uint32_t n_chunks = t.n_pad >> 2;
-    const uint32_t n_words = t.n_pad >> 5;
+    static_assert(kMaxBatchViews <= 64, "a view a bit of a 64-bit mask");
+    const uint32_t n_words = t.n_pad >> 5, n_box = t.n_pad >> 7;
     const uint32_t lane = threadIdx.x & 31;
-    const uint32_t stride = gridDim.x * blockDim.x;       // a multiple of 32: warps keep 128-node chunks
-    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n_chunks; i += stride) {
-        const uint32_t n0 = i << 2;
-        const uint32_t c = i >> 5;
-        const float4 lo = __ldg(t.cbox + 2 * c), hi = __ldg(t.cbox + 2 * c + 1);
-        static_assert(kMaxBatchViews <= 64, "two ballots of views");
-        const unsigned long long vmask =
-            (unsigned long long)__ballot_sync(0xffffffffu, (int)lane < V && !chunk_outside(s_planes[lane], lo, hi)) |
-            ((unsigned long long)__ballot_sync(0xffffffffu, (int)lane + 32 < V &&
-                                                                !chunk_outside(s_planes[lane + 32 < kMaxBatchViews ? lane + 32 : 0], lo, hi))
-             << 32);
-        if (vmask == 0ull) {
-            for (int v = 0; v < V; ++v)
-                if ((lane & 7) == 0) pbits[(size_t)v * n_words + (i >> 3)] = 0u;
-            continue;
+    const uint32_t n_warps = (gridDim.x * blockDim.x) >> 5;
+    for (uint32_t cb = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; cb < n_box; cb += 32u * n_warps) {
+        const uint32_t cl = cb + lane * n_warps;
+        unsigned long long views = 0ull;                  // that may hold a centre of this lane's chunk
+        if (cl < n_box) {
+            const float4 lo = __ldg(t.cbox + 2 * cl), hi = __ldg(t.cbox + 2 * cl + 1);
+            for (int v = 0; v < V; ++v) {
+                if (chunk_outside(s_planes[v], lo, hi))
+                    reinterpret_cast<uint4*>(pbits + (size_t)v * n_words)[cl] = make_uint4(0u, 0u, 0u, 0u);
+                else
+                    views |= 1ull << v;
+            }
         }
-        const float4 mx = __ldg(reinterpret_cast<const float4*>(t.mu) + i);
-        const float4 my = __ldg(reinterpret_cast<const float4*>(t.mu + t.n_pad) + i);
-        const float4 mz = __ldg(reinterpret_cast<const float4*>(t.mu + 2 * (size_t)t.n_pad) + i);
-        const uint32_t leaf = (__ldg(t.leaf_bits + (i >> 3)) >> ((i & 7) << 2)) & 0xFu;
-        const float xs[4] = {mx.x, mx.y, mx.z, mx.w};
-        const float ys[4] = {my.x, my.y, my.z, my.w};
-        const float zs[4] = {mz.x, mz.y, mz.z, mz.w};
-        float4 cv[6];
-        bool have_cov = false;
-        for (int v = 0; v < V; ++v) {
-            if (!((vmask >> v) & 1ull)) {
-                if ((lane & 7) == 0) pbits[(size_t)v * n_words + (i >> 3)] = 0u;
-                continue;
+        uint32_t todo = __ballot_sync(0xffffffffu, views != 0ull);
+        while (todo) {
+            const uint32_t j = (uint32_t)__ffs(todo) - 1u;
+            todo &= todo - 1u;
+            if (todo) {
+                const uint32_t cn = cb + ((uint32_t)__ffs(todo) - 1u) * n_warps;
+                const float* nx = t.mu + ((size_t)cn << 7) + (lane << 2);
+                asm volatile("prefetch.global.L2 [%0];" ::"l"(nx));
+                asm volatile("prefetch.global.L2 [%0];" ::"l"(nx + t.n_pad));
+                asm volatile("prefetch.global.L2 [%0];" ::"l"(nx + 2 * (size_t)t.n_pad));
             }
-            const DevCamera& cam = s_cam[v];
-            float vz[4], txtz[4], tytz[4];
-            uint32_t inf = 0;
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                float vx, vy;
-                camera_space(cam, xs[k], ys[k], zs[k], vx, vy, vz[k]);
-                txtz[k] = tytz[k] = 0.0f;
-                const bool in = (n0 + k < t.n) && frustum_test(cam, vx, vy, vz[k], txtz[k], tytz[k]);
-                inf |= (uint32_t)in << k;
-            }
-            uint32_t pnib = inf & leaf;
-            const uint32_t need = inf & ~leaf;
-            if (need) {
-                if (!have_cov) {
-#pragma unroll
-                    for (int q = 0; q < 6; ++q)
-                        cv[q] = __ldg(reinterpret_cast<const float4*>(t.cov + q * (size_t)t.n_pad) + i);
-                    have_cov = true;
-                }
+            unsigned long long vm = ((unsigned long long)__shfl_sync(0xffffffffu, (uint32_t)(views >> 32), j) << 32) |
+                                    __shfl_sync(0xffffffffu, (uint32_t)views, j);
+            const uint32_t i = ((cb + j * n_warps) << 5) + lane;   // this lane's 4 nodes
+            const uint32_t n0 = i << 2;
+            const float4 mx = __ldg(reinterpret_cast<const float4*>(t.mu) + i);
+            const float4 my = __ldg(reinterpret_cast<const float4*>(t.mu + t.n_pad) + i);
+            const float4 mz = __ldg(reinterpret_cast<const float4*>(t.mu + 2 * (size_t)t.n_pad) + i);
+            const uint32_t leaf = (__ldg(t.leaf_bits + (i >> 3)) >> ((i & 7) << 2)) & 0xFu;
+            const float xs[4] = {mx.x, mx.y, mx.z, mx.w};
+            const float ys[4] = {my.x, my.y, my.z, my.w};
+            const float zs[4] = {mz.x, mz.y, mz.z, mz.w};
+            float4 cv[6];
+            bool have_cov = false;
+            while (vm) {
+                const int v = __ffsll((long long)vm) - 1;
+                vm &= vm - 1ull;
+                const DevCamera& cam = s_cam[v];
+                float vz[4], txtz[4], tytz[4];
+                uint32_t inf = 0;
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
-                    if (!((need >> k) & 1u)) continue;
-                    float s6[6];
-#pragma unroll
-                    for (int q = 0; q < 6; ++q)
-                        s6[q] = k == 0 ? cv[q].x : k == 1 ? cv[q].y : k == 2 ? cv[q].z : cv[q].w;
-                    float a, b, cc, lam;
-                    ewa_cov2d(cam, vz[k], txtz[k], tytz[k], s6, a, b, cc, lam);
-                    if (fm(3.0f, fsq(lam)) <= cam.tau_R) pnib |= 1u << k;
+                    float vx, vy;
+                    camera_space(cam, xs[k], ys[k], zs[k], vx, vy, vz[k]);
+                    txtz[k] = tytz[k] = 0.0f;
+                    const bool in = (n0 + k < t.n) && frustum_test(cam, vx, vy, vz[k], txtz[k], tytz[k]);
+                    inf |= (uint32_t)in << k;
                 }
+                uint32_t pnib = inf & leaf;
+                const uint32_t need = inf & ~leaf;
+                if (need) {
+                    if (!have_cov) {
+#pragma unroll
+                        for (int q = 0; q < 6; ++q)
+                            cv[q] = __ldg(reinterpret_cast<const float4*>(t.cov + q * (size_t)t.n_pad) + i);
+                        have_cov = true;
+                    }
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        if (!((need >> k) & 1u)) continue;
+                        float s6[6];
+#pragma unroll
+                        for (int q = 0; q < 6; ++q)
+                            s6[q] = k == 0 ? cv[q].x : k == 1 ? cv[q].y : k == 2 ? cv[q].z : cv[q].w;
+                        float a, b, cc, lam;
+                        ewa_cov2d(cam, vz[k], txtz[k], tytz[k], s6, a, b, cc, lam);
+                        if (fm(3.0f, fsq(lam)) <= cam.tau_R) pnib |= 1u << k;
+                    }
+                }
+                uint32_t w = pnib << ((lane & 7) << 2);
+                w |= __shfl_xor_sync(0xffffffffu, w, 1);
+                w |= __shfl_xor_sync(0xffffffffu, w, 2);
+                w |= __shfl_xor_sync(0xffffffffu, w, 4);
+                if ((lane & 7) == 0) pbits[(size_t)v * n_words + (i >> 3)] = w;
             }
-            uint32_t w = pnib << ((lane & 7) << 2);
-            w |= __shfl_xor_sync(0xffffffffu, w, 1);
-            w |= __shfl_xor_sync(0xffffffffu, w, 2);
-            w |= __shfl_xor_sync(0xffffffffu, w, 4);
-            if ((lane & 7) == 0) pbits[(size_t)v * n_words + (i >> 3)] = w;
         }
     }
 }
 
-// Ancestor filter for V views: the path is read once per node, then checked
-// against the P bits of every view in which the node passed.
+// Ancestor filter for V views, a warp 8 words of 32 nodes at a time: lane l reads word
+// l % 8 of views l / 8, l / 8 + 4, ..., so the words without a P bit in any view (most)
+// cost a few loads and stores for all 8 together.  For the others the path of each node
+// is read once for all views, and in each view with a P bit in the word the ancestors'
+// bits in one batch of independent loads.  The survivors of every compaction tile are
+// counted.  Bound: latency; a word at a time over every view, with an ancestor's bit
+// looked up before the next, took 238 us for 8 views of 12.5M nodes.
 __global__ void __launch_bounds__(256) banc_kernel(DevTree t, int V, const uint32_t* __restrict__ pbits,
-                                                   uint32_t* __restrict__ selbits)
+                                                   uint32_t* __restrict__ selbits, uint32_t* __restrict__ sel_cnt)
 {
+    grid_dep_wait();
     const uint32_t lane = threadIdx.x & 31;
-    const uint32_t n_words = t.n_pad >> 5;
+    const uint32_t n_words = t.n_pad >> 5;                // a multiple of 128
     const uint32_t n_warps = (gridDim.x * blockDim.x) >> 5;
-    for (uint32_t w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < n_words; w += n_warps) {
-        const uint32_t n = (w << 5) + lane;
-        uint64_t mine = 0;                        // bit v: P in view v
-        for (int v = 0; v < V; ++v)
-            if ((__ldg(pbits + (size_t)v * n_words + w) >> lane) & 1u) mine |= 1ull << v;
-        if (n >= t.n) mine = 0;
-        uint64_t keep = mine;
-        if (mine) {
+    for (uint32_t w0 = 8u * ((blockIdx.x * blockDim.x + threadIdx.x) >> 5); w0 < n_words; w0 += 8u * n_warps) {
+        const uint32_t wl = w0 + (lane & 7u);
+        uint32_t any = 0u;
+        for (int v = (int)(lane >> 3); v < V; v += 4) any |= __ldg(pbits + (size_t)v * n_words + wl);
+        any = __ballot_sync(0xffffffffu, any != 0u);
+        uint32_t act = (any | any >> 8 | any >> 16 | any >> 24) & 0xFFu;
+        if (!((act >> (lane & 7u)) & 1u))
+            for (int v = (int)(lane >> 3); v < V; v += 4) selbits[(size_t)v * n_words + wl] = 0u;
+        while (act) {
+            const uint32_t k = (uint32_t)__ffs(act) - 1u;
+            act &= act - 1u;
+            const uint32_t w = w0 + k;
+            const uint32_t n = (w << 5) + lane;
+            uint64_t mine = 0;                            // bit v: P in view v
+#pragma unroll 4
+            for (int v = 0; v < V; ++v)
+                mine |= (uint64_t)((__ldg(pbits + (size_t)v * n_words + w) >> lane) & 1u) << v;
+            if (n >= t.n) mine = 0;
             uint32_t a[16];
-            for (uint32_t k0 = 0; k0 < t.depth && keep; k0 += 16) {
 #pragma unroll
-                for (int q = 0; q < 16; ++q)
-                    a[q] = (k0 + q < t.depth) ? __ldg(t.ap + (size_t)(k0 + q) * t.n_pad + n) : kApPad;
-                uint64_t left = keep;
-                while (left) {
-                    const int v = __ffsll((long long)left) - 1;
-                    left &= left - 1;
+            for (int q = 0; q < 16; ++q)
+                a[q] = mine && (uint32_t)q < t.depth ? __ldg(t.ap + (size_t)q * t.n_pad + n) : kApPad;
+            for (int v = 0; v < V; ++v) {
+                bool keep = (mine >> v) & 1ull;
+                uint32_t b = 0u;
+                if (__any_sync(0xffffffffu, keep)) {
                     const uint32_t* pv = pbits + (size_t)v * n_words;
-                    bool blocked = false;
+                    uint32_t hit = 0u;
 #pragma unroll
-                    for (int q = 0; q < 16; ++q) {
-                        if (a[q] == kApPad) break;
-                        if ((__ldg(pv + (a[q] >> 5)) >> (a[q] & 31)) & 1u) { blocked = true; break; }
+                    for (int q = 0; q < 16; ++q)
+                        if (keep && a[q] != kApPad) hit |= __ldg(pv + (a[q] >> 5)) >> (a[q] & 31) & 1u;
+                    if (hit) keep = false;
+                    // levels above the 16th (a tree so deep): one at a time
+                    for (uint32_t q = 16; keep && q < t.depth; ++q) {
+                        const uint32_t an = __ldg(t.ap + (size_t)q * t.n_pad + n);
+                        if (an == kApPad) break;
+                        if (__ldg(pv + (an >> 5)) >> (an & 31) & 1u) keep = false;
                     }
-                    if (blocked) keep &= ~(1ull << v);
+                    b = __ballot_sync(0xffffffffu, keep);
                 }
-                if (a[15] == kApPad) break;
+                if (lane == 0) {
+                    const size_t at = (size_t)v * n_words + w;
+                    selbits[at] = b;
+                    if (b) atomicAdd(sel_cnt + at / kBatchSelTileWords, (uint32_t)__popc(b));
+                }
             }
-        }
-        for (int v = 0; v < V; ++v) {
-            const uint32_t b = __ballot_sync(0xffffffffu, (keep >> v) & 1ull);
-            if (lane == (uint32_t)(v & 31)) selbits[(size_t)v * n_words + w] = b;
         }
     }
 }
@@ -180,6 +203,7 @@ __global__ void __launch_bounds__(kProjThreads) bproject_kernel(
 {
     __shared__ DevCamera s_cam[kMaxBatchViews];
     __shared__ uint32_t s_base[kMaxBatchViews];
+    grid_dep_wait();
     for (int i = threadIdx.x; i < V * (int)(sizeof(DevCamera) / 4); i += blockDim.x)
         reinterpret_cast<uint32_t*>(s_cam)[i] = reinterpret_cast<const uint32_t*>(cams)[i];
     for (int i = threadIdx.x; i < V; i += blockDim.x) s_base[i] = tile_base[i];
@@ -210,6 +234,7 @@ __global__ void __launch_bounds__(blendk::kWalkChunk) bblend_kernel(
 {
     __shared__ __align__(128) blendk::WalkSmem<false> S;
     __shared__ DevCamera s_cam;
+    grid_dep_wait();
     // the tile's view: its camera to s_cam; first tile and image offset
     auto locate = [&](uint32_t gtile, uint32_t& base) {
         int lo = 0, hi = V;                            // largest v with tile_base[v] <= gtile
@@ -247,22 +272,21 @@ void launch_batch_front(const DevTree& t, const DevCamera* cams, int V, uint32_t
                         const uint32_t* tile_base, uint32_t* pbits, uint32_t* selbits, uint32_t* sel,
                         uint32_t sel_cap, float* splat, uint4* foot, uint32_t* tile_cnt, uint32_t* large, uint32_t* heavy,
                         unsigned long long* items, unsigned long long* keys, uint32_t* vals,
-                        unsigned long long cap, unsigned long long* lb_compact, unsigned long long* lb_scan,
+                        unsigned long long cap, uint32_t* sel_cnt, unsigned long long* lb_scan,
                         uint2* ranges, FrameState* st, int sms, cudaStream_t s)
 {
     const uint32_t n_words = t.n_pad >> 5;
-    int b0 = (int)((total_tiles + 255) / 256);
-    bframe_begin_kernel<<<b0 < 8 ? 8 : b0, 256, 0, s>>>(st, tile_cnt, total_tiles);
+    const uint32_t all_words = (uint32_t)((size_t)n_words * V);
+    const FrameBegin begin{st, tile_cnt, (int)total_tiles, sel_cnt, (int)batch_sel_tiles(all_words)};
     int occ = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, bpred_kernel, 256, 0);
-    bpred_kernel<<<sms * (occ > 0 ? occ : 1), 256, 0, s>>>(t, cams, V, pbits);
+    launch_pdl(bpred_kernel, sms * (occ > 0 ? occ : 1), 256, 0, s, t, cams, V, pbits, begin);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, banc_kernel, 256, 0);
-    banc_kernel<<<sms * (occ > 0 ? occ : 1), 256, 0, s>>>(t, V, pbits, selbits);
-    launch_compact(selbits, (uint32_t)((size_t)n_words * V), sel, sel_cap, lb_compact, st,
-                   sms * occ_compact(), s);
+    launch_pdl(banc_kernel, sms * (occ > 0 ? occ : 1), 256, 0, s, t, V, pbits, selbits, sel_cnt);
+    launch_compact_counted_batch(selbits, all_words, sel, sel_cap, sel_cnt, st, s);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, bproject_kernel, kProjThreads, 0);
-    bproject_kernel<<<sms * (occ > 0 ? occ : 1), kProjThreads, 0, s>>>(t, cams, V, tile_base, sel, splat,
-                                                                       foot, tile_cnt, st);
+    launch_pdl(bproject_kernel, sms * (occ > 0 ? occ : 1), kProjThreads, 0, s, t, cams, V, tile_base, sel, splat, foot,
+               tile_cnt, st);
     launch_tile_scan(tile_cnt, ranges, total_tiles, large, cap, lb_scan, st, sms * occ_tile_scan(), s);
     launch_scatter_batch(cams, tile_base, t.n_pad, sel, foot, tile_cnt, items, cap, st, sms * occ_scatter(), s);
     launch_segsort(ranges, total_tiles, large, items, keys, vals, heavy, st, sms * occ_segsort(), s);
@@ -274,8 +298,8 @@ void launch_batch_blend(const DevCamera* cams, int V, uint32_t total_tiles, cons
                         cudaStream_t s)
 {
     const uint32_t grid = total_tiles + 2u * (uint32_t)split_slots((int)total_tiles);
-    bblend_kernel<<<grid, blendk::kWalkChunk, 0, s>>>(cams, V, total_tiles, tile_base, img_off, ranges, heavy, vals,
-                                                      splat, rgb, T, st);
+    launch_pdl(bblend_kernel, grid, blendk::kWalkChunk, 0, s, cams, V, total_tiles, tile_base, img_off, ranges, heavy,
+               vals, splat, rgb, T, st);
 }
 
 }  // namespace fgs

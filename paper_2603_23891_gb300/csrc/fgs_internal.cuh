@@ -23,6 +23,8 @@ constexpr int kSegSmem = 2048;            // pairs of a tile sorted by one block
 constexpr int kFilterTile = 4096;         // node arrays are padded to a multiple of this
 constexpr int kCompactWords = 1024;       // 32-bit selection words per compaction tile (32K nodes)
 constexpr int kSelTileWords = 256;        // words per counted tile (the Ancestor filter's sel_cnt)
+constexpr int kBatchSelTileWords = 1024;  // the same in the batched form
+inline size_t batch_sel_tiles(size_t words) { return (words + kBatchSelTileWords - 1) / kBatchSelTileWords; }
 constexpr int kAncCacheWords = 4096;      // P-bit words of the lowest node ids kept in shared memory
 constexpr uint32_t kSplitTiles = 912;      // fewer tiles than that of a blend are split (6 an SM)
 constexpr int kProjThreads = 256;         // selected Gaussians per projection tile
@@ -403,6 +405,38 @@ __device__ __forceinline__ uint32_t warp_lookback(const unsigned long long* lb, 
     return prefix;
 }
 
+// The frame's counters to be zeroed: FrameState, the per-tile pair counts tile_cnt and
+// the per-compaction-tile selection counts sel_cnt.
+struct FrameBegin {
+    FrameState* st;
+    uint32_t* tile_cnt;
+    int n_tiles;
+    uint32_t* sel_cnt;
+    int n_sel_tiles;
+};
+
+// The frame's counters to zero (n_threads threads, this one's index tid).
+__device__ __forceinline__ void frame_begin(const FrameBegin& f, int tid, int n_threads)
+{
+    FrameState* st = f.st;
+    if (tid == 0) {
+        st->epoch = st->epoch + 1;
+        st->M = 0;
+        st->n_pairs = 0;
+        st->blend_entries = 0;
+        st->blend_evals = 0;
+        st->blend_hits = 0;
+        st->blend_active = 0;
+        st->n_emitting = 0;
+        st->filter_in_frustum = 0;
+        st->filter_cov_nodes = 0;
+        st->filter_chunks = 0;
+    }
+    if (tid < 16) st->tickets[tid] = 0;
+    for (int i = tid; i < f.n_tiles; i += n_threads) f.tile_cnt[i] = 0;
+    for (int i = tid; i < f.n_sel_tiles; i += n_threads) f.sel_cnt[i] = 0;
+}
+
 // ---------------------------------------------------------------------
 // host launchers (one per kernel family)
 // ---------------------------------------------------------------------
@@ -434,15 +468,6 @@ int occ_segsort();
 
 // All launchers enqueue on `s` and read counts (M, N_P) from device memory,
 // so a frame needs no host synchronisation.
-// The frame's counters to be zeroed: FrameState, the per-tile pair counts tile_cnt and
-// the per-compaction-tile selection counts sel_cnt.
-struct FrameBegin {
-    FrameState* st;
-    uint32_t* tile_cnt;
-    int n_tiles;
-    uint32_t* sel_cnt;
-    int n_sel_tiles;
-};
 void launch_frame_begin(const FrameBegin& f, cudaStream_t s);
 // begin.st null: the counters are not zeroed (launch_frame_begin has done it).
 void launch_filter_pred(const DevTree& t, const DevCamera& cam, uint32_t* pbits, FrameState* count_st,
@@ -464,6 +489,9 @@ void launch_compact(const uint32_t* selbits, uint32_t n_words, uint32_t* sel, ui
 // The same result from the Ancestor filter's per-tile counts (one block a tile).
 void launch_compact_counted(const uint32_t* selbits, uint32_t n_words, uint32_t* sel, uint32_t cap,
                             const uint32_t* sel_cnt, FrameState* st, cudaStream_t s);
+// The same for a batch: sel_cnt per kBatchSelTileWords words.
+void launch_compact_counted_batch(const uint32_t* selbits, uint32_t n_words, uint32_t* sel, uint32_t cap,
+                                  const uint32_t* sel_cnt, FrameState* st, cudaStream_t s);
 // Projection (splat records, footprints) and the per-tile pair counts
 // tile_cnt[tiles] (zeroed by launch_frame_begin).
 void launch_project(const DevTree& t, const DevCamera& cam, const uint32_t* sel, float* splat,
@@ -505,7 +533,7 @@ void launch_batch_front(const DevTree& t, const DevCamera* cams, int V, uint32_t
                         const uint32_t* tile_base, uint32_t* pbits, uint32_t* selbits, uint32_t* sel,
                         uint32_t sel_cap, float* splat, uint4* foot, uint32_t* tile_cnt, uint32_t* large, uint32_t* heavy,
                         unsigned long long* items, unsigned long long* keys, uint32_t* vals,
-                        unsigned long long cap, unsigned long long* lb_compact, unsigned long long* lb_scan, uint2* ranges,
+                        unsigned long long cap, uint32_t* sel_cnt, unsigned long long* lb_scan, uint2* ranges,
                         FrameState* st, int sms, cudaStream_t s);
 void launch_batch_blend(const DevCamera* cams, int V, uint32_t total_tiles, const uint32_t* tile_base,
                         const unsigned long long* img_off, const uint2* ranges, const uint32_t* heavy,
