@@ -32,8 +32,8 @@ constexpr int kMaxBatchViews = 64;
 // a lane, once for the views that need them, and evaluated for those.  The batch's
 // counters are zeroed here first.  Bound: the box tests' issue and the in-frustum chunks'
 // loads; a box tested by one lane a view, a chunk at a time, left most lanes idle and
-// a round trip a chunk (8 views of 12.5M nodes: 111 us).
-__global__ void __launch_bounds__(256) bpred_kernel(DevTree t, const DevCamera* __restrict__ cams,
+// a round trip a chunk (8 views of 12.5M nodes: 111 us, now 70).
+__global__ void __launch_bounds__(256, 3) bpred_kernel(DevTree t, const DevCamera* __restrict__ cams,
                                                     int V, uint32_t* __restrict__ pbits, FrameBegin begin)
 {
     __shared__ DevCamera s_cam[kMaxBatchViews];
@@ -130,64 +130,88 @@ __global__ void __launch_bounds__(256) bpred_kernel(DevTree t, const DevCamera* 
     }
 }
 
-// Ancestor filter for V views, a warp 8 words of 32 nodes at a time: lane l reads word
-// l % 8 of views l / 8, l / 8 + 4, ..., so the words without a P bit in any view (most)
-// cost a few loads and stores for all 8 together.  For the others the path of each node
-// is read once for all views, and in each view with a P bit in the word the ancestors'
-// bits in one batch of independent loads.  The survivors of every compaction tile are
-// counted.  Bound: latency; a word at a time over every view, with an ancestor's bit
-// looked up before the next, took 238 us for 8 views of 12.5M nodes.
-__global__ void __launch_bounds__(256) banc_kernel(DevTree t, int V, const uint32_t* __restrict__ pbits,
-                                                   uint32_t* __restrict__ selbits, uint32_t* __restrict__ sel_cnt)
+// Ancestor filter for V views, a warp 4 words of 32 nodes at a time: lane l reads word
+// l % 4 of views l / 4, l / 4 + 8, ..., so the words without a P bit in any view (most)
+// cost a few loads and stores for all 4 together.  For the others the path of each node
+// is read once for all views (and the next such word's paths are prefetched), and the
+// ancestors' bits of two views that have a P bit in the word in one batch of independent
+// loads.  The survivors of every compaction tile are counted.  Bound: latency; a word at
+// a time over every view, an ancestor's bit looked up before the next, took 238 us for 8
+// views of 12.5M nodes; one view a turn 214, two 157, 4 words instead of 8 at a time 133.
+__global__ void __launch_bounds__(256, 5) banc_kernel(DevTree t, int V, const uint32_t* __restrict__ pbits,
+                                                      uint32_t* __restrict__ selbits, uint32_t* __restrict__ sel_cnt)
 {
     grid_dep_wait();
     const uint32_t lane = threadIdx.x & 31;
     const uint32_t n_words = t.n_pad >> 5;                // a multiple of 128
     const uint32_t n_warps = (gridDim.x * blockDim.x) >> 5;
-    for (uint32_t w0 = 8u * ((blockIdx.x * blockDim.x + threadIdx.x) >> 5); w0 < n_words; w0 += 8u * n_warps) {
-        const uint32_t wl = w0 + (lane & 7u);
+    for (uint32_t w0 = 4u * ((blockIdx.x * blockDim.x + threadIdx.x) >> 5); w0 < n_words; w0 += 4u * n_warps) {
+        const uint32_t wl = w0 + (lane & 3u);
         uint32_t any = 0u;
-        for (int v = (int)(lane >> 3); v < V; v += 4) any |= __ldg(pbits + (size_t)v * n_words + wl);
+        for (int v = (int)(lane >> 2); v < V; v += 8) any |= __ldg(pbits + (size_t)v * n_words + wl);
         any = __ballot_sync(0xffffffffu, any != 0u);
-        uint32_t act = (any | any >> 8 | any >> 16 | any >> 24) & 0xFFu;
-        if (!((act >> (lane & 7u)) & 1u))
-            for (int v = (int)(lane >> 3); v < V; v += 4) selbits[(size_t)v * n_words + wl] = 0u;
+        any |= any >> 16;
+        any |= any >> 8;
+        uint32_t act = (any | any >> 4) & 0xFu;
+        if (!((act >> (lane & 3u)) & 1u))
+            for (int v = (int)(lane >> 2); v < V; v += 8) selbits[(size_t)v * n_words + wl] = 0u;
         while (act) {
             const uint32_t k = (uint32_t)__ffs(act) - 1u;
             act &= act - 1u;
             const uint32_t w = w0 + k;
             const uint32_t n = (w << 5) + lane;
-            uint64_t mine = 0;                            // bit v: P in view v
-#pragma unroll 4
-            for (int v = 0; v < V; ++v)
-                mine |= (uint64_t)((__ldg(pbits + (size_t)v * n_words + w) >> lane) & 1u) << v;
-            if (n >= t.n) mine = 0;
-            uint32_t a[16];
+            if (act && lane < t.depth)                    // the next word's paths
+                asm volatile("prefetch.global.L2 [%0];" ::"l"(t.ap + (size_t)lane * t.n_pad +
+                                                              ((size_t)(w0 + (uint32_t)__ffs(act) - 1u) << 5)));
+            for (int vb = 0; vb < V; vb += 32) {          // 32 views at a time, lane l reads the word of view vb + l
+                const uint32_t pw = vb + (int)lane < V ? __ldg(pbits + (size_t)(vb + lane) * n_words + w) : 0u;
+                uint32_t vm = __ballot_sync(0xffffffffu, pw != 0u);
+                if (vb + (int)lane < V && !pw) selbits[(size_t)(vb + lane) * n_words + w] = 0u;
+                if (!vm) continue;
+                uint32_t nodes = pw;                      // with a P bit in any of these views
 #pragma unroll
-            for (int q = 0; q < 16; ++q)
-                a[q] = mine && (uint32_t)q < t.depth ? __ldg(t.ap + (size_t)q * t.n_pad + n) : kApPad;
-            for (int v = 0; v < V; ++v) {
-                bool keep = (mine >> v) & 1ull;
-                uint32_t b = 0u;
-                if (__any_sync(0xffffffffu, keep)) {
-                    const uint32_t* pv = pbits + (size_t)v * n_words;
-                    uint32_t hit = 0u;
+                for (int o = 16; o; o >>= 1) nodes |= __shfl_xor_sync(0xffffffffu, nodes, o);
+                const bool mine = (nodes >> lane) & 1u;
+                uint32_t a[16];
 #pragma unroll
-                    for (int q = 0; q < 16; ++q)
-                        if (keep && a[q] != kApPad) hit |= __ldg(pv + (a[q] >> 5)) >> (a[q] & 31) & 1u;
-                    if (hit) keep = false;
+                for (int q = 0; q < 16; ++q)
+                    a[q] = mine && (uint32_t)q < t.depth ? __ldg(t.ap + (size_t)q * t.n_pad + n) : kApPad;
+                while (vm) {                              // two views at a time
+                    const uint32_t v0 = (uint32_t)__ffs(vm) - 1u;
+                    vm &= vm - 1u;
+                    const uint32_t v1 = vm ? (uint32_t)__ffs(vm) - 1u : v0;
+                    vm &= vm - 1u;
+                    const uint32_t* p0 = pbits + (size_t)(vb + v0) * n_words;
+                    const uint32_t* p1 = pbits + (size_t)(vb + v1) * n_words;
+                    bool k0 = (__shfl_sync(0xffffffffu, pw, v0) >> lane) & 1u;
+                    bool k1 = (__shfl_sync(0xffffffffu, pw, v1) >> lane) & 1u;
+                    uint32_t h0 = 0u, h1 = 0u;
+#pragma unroll
+                    for (int h = 0; h < 16; h += 8) {
+                        if (h && t.depth <= 8u) break;
+#pragma unroll
+                        for (int q = h; q < h + 8; ++q)
+                            if (a[q] != kApPad) {
+                                if (k0) h0 |= __ldg(p0 + (a[q] >> 5)) >> (a[q] & 31);
+                                if (k1) h1 |= __ldg(p1 + (a[q] >> 5)) >> (a[q] & 31);
+                            }
+                    }
+                    k0 = k0 && !(h0 & 1u);
+                    k1 = k1 && !(h1 & 1u);
                     // levels above the 16th (a tree so deep): one at a time
-                    for (uint32_t q = 16; keep && q < t.depth; ++q) {
+                    for (uint32_t q = 16; (k0 || k1) && q < t.depth; ++q) {
                         const uint32_t an = __ldg(t.ap + (size_t)q * t.n_pad + n);
                         if (an == kApPad) break;
-                        if (__ldg(pv + (an >> 5)) >> (an & 31) & 1u) keep = false;
+                        if (__ldg(p0 + (an >> 5)) >> (an & 31) & 1u) k0 = false;
+                        if (__ldg(p1 + (an >> 5)) >> (an & 31) & 1u) k1 = false;
                     }
-                    b = __ballot_sync(0xffffffffu, keep);
-                }
-                if (lane == 0) {
-                    const size_t at = (size_t)v * n_words + w;
-                    selbits[at] = b;
-                    if (b) atomicAdd(sel_cnt + at / kBatchSelTileWords, (uint32_t)__popc(b));
+                    const uint32_t b0 = __ballot_sync(0xffffffffu, k0), b1 = __ballot_sync(0xffffffffu, k1);
+                    if (lane < 2u && (lane == 0u || v1 != v0)) {
+                        const uint32_t b = lane ? b1 : b0;
+                        const size_t at = (size_t)(vb + (lane ? v1 : v0)) * n_words + w;
+                        selbits[at] = b;
+                        if (b) atomicAdd(sel_cnt + at / kBatchSelTileWords, (uint32_t)__popc(b));
+                    }
                 }
             }
         }
