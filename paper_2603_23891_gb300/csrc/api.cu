@@ -45,7 +45,7 @@ struct fgs_ctx {
     std::string err;
     fgs_params params{};
     // occupancy (resident blocks per SM)
-    int occ_pred = 1, occ_anc = 1, occ_compact = 1, occ_proj = 1, occ_scatter = 1, occ_segsort = 1, occ_scan = 1;
+    int occ_pred = 1, occ_anc = 1, occ_compact = 1, occ_scatter = 1, occ_segsort = 1, occ_scan = 1;
     // tree
     bool has_tree = false;
     DevTree tree{};
@@ -367,7 +367,7 @@ int enqueue_front(fgs_ctx* c, const DevCamera& dc, cudaStream_t s, cudaEvent_t* 
     launch_filter_anc(c->tree, c->pbits, c->selbits, c->sel_cnt, c->sms * c->occ_anc, s);
     launch_compact_counted(c->selbits, c->tree.n_pad / 32, c->sel, c->tree.n_pad, c->sel_cnt, c->st, s);
     if (ev) cudaEventRecord(ev[2], s);
-    launch_project(c->tree, dc, c->sel, c->splat, c->foot, c->tile_cnt, c->st, c->sms * c->occ_proj, s);
+    launch_project(c->tree, dc, c->sel, c->splat, c->foot, c->tile_cnt, c->st, c->sms, s);
     if (ev) cudaEventRecord(ev[3], s);
     launch_tile_scan(c->tile_cnt, c->ranges, tiles, c->large, c->pair_cap, c->lb_scan, c->st, c->sms * c->occ_scan,
                      s);
@@ -432,7 +432,6 @@ int fgs_create(fgs_ctx** out, int device)
     c->occ_pred = occ_filter_pred();
     c->occ_anc = occ_filter_anc();
     c->occ_compact = occ_compact();
-    c->occ_proj = occ_project();
     c->occ_scatter = occ_scatter();
     c->occ_segsort = occ_segsort();
     c->occ_scan = occ_tile_scan();

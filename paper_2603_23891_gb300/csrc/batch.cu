@@ -220,11 +220,13 @@ __global__ void __launch_bounds__(256, 5) banc_kernel(DevTree t, int V, const ui
 
 // Projection of every selected entry (entry = view * n_pad + node), with the
 // pairs counted into global tile ids.
-__global__ void __launch_bounds__(kProjThreads) bproject_kernel(
+template <int kDeg>
+__global__ void __launch_bounds__(kProjectThreads, kProjectBlocks) bproject_kernel(
     DevTree t, const DevCamera* __restrict__ cams, int V, const uint32_t* __restrict__ tile_base,
     const uint32_t* __restrict__ sel, float* __restrict__ splat, uint4* __restrict__ foot,
     uint32_t* __restrict__ tile_cnt, FrameState* st)
 {
+    __shared__ proj::Rows<kDeg> S;
     __shared__ DevCamera s_cam[kMaxBatchViews];
     __shared__ uint32_t s_base[kMaxBatchViews];
     grid_dep_wait();
@@ -232,21 +234,14 @@ __global__ void __launch_bounds__(kProjThreads) bproject_kernel(
         reinterpret_cast<uint32_t*>(s_cam)[i] = reinterpret_cast<const uint32_t*>(cams)[i];
     for (int i = threadIdx.x; i < V; i += blockDim.x) s_base[i] = tile_base[i];
     __syncthreads();
-    const uint32_t M = st->M;
-    const uint32_t n_groups = (M + kProjThreads - 1) / kProjThreads;
-    for (uint32_t g = blockIdx.x; g < n_groups; g += gridDim.x) {
-        const uint32_t m = g * kProjThreads + threadIdx.x;
-        uint4 f = make_uint4(0, 0, 0, 0);
-        uint32_t tiles_x = 1, tbase = 0;
-        if (m < M) {
-            const uint32_t e = __ldg(sel + m);
-            const uint32_t v = e / t.n_pad;
-            f = proj::project_one(t, s_cam[v], e - v * t.n_pad, m, splat, foot);
-            tiles_x = (uint32_t)s_cam[v].tiles_x;
-            tbase = s_base[v];
-        }
-        warp_count_pairs(f.z, f.x, f.y, tiles_x, tbase, tile_cnt);
-    }
+    proj::project_walk<kDeg>(t, sel, S, splat, foot, tile_cnt, st,
+                             [&](uint32_t e, uint32_t& n, uint32_t& tiles_x, uint32_t& tbase) -> const DevCamera& {
+                                 const uint32_t v = e / t.n_pad;
+                                 n = e - v * t.n_pad;
+                                 tiles_x = (uint32_t)s_cam[v].tiles_x;
+                                 tbase = s_base[v];
+                                 return s_cam[v];
+                             });
 }
 
 // Blend every tile of every view; the tile's view is found by binary search.
@@ -308,8 +303,11 @@ void launch_batch_front(const DevTree& t, const DevCamera* cams, int V, uint32_t
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, banc_kernel, 256, 0);
     launch_pdl(banc_kernel, sms * (occ > 0 ? occ : 1), 256, 0, s, t, V, pbits, selbits, sel_cnt);
     launch_compact_counted_batch(selbits, all_words, sel, sel_cap, sel_cnt, st, s);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, bproject_kernel, kProjThreads, 0);
-    launch_pdl(bproject_kernel, sms * (occ > 0 ? occ : 1), kProjThreads, 0, s, t, cams, V, tile_base, sel, splat, foot,
+    const auto bproject = t.sh_degree == 0   ? bproject_kernel<0>
+                          : t.sh_degree == 1 ? bproject_kernel<1>
+                          : t.sh_degree == 2 ? bproject_kernel<2>
+                                             : bproject_kernel<3>;
+    launch_pdl(bproject, sms * kProjectBlocks, kProjectThreads, 0, s, t, cams, V, tile_base, sel, splat, foot,
                tile_cnt, st);
     launch_tile_scan(tile_cnt, ranges, total_tiles, large, cap, lb_scan, st, sms * occ_tile_scan(), s);
     launch_scatter_batch(cams, tile_base, t.n_pad, sel, foot, tile_cnt, items, cap, st, sms * occ_scatter(), s);

@@ -27,7 +27,9 @@ constexpr int kBatchSelTileWords = 1024;  // the same in the batched form
 inline size_t batch_sel_tiles(size_t words) { return (words + kBatchSelTileWords - 1) / kBatchSelTileWords; }
 constexpr int kAncCacheWords = 4096;      // P-bit words of the lowest node ids kept in shared memory
 constexpr uint32_t kSplitTiles = 912;      // fewer tiles than that of a blend are split (6 an SM)
-constexpr int kProjThreads = 256;         // selected Gaussians per projection tile
+constexpr int kProjectThreads = 128;      // threads per projection block
+constexpr int kProjectBlocks = 6;         // projection blocks an SM (registers; 160 KB of staged SH rows)
+constexpr int kProjThreads = 256;         // Gaussians per scatter tile
 constexpr uint64_t kSpinLimit = 1ull << 24;   // bounded spin-waits
 
 // device status codes (mirrors FGS_ERR_* of the C ABI)
@@ -462,7 +464,6 @@ inline void launch_pdl(void (*kernel)(KArgs...), unsigned grid, unsigned block, 
 int occ_filter_pred();
 int occ_filter_anc();
 int occ_compact();
-int occ_project();
 int occ_scatter();
 int occ_segsort();
 
@@ -495,7 +496,7 @@ void launch_compact_counted_batch(const uint32_t* selbits, uint32_t n_words, uin
 // Projection (splat records, footprints) and the per-tile pair counts
 // tile_cnt[tiles] (zeroed by launch_frame_begin).
 void launch_project(const DevTree& t, const DevCamera& cam, const uint32_t* sel, float* splat,
-                    uint4* foot, uint32_t* tile_cnt, FrameState* st, int blocks, cudaStream_t s);
+                    uint4* foot, uint32_t* tile_cnt, FrameState* st, int sms, cudaStream_t s);
 // Tile ranges (clamped to cap), scatter cursors (in tile_cnt), N_P and the list
 // of tiles with more than kSegSmall pairs (large[], their number in
 // FrameState::tickets[kTicketLarge]); lookback holds
