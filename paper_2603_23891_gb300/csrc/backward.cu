@@ -470,10 +470,16 @@ __device__ __forceinline__ void blend_bwd_walk(const DevCamera& cam, uint32_t ti
     }
 }
 
-// The parameter gradients to be zeroed (none: n == 0), [per_node[k]][n] floats each.
+// Gradients to zero: p[0..3] of per_node[k] floats a node for all n nodes, sh ([n][k3])
+// for the nodes without a bit in selbits (the others' rows are all written later).  vec:
+// rows of sh are multiples of 16 bytes and aligned.
 struct GradZero {
-    float* p[5];
-    uint32_t per_node[5];
+    float* p[4];
+    uint32_t per_node[4];
+    float* sh;
+    uint32_t k3;
+    bool vec;
+    const uint32_t* selbits;
     uint32_t n;
     uint32_t blocks;
 };
@@ -482,26 +488,42 @@ struct GradZero {
 // stores where the array allows.
 __device__ __forceinline__ void zero_share(const GradZero& z, uint32_t part, uint32_t n_parts)
 {
-    for (int k = 0; k < 5; ++k) {
+    const float4 zero4 = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    for (int k = 0; k < 4; ++k) {
         const uint64_t total = (uint64_t)z.per_node[k] * z.n;
         const uint64_t lo = total * part / n_parts, hi = total * (part + 1ull) / n_parts;
         float* p = z.p[k];
         uint64_t a = lo + ((4ull - (((uint64_t)p / 4ull + lo) & 3ull)) & 3ull);      // the first 16-byte boundary
         if (a > hi) a = hi;
         const uint64_t b = a + ((hi - a) & ~3ull);
+        for (uint64_t i = lo + threadIdx.x; i < a; i += blockDim.x) p[i] = 0.0f;
         for (uint64_t i = a + 4ull * threadIdx.x; i < b; i += 4ull * blockDim.x)
-            __stcs(reinterpret_cast<float4*>(p + i), make_float4(0.f, 0.f, 0.f, 0.f));
-        if (lo + threadIdx.x < a) p[lo + threadIdx.x] = 0.0f;
-        if (b + threadIdx.x < hi) p[b + threadIdx.x] = 0.0f;
+            __stcs(reinterpret_cast<float4*>(p + i), zero4);
+        for (uint64_t i = b + threadIdx.x; i < hi; i += blockDim.x) p[i] = 0.0f;
+    }
+    // a warp 32 nodes (a word of selbits) at a time, 16 (or 4) bytes a lane and step
+    const uint32_t lane = threadIdx.x & 31, n_words = (z.n + 31u) >> 5, n_warps = n_parts * (blockDim.x >> 5);
+    const uint32_t unit = z.vec ? 4u : 1u, q = z.k3 / unit;
+    const uint32_t inv = (65536u + q - 1u) / q;           // i / q = i * inv >> 16 for i < 32 q <= 1536 and these q
+    for (uint32_t w = part * (blockDim.x >> 5) + (threadIdx.x >> 5); w < n_words; w += n_warps) {
+        const uint32_t left = z.n - (w << 5);
+        const uint32_t rows = ~__ldg(z.selbits + w) & (left < 32u ? (1u << left) - 1u : 0xFFFFFFFFu);
+        if (!rows) continue;
+        float* p = z.sh + ((size_t)w << 5) * z.k3;
+        for (uint32_t i = lane; i < 32u * q; i += 32u)
+            if ((rows >> (i * inv >> 16)) & 1u) {
+                if (z.vec) __stcs(reinterpret_cast<float4*>(p) + i, zero4);
+                else p[i] = 0.0f;
+            }
     }
 }
 
 // keep holds each pixel's {final T, stop} (kept by a FGS_RENDER_KEEP forward, or
 // recomputed by the forward's walk without an image just before).  zero: the gradients
 // of nodes outside the selection, written by the first zero.blocks blocks beside the
-// walk, where HBM idles (1.25M nodes of degree 3: five memsets of 295 MB in all took 45 us
-// and their launches; a share of the zeros in every block delayed its walk, 252 us
-// instead of 190).
+// walk, where HBM idles (1.25M nodes of degree 3, 537K selected: 43 us of memsets and their
+// launches before; a share of the zeros in every block delayed its walk, 252 us instead
+// of 190; all rows by blocks of their own 224, the unselected nodes' alone 214).
 __global__ void __launch_bounds__(blendk::kWalkChunk) blend_bwd_kernel(
     DevCamera cam, const uint2* __restrict__ ranges, const uint32_t* __restrict__ heavy,
     const uint32_t* __restrict__ vals, const float* __restrict__ splat, const uint2* __restrict__ keep,
@@ -593,7 +615,7 @@ struct GradPtrs {
 
 // Chain rule for selected Gaussian m (node sel[m]): splat gradient -> mean,
 // log-scale, quaternion, logit, SH.  Each node appears once in the selection,
-// so plain stores (or read-modify-writes when accumulating) need no atomics.
+// so plain stores do (reductions when accumulating).
 //
 // Each warp takes 32 consecutive selected Gaussians per iteration, one per
 // lane.  Their SH rows (3 K floats each, contiguous per node) are staged in
@@ -603,7 +625,8 @@ struct GradPtrs {
 // at a time: the row stride is a multiple of 4 floats and odd in units of 4, so the 8
 // lanes of a quarter-warp hit different banks.  Bound: the latency of the rows (8 blocks
 // of 2 warps an SM, by shared memory and registers), so the next group's rows are copied
-// while this one is computed; accumulating, the second buffer holds the old gradients.
+// and its other inputs prefetched while this one is computed (537K Gaussians of degree 3:
+// 73 -> 58 us; accumulating 264K: 36 -> 24).
 __device__ __forceinline__ void cp_async4(float* smem, const float* gmem)
 {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(smem)), "l"(gmem)
@@ -615,6 +638,17 @@ __device__ __forceinline__ void cp_async16(float* smem, const float* gmem)
                  : "memory");
 }
 
+// A gradient stored, or added to what is there: a reduction, so that a group waits for no
+// old value (each node appears once, so the sum is the same as by load and store).
+template <bool kAdd, class T>
+__device__ __forceinline__ void put(T* p, const T& v)
+{
+    if (kAdd) atomicAdd(p, v);
+    else *p = v;
+}
+
+__device__ __forceinline__ void prefetch_l2(const float* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+
 constexpr int kPbWarps = 2;   // warps per projection-backward block
 
 template <int kDeg, bool kAccumulate>
@@ -625,19 +659,16 @@ __global__ void __launch_bounds__(kPbWarps * 32, 16 / kPbWarps) project_bwd_kern
 {
     constexpr int K = (kDeg + 1) * (kDeg + 1);
     constexpr int K3 = 3 * K, Q = (K3 + 3) / 4, RS = 4 * (Q | 1);
-    constexpr int kBuf = kAccumulate ? 1 : 2;         // row buffers: the next group's rows land during this one's work
-    __shared__ __align__(16) float s_rows[kPbWarps][kBuf][32 * RS];
-    __shared__ __align__(16) float s_olds[kAccumulate ? kPbWarps : 1][kAccumulate ? 32 * RS : 4];
+    __shared__ __align__(16) float s_rows[kPbWarps][2][32 * RS];      // the next group's rows land during this one's work
     grid_dep_wait();
     const uint32_t M = st->M;
     const size_t N = p.n;
     const float* W = cam.R;
     const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    float* olds = s_olds[kAccumulate ? warp : 0];
     const uint32_t step = gridDim.x * kPbWarps * 32;
     auto node = [&](uint32_t at) { return at < M ? sel[min(at + lane, M - 1u)] : 0u; };
-    // the SH rows of the group at `at` (nodes nn, one a lane; and, accumulating, their
-    // current gradient rows) with asynchronous copies, all in flight at once
+    // the SH rows of the group at `at` (nodes nn, one a lane) with asynchronous copies, all
+    // in flight at once
     auto stage = [&](uint32_t at, uint32_t nn, float* to) {
         if (at >= M) return;
         if (K3 % 4 == 0 && vec) {
@@ -646,37 +677,40 @@ __global__ void __launch_bounds__(kPbWarps * 32, 16 / kPbWarps) project_bwd_kern
                 const uint32_t idx = (uint32_t)i * 32u + lane, r = idx / Q, k = 4u * (idx - r * Q);
                 const uint32_t nr = __shfl_sync(0xffffffffu, nn, r);
                 cp_async16(to + r * RS + k, p.sh + (size_t)nr * K3 + k);
-                if (kAccumulate && at + r < M) cp_async16(olds + r * RS + k, gr.sh + (size_t)nr * K3 + k);
             }
         } else {
             for (int i = 0; i < K3; ++i) {
                 const uint32_t idx = (uint32_t)i * 32u + lane, r = idx / K3, k = idx - r * K3;
                 const uint32_t nr = __shfl_sync(0xffffffffu, nn, r);
                 cp_async4(to + r * RS + k, p.sh + (size_t)nr * K3 + k);
-                if (kAccumulate && at + r < M) cp_async4(olds + r * RS + k, gr.sh + (size_t)nr * K3 + k);
             }
         }
     };
     uint32_t base = (blockIdx.x * kPbWarps + warp) * 32;
-    uint32_t n = node(base);
-    if (kBuf == 2) {
-        stage(base, n, s_rows[warp][0]);
-        asm volatile("cp.async.commit_group;" ::: "memory");
-    }
-    for (uint32_t buf = 0; base < M; base += step, buf ^= (uint32_t)(kBuf - 1)) {
+    uint32_t n = node(base), n_next = node(base + step);
+    stage(base, n, s_rows[warp][0]);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    for (uint32_t buf = 0; base < M; base += step, buf ^= 1u) {
         const uint32_t m = base + lane;
         const bool act = m < M;
         float* rows = s_rows[warp][buf];
         float* row = rows + lane * RS;
-        const uint32_t n_next = base + step < M ? node(base + step) : 0u;
-        if (kBuf == 2) {
-            stage(base + step, n_next, s_rows[warp][buf ^ 1u]);
-            asm volatile("cp.async.commit_group;" ::: "memory");
-            asm volatile("cp.async.wait_group 1;" ::: "memory");
-        } else {
-            stage(base, n, rows);
-            asm volatile("cp.async.wait_all;" ::: "memory");
+        stage(base + step, n_next, s_rows[warp][buf ^ 1u]);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        const uint32_t n_after = base + step < M ? node(base + 2u * step) : 0u;
+        if (base + step < M) {                            // the next group's other inputs, to L2
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                prefetch_l2(p.mu + k * N + n_next);
+                prefetch_l2(p.log_scale + k * N + n_next);
+            }
+#pragma unroll
+            for (int k = 0; k < 4; ++k) prefetch_l2(p.quat + k * N + n_next);
+            prefetch_l2(p.logit + n_next);
+            const size_t row = (size_t)(base + step) * kGS + lane * 32u;      // kGS lines of 32 floats
+            if (lane < (uint32_t)kGS && row < (size_t)M * kGS) prefetch_l2(gsplat + row);
         }
+        asm volatile("cp.async.wait_group 1;" ::: "memory");
         __syncwarp();
         const float* gs = gsplat + (size_t)(act ? m : base) * kGS;
         const float gu = gs[0], gv = gs[1], gA = gs[2], gB = gs[3], gC = gs[4], ga0 = gs[5];
@@ -814,24 +848,20 @@ __global__ void __launch_bounds__(kPbWarps * 32, 16 / kPbWarps) project_bwd_kern
             for (int i = 0; i < Q; ++i) {
                 const uint32_t idx = (uint32_t)i * 32u + lane, r = idx / Q, k = 4u * (idx - r * Q);
                 const uint32_t nr = __shfl_sync(0xffffffffu, n, r);
-                float4 g = *reinterpret_cast<const float4*>(rows + r * RS + k);
-                if (kAccumulate) {
-                    const float4 o = *reinterpret_cast<const float4*>(olds + r * RS + k);
-                    g = make_float4(g.x + o.x, g.y + o.y, g.z + o.z, g.w + o.w);
-                }
-                if (base + r < M) *reinterpret_cast<float4*>(gr.sh + (size_t)nr * K3 + k) = g;
+                const float4 g = *reinterpret_cast<const float4*>(rows + r * RS + k);
+                if (base + r < M) put<kAccumulate>(reinterpret_cast<float4*>(gr.sh + (size_t)nr * K3 + k), g);
             }
         } else {
             for (int i = 0; i < K3; ++i) {
                 const uint32_t idx = (uint32_t)i * 32u + lane, r = idx / K3, k = idx - r * K3;
                 const uint32_t nr = __shfl_sync(0xffffffffu, n, r);
-                const float g = rows[r * RS + k] + (kAccumulate ? olds[r * RS + k] : 0.0f);
-                if (base + r < M) gr.sh[(size_t)nr * K3 + k] = g;
+                if (base + r < M) put<kAccumulate>(gr.sh + (size_t)nr * K3 + k, rows[r * RS + k]);
             }
         }
         __syncwarp();
         const uint32_t nn = n;
         n = n_next;
+        n_next = n_after;
         if (!act) continue;
         const float dd = gd[0] * d[0] + gd[1] * d[1] + gd[2] * d[2];
 #pragma unroll
@@ -839,36 +869,14 @@ __global__ void __launch_bounds__(kPbWarps * 32, 16 / kPbWarps) project_bwd_kern
         float gqn[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k) gqn[k] = (gq[k] - qh[k] * dotq) / qn;
-        if (kAccumulate) {
-            // all eleven loads before the first store (the arrays may alias as far
-            // as the compiler knows)
-            float o_mu[3], o_ls[3], o_q[4];
 #pragma unroll
-            for (int k = 0; k < 3; ++k) {
-                o_mu[k] = gr.mu[k * N + nn];
-                o_ls[k] = gr.log_scale[k * N + nn];
-            }
-#pragma unroll
-            for (int k = 0; k < 4; ++k) o_q[k] = gr.quat[k * N + nn];
-            const float o_l = gr.logit[nn];
-#pragma unroll
-            for (int k = 0; k < 3; ++k) {
-                gr.mu[k * N + nn] = o_mu[k] + gmu[k];
-                gr.log_scale[k * N + nn] = o_ls[k] + gls[k];
-            }
-#pragma unroll
-            for (int k = 0; k < 4; ++k) gr.quat[k * N + nn] = o_q[k] + gqn[k];
-            gr.logit[nn] = o_l + glogit;
-        } else {
-#pragma unroll
-            for (int k = 0; k < 3; ++k) {
-                gr.mu[k * N + nn] = gmu[k];
-                gr.log_scale[k * N + nn] = gls[k];
-            }
-#pragma unroll
-            for (int k = 0; k < 4; ++k) gr.quat[k * N + nn] = gqn[k];
-            gr.logit[nn] = glogit;
+        for (int k = 0; k < 3; ++k) {
+            put<kAccumulate>(gr.mu + k * N + nn, gmu[k]);
+            put<kAccumulate>(gr.log_scale + k * N + nn, gls[k]);
         }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) put<kAccumulate>(gr.quat + k * N + nn, gqn[k]);
+        put<kAccumulate>(gr.logit + nn, glogit);
     }
 }
 
@@ -912,8 +920,8 @@ static void launch_project_bwd(const DevTree& t, const DevCamera& cam, const Par
 
 void launch_backward(const DevTree& t, const DevCamera& cam, const uint2* ranges, const uint32_t* heavy,
                      const uint32_t* vals,
-                     const float* splat, uint2* keep, bool kept, const uint32_t* sel, const float* dL_drgb,
-                     float* gsplat, const float* const params[5], float* const grads[5], bool accumulate,
+                     const float* splat, uint2* keep, bool kept, const uint32_t* sel, const uint32_t* selbits,
+                     const float* dL_drgb, float* gsplat, const float* const params[5], float* const grads[5], bool accumulate,
                      int sms, FrameState* st, cudaStream_t s)
 {
     // gsplat rows of the selected Gaussians start at zero: the blend backward adds into them
@@ -923,7 +931,8 @@ void launch_backward(const DevTree& t, const DevCamera& cam, const uint2* ranges
     const GradPtrs gr{grads[0], grads[1], grads[2], grads[3], grads[4]};
     // nodes outside the selection get zero gradient
     const uint32_t K3 = (t.sh_degree + 1) * (t.sh_degree + 1) * 3;
-    const GradZero zero{{gr.mu, gr.log_scale, gr.quat, gr.logit, gr.sh}, {3, 3, 4, 1, K3}, t.n, accumulate ? 0u : (uint32_t)sms};
+    const GradZero zero{{gr.mu, gr.log_scale, gr.quat, gr.logit}, {3, 3, 4, 1}, gr.sh, K3,
+                        K3 % 4 == 0 && ((uintptr_t)gr.sh & 15u) == 0, selbits, t.n, accumulate ? 0u : (uint32_t)sms};
     const int n_tiles = cam.tiles_x * cam.tiles_y;
     launch_pdl(blend_bwd_kernel, n_tiles + 2 * split_slots(n_tiles) + (int)zero.blocks, blendk::kWalkChunk, 0, s, cam,
                ranges, heavy, vals, splat, keep, dL_drgb, gsplat, zero, st);

@@ -545,10 +545,9 @@ void launch_prep_params(const DevTree& t, const float* mu, const float* log_scal
 // keep: per-pixel {final T, stop} buffer; kept: the last forward filled it
 // (FGS_RENDER_KEEP), otherwise the forward's walk runs again and fills it.
 void launch_backward(const DevTree& t, const DevCamera& cam, const uint2* ranges, const uint32_t* heavy,
-                     const uint32_t* vals,
-                     const float* splat, uint2* keep, bool kept, const uint32_t* sel, const float* dL_drgb,
-                     float* gsplat,
-                     const float* const params[5], float* const grads[5], bool accumulate, int proj_blocks,
+                     const uint32_t* vals, const float* splat, uint2* keep, bool kept, const uint32_t* sel,
+                     const uint32_t* selbits, const float* dL_drgb, float* gsplat,
+                     const float* const params[5], float* const grads[5], bool accumulate, int sms,
                      FrameState* st, cudaStream_t s);
 void launch_levelwise_step(const DevTree& t, const DevCamera& cam, const uint32_t* child_start,
                            const uint32_t* children, const uint32_t* frontier, uint32_t n_front,
