@@ -172,7 +172,6 @@ OPS_PER_HIT = 24.0    # exp (15: k by one FMA and a subtraction, reduction 2 FMA
 # source files of each frame kernel (a kernel's committed DRAM figure is used only
 # while these files are unchanged)
 KERNEL_SOURCES = {
-    "frame_begin_kernel": ["filter.cu", "fgs_internal.cuh"],
     "filter_pred_kernel": ["filter.cu", "fgs_internal.cuh"],
     "filter_anc_kernel": ["filter.cu", "fgs_internal.cuh"],
     "compact_counted_kernel": ["filter.cu", "fgs_internal.cuh"],
@@ -184,7 +183,7 @@ KERNEL_SOURCES = {
 }
 # the kernels of each bench stage
 STAGE_KERNELS = {
-    "filter_rl": ["frame_begin_kernel", "filter_pred_kernel"],
+    "filter_rl": ["filter_pred_kernel"],
     "ancestor_compact": ["filter_anc_kernel", "compact_counted_kernel"],
     "project": ["project_kernel"],
     "tile_ranges": ["tile_scan_kernel"],

@@ -29,10 +29,7 @@
  *  - Errors raised on the device (pair capacity exceeded, a bounded spin-wait
  *    that timed out) are latched in a device status word and returned by the
  *    next synchronising call or fgs_sync().  After FGS_ERR_TIMEOUT from a
- *    render (a blend's staging copy whose wait gave up may still have been in
- *    flight when its block exited) the frame and the context are not to be
- *    trusted: destroy the context.  (fgs_probe_wait_timeout's timeout is the
- *    exception: its wait has no copy in flight.)
+ *    render (a look-back of the tile scan gave up) the frame is not to be used.
  *  - A context is not thread-safe; use one context per host thread.
  */
 #ifndef FILTERGS_H
@@ -127,7 +124,8 @@ typedef struct fgs_params {
     int32_t tile_w, tile_h;   /* tile size in pixels: 64x4, 32x8, 16x16 (default) or 8x32 */
     float bg[3];              /* background colour added as T * bg */
     uint64_t pair_capacity;   /* max Gaussian-tile pairs per frame (0 = keep current / default) */
-    int32_t blend_warp_w;     /* blend block shape: warps of 8x4 (8, default; 0 = 8) or 4x8 (4) pixels */
+    int32_t blend_warp_w;     /* 8 (default; 0 = 8) or 4: accepted and checked against the tile, without
+                                 effect (the blend walks 4x4 blocks) */
     int32_t reserved;
 } fgs_params;
 

@@ -86,10 +86,10 @@ struct FrameState {
     int32_t status;            // latched error (0 = ok)
     uint32_t status_info;
     uint32_t reserved0;
-    unsigned long long blend_entries;     // lockstep warp steps of the list walk (counting frames only)
+    unsigned long long blend_entries;     // test steps of the list walk (counting frames only)
     unsigned long long blend_evals;       // pixel-Gaussian evaluations (lanes not yet stopped)
     unsigned long long blend_hits;        // evaluations that reached the alpha / T update
-    unsigned long long blend_active;      // lockstep steps where some lane reached it
+    unsigned long long blend_active;      // steps where some pixel reached it
     uint32_t n_emitting;                  // selected Gaussians with at least one pair
     unsigned long long filter_in_frustum; // counting frames: nodes in the frustum
     unsigned long long filter_cov_nodes;  // counting frames: in-frustum internal nodes
@@ -494,7 +494,7 @@ void launch_compact_counted(const uint32_t* selbits, uint32_t n_words, uint32_t*
 void launch_compact_counted_batch(const uint32_t* selbits, uint32_t n_words, uint32_t* sel, uint32_t cap,
                                   const uint32_t* sel_cnt, FrameState* st, cudaStream_t s);
 // Projection (splat records, footprints) and the per-tile pair counts
-// tile_cnt[tiles] (zeroed by launch_frame_begin).
+// tile_cnt[tiles] (zeroed at the frame's begin).
 void launch_project(const DevTree& t, const DevCamera& cam, const uint32_t* sel, float* splat,
                     uint4* foot, uint32_t* tile_cnt, FrameState* st, int sms, cudaStream_t s);
 // Tile ranges (clamped to cap), scatter cursors (in tile_cnt), N_P and the list

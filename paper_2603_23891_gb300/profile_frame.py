@@ -9,7 +9,7 @@ so the launch sequence is exactly the per-frame path (9 kernels per frame:
 frame_begin, filter_pred, filter_anc, compact_counted, project, tile_scan, scatter,
 segsort, blend).
 Without it the frames use the 3-sigma footprint.  With --backward the tree's
-attributes are first recomputed from its parameters (one prep_params launch)
+attributes are first recomputed from its parameters (one prep launch)
 and every frame is followed by the differentiable form's backward for
 dL/drgb ~ N(0, 1) (accumulate mode: zero_rows, blend_bwd, project_bwd).
 """
