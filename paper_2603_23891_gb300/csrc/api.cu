@@ -126,7 +126,6 @@ struct fgs_ctx {
         uint32_t total_tiles = 0;
         uint64_t sel_cap = 0, pair_cap = 0;
         DevCamera* d_cams = nullptr;
-        DevCamera* h_cams = nullptr;              // pinned staging
         uint32_t* d_tile_base = nullptr;
         unsigned long long* d_img_off = nullptr;
         uint32_t *pbits = nullptr, *selbits = nullptr, *sel = nullptr;
@@ -479,7 +478,6 @@ int fgs_destroy(fgs_ctx* c)
                       b.foot, b.items, b.keys, b.vals, b.sel_cnt, b.lb_scan, b.ranges, b.tile_cnt, b.large,
                       b.heavy, b.st};
         for (void* p : bb) free_ptr(p);
-        if (b.h_cams) cudaFreeHost(b.h_cams);
         if (b.graph) cudaGraphExecDestroy(b.graph);
     }
     if (c->st_host) cudaFreeHost(c->st_host);
@@ -1185,7 +1183,7 @@ int fgs_backward(fgs_ctx* c, void* stream, const float* dL_drgb, const fgs_gauss
 int fgs_batch_setup(fgs_ctx* c, const fgs_camera* views, int n_views, const int32_t* tile_shapes,
                     uint64_t sel_capacity, uint64_t pair_capacity)
 {
-    if (!c || !views || n_views < 1 || n_views > 64) return FGS_ERR_ARG;
+    if (!c || !views || n_views < 1 || n_views > kMaxBatchViews) return FGS_ERR_ARG;
     if (!c->has_tree) return fail(c, FGS_ERR_STATE, "no tree loaded");
     for (int v = 0; v < n_views; ++v)
         if (!valid_camera(views + v)) return fail(c, FGS_ERR_ARG, "view %d: invalid camera", v);
@@ -1230,7 +1228,6 @@ int fgs_batch_setup(fgs_ctx* c, const fgs_camera* views, int n_views, const int3
     const size_t n_words = c->tree.n_pad / 32;
     int r;
     if ((r = grow(c, (void**)&b.d_cams, sizeof(DevCamera) * n_views))) return r;
-    if (!b.h_cams) FGS_CUDA(c, cudaMallocHost((void**)&b.h_cams, sizeof(DevCamera) * 64));
     if ((r = grow(c, (void**)&b.d_tile_base, 4 * (n_views + 1)))) return r;
     if ((r = grow(c, (void**)&b.d_img_off, 8 * (n_views + 1)))) return r;
     if ((r = grow(c, (void**)&b.pbits, 4 * n_words * n_views))) return r;
@@ -1309,12 +1306,10 @@ int fgs_render_batch(fgs_ctx* c, void* stream, float* rgb_out, float* T_out, uin
     if (!c->has_tree) return fail(c, FGS_ERR_STATE, "no tree loaded");
     DeviceGuard g(c->device);
     cudaStream_t s = (cudaStream_t)stream;
-    for (int v = 0; v < b.V; ++v) {
-        DevCamera d = make_devcam_for(c, b.cams[v], b.tile_w[v], b.tile_h[v], b.warp_w[v]);
-        b.h_cams[v] = d;
-    }
-    FGS_CUDA(c, cudaMemcpyAsync(b.d_cams, b.h_cams, sizeof(DevCamera) * b.V, cudaMemcpyHostToDevice, s));
-    const int launches = 8;
+    DevCamera cams[kMaxBatchViews];
+    for (int v = 0; v < b.V; ++v) cams[v] = make_devcam_for(c, b.cams[v], b.tile_w[v], b.tile_h[v], b.warp_w[v]);
+    launch_batch_cameras(cams, b.V, b.d_cams, s);
+    const int launches = 9;
     if (flags & FGS_BATCH_GRAPH) {
         if (!b.graph || b.graph_rgb != rgb_out || b.graph_T != T_out) {
             if (b.graph) {

@@ -21,9 +21,34 @@
 #include "pairs_impl.cuh"
 #include "project_impl.cuh"
 
+#include <cstring>
+
 namespace fgs {
 
-constexpr int kMaxBatchViews = 64;
+// The cameras by value: the launch takes its copy, so the host may set the next call's at
+// once and no staging buffer has to outlive a copy in flight.  (64 cameras are 9.5 KB of
+// parameters; most batches need the smaller form.)
+template <int N>
+struct CameraPack {
+    DevCamera c[N];
+};
+
+template <int N>
+__global__ void __launch_bounds__(128) bcameras_kernel(const __grid_constant__ CameraPack<N> pack, int V,
+                                                       DevCamera* __restrict__ dst)
+{
+    grid_dep_wait();
+    for (int i = threadIdx.x; i < V * (int)(sizeof(DevCamera) / 4); i += blockDim.x)
+        reinterpret_cast<uint32_t*>(dst)[i] = reinterpret_cast<const uint32_t*>(pack.c)[i];
+}
+
+template <int N>
+static void launch_cameras(const DevCamera* cams, int V, DevCamera* dst, cudaStream_t s)
+{
+    CameraPack<N> pack;
+    memcpy(pack.c, cams, sizeof(DevCamera) * V);
+    launch_pdl(bcameras_kernel<N>, 1, 128, 0, s, pack, V, dst);
+}
 
 // R&L for V views: a warp takes chunks of 128 nodes g, g + W, g + 2W, ... (W warps), 32
 // at a time: lane l tests the box of the l-th against every view's frustum planes (in
@@ -287,6 +312,12 @@ __global__ void __launch_bounds__(blendk::kWalkChunk) bblend_kernel(
 // ---------------------------------------------------------------------------
 // launchers
 // ---------------------------------------------------------------------------
+void launch_batch_cameras(const DevCamera* cams, int V, DevCamera* dst, cudaStream_t s)
+{
+    if (V <= 16) launch_cameras<16>(cams, V, dst, s);
+    else launch_cameras<kMaxBatchViews>(cams, V, dst, s);
+}
+
 void launch_batch_front(const DevTree& t, const DevCamera* cams, int V, uint32_t total_tiles,
                         const uint32_t* tile_base, uint32_t* pbits, uint32_t* selbits, uint32_t* sel,
                         uint32_t sel_cap, float* splat, uint4* foot, uint32_t* tile_cnt, uint32_t* large, uint32_t* heavy,

@@ -30,6 +30,7 @@ constexpr uint32_t kSplitTiles = 912;      // fewer tiles than that of a blend a
 constexpr int kProjectThreads = 128;      // threads per projection block
 constexpr int kProjectBlocks = 6;         // projection blocks an SM (registers; 160 KB of staged SH rows)
 constexpr int kProjThreads = 256;         // Gaussians per scatter tile
+constexpr int kMaxBatchViews = 64;
 constexpr uint64_t kSpinLimit = 1ull << 24;   // bounded spin-waits
 
 // device status codes (mirrors FGS_ERR_* of the C ABI)
@@ -530,6 +531,8 @@ void launch_blend_kpc(const DevCamera& cam, const uint2* ranges, const uint32_t*
                       const float* splat, float* kpc, float* G, FrameState* st, cudaStream_t s);
 
 void launch_eval_exp(const float* x, float* y, uint64_t n, cudaStream_t s);
+// The batch's cameras to dst (device), read from the host's array before it returns.
+void launch_batch_cameras(const DevCamera* cams, int V, DevCamera* dst, cudaStream_t s);
 void launch_batch_front(const DevTree& t, const DevCamera* cams, int V, uint32_t total_tiles,
                         const uint32_t* tile_base, uint32_t* pbits, uint32_t* selbits, uint32_t* sel,
                         uint32_t sel_cap, float* splat, uint4* foot, uint32_t* tile_cnt, uint32_t* large, uint32_t* heavy,
