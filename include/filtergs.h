@@ -337,7 +337,9 @@ int fgs_compact_selection_noalloc(const uint32_t* selbits, uint64_t n_words, uin
  * entries and Gaussian-tile pairs of the whole batch (0 = defaults: views x
  * nodes up to 64 Mi entries, 128 Mi pairs).  Allocates the batch buffers.
  * The batch keeps the context's tau_R, background and shrink mode as they are
- * at each fgs_render_batch call.  Errors: FGS_ERR_ARG, FGS_ERR_STATE (no
+ * at each fgs_render_batch call.  A tree loaded later is rendered with the same
+ * set-up if it is no larger (node count rounded up to 4096); for a larger one
+ * fgs_render_batch returns FGS_ERR_STATE until the batch is set up again.  Errors: FGS_ERR_ARG, FGS_ERR_STATE (no
  * tree), FGS_ERR_NOMEM. */
 int fgs_batch_setup(fgs_ctx* ctx, const fgs_camera* views, int n_views, const int32_t* tile_shapes,
                     uint64_t sel_capacity, uint64_t pair_capacity);
@@ -362,7 +364,8 @@ int fgs_batch_image_offsets(const fgs_ctx* ctx, uint64_t* offsets_out);
  * FGS_BATCH_GRAPH replays a CUDA graph captured on first use for these output
  * pointers (re-captured when they change); FGS_RENDER_STATS synchronises and
  * fills st (n_selected, n_pairs over the batch).  Asynchronous otherwise.
- * Errors: FGS_ERR_STATE (no set-up), FGS_ERR_CAPACITY (with STATS), CUDA. */
+ * Errors: FGS_ERR_STATE (no set-up, or one for a smaller tree than the loaded
+ * one), FGS_ERR_CAPACITY (with STATS), CUDA. */
 int fgs_render_batch(fgs_ctx* ctx, void* stream, float* rgb_out, float* T_out, uint32_t flags,
                      fgs_stats* st);
 

@@ -119,6 +119,7 @@ struct fgs_ctx {
     // batched multi-view state
     struct Batch {
         int V = 0;
+        uint32_t n_pad = 0;                       // nodes a view the buffers hold (the tree's at set-up)
         std::vector<fgs_camera> cams;
         std::vector<int32_t> tile_w, tile_h, warp_w;
         std::vector<uint32_t> tile_base;          // V + 1
@@ -182,6 +183,13 @@ int grow(fgs_ctx* c, void** p, size_t bytes)
     FGS_CUDA(c, cudaMalloc(p, bytes));
     FGS_CUDA(c, cudaMemset(*p, 0, bytes));
     return FGS_OK;
+}
+
+// The batch's captured graph is captured again when it is next asked for.
+void drop_graph(fgs_ctx* c)
+{
+    if (c->batch.graph) cudaGraphExecDestroy(c->batch.graph);
+    c->batch.graph = nullptr;
 }
 
 // Pair buffers sized exactly for `cap` pairs (reallocated when it changes).
@@ -478,8 +486,8 @@ int fgs_destroy(fgs_ctx* c)
                       b.foot, b.items, b.keys, b.vals, b.sel_cnt, b.lb_scan, b.ranges, b.tile_cnt, b.large,
                       b.heavy, b.st};
         for (void* p : bb) free_ptr(p);
-        if (b.graph) cudaGraphExecDestroy(b.graph);
     }
+    drop_graph(c);
     if (c->st_host) cudaFreeHost(c->st_host);
     if (c->G_host) cudaFreeHost(c->G_host);
     if (c->h_counter) cudaFreeHost(c->h_counter);
@@ -624,6 +632,7 @@ int fgs_load_tree(fgs_ctx* c, const fgs_tree* t)
     c->has_tree = false;
     c->have_frame = false;
     c->batch.have_frame = false;
+    drop_graph(c);                        // it holds the old tree's pointers
     FGS_CUDA(c, cudaMalloc(&c->tree_mem, total));
     FGS_CUDA(c, cudaMemset(c->tree_mem, 0, total));
     char* base = (char*)c->tree_mem;
@@ -1191,11 +1200,9 @@ int fgs_batch_setup(fgs_ctx* c, const fgs_camera* views, int n_views, const int3
         return fail(c, FGS_ERR_ARG, "views x nodes exceeds 2^32 selection entries");
     DeviceGuard g(c->device);
     auto& b = c->batch;
-    if (b.graph) {
-        cudaGraphExecDestroy(b.graph);
-        b.graph = nullptr;
-    }
+    drop_graph(c);
     b.V = n_views;
+    b.n_pad = c->tree.n_pad;
     b.have_frame = false;
     b.cams.assign(views, views + n_views);
     b.tile_w.assign(n_views, c->params.tile_w);
@@ -1304,6 +1311,9 @@ int fgs_render_batch(fgs_ctx* c, void* stream, float* rgb_out, float* T_out, uin
     auto& b = c->batch;
     if (b.V == 0) return fail(c, FGS_ERR_STATE, "no batch set up");
     if (!c->has_tree) return fail(c, FGS_ERR_STATE, "no tree loaded");
+    if (c->tree.n_pad > b.n_pad)
+        return fail(c, FGS_ERR_STATE, "the batch was set up for a smaller tree (%u nodes a view, now %u)", b.n_pad,
+                    c->tree.n_pad);
     DeviceGuard g(c->device);
     cudaStream_t s = (cudaStream_t)stream;
     DevCamera cams[kMaxBatchViews];
@@ -1312,10 +1322,7 @@ int fgs_render_batch(fgs_ctx* c, void* stream, float* rgb_out, float* T_out, uin
     const int launches = 9;
     if (flags & FGS_BATCH_GRAPH) {
         if (!b.graph || b.graph_rgb != rgb_out || b.graph_T != T_out) {
-            if (b.graph) {
-                cudaGraphExecDestroy(b.graph);
-                b.graph = nullptr;
-            }
+            drop_graph(c);
             cudaStream_t cs;
             FGS_CUDA(c, cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
             FGS_CUDA(c, cudaStreamSynchronize(s));

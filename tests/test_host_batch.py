@@ -92,3 +92,25 @@ def test_calls_in_flight_keep_their_cameras(api, ctx, n_views, flags):
     for k in range(4):
         for r in recs[2 * k: 2 * k + 2]:
             assert r["nulls"] == 0 and np.array_equal(r["t"], want[k]), k
+
+
+@pytest.mark.parametrize("flags", [0, 4])
+def test_tree_loaded_after_the_set_up(api, ctx, flags):
+    """A tree that the batch's buffers cannot hold is refused until the next set-up; one that
+    they hold is rendered, and by a graph captured on that tree."""
+    out = C.c_void_p(0x1000)
+    _load(api, ctx, n_leaves=3000)                         # 4096 to 8192 nodes
+    assert _setup(api, ctx, _cams(api, 3, 0.0)) == 0
+    assert api.fgs_render_batch(ctx, None, out, out, flags, None) == 0
+    assert api.fake_graphs() == (flags == 4)
+    _load(api, ctx, n_leaves=30000)
+    assert api.fake_graphs() == 0
+    assert api.fgs_render_batch(ctx, None, out, out, flags, None) == api.b.FGS_ERR_STATE
+    assert _setup(api, ctx, _cams(api, 3, 0.0)) == 0
+    assert api.fgs_render_batch(ctx, None, out, out, flags, None) == 0
+    _load(api, ctx, n_leaves=200)
+    assert api.fake_graphs() == 0
+    assert api.fgs_render_batch(ctx, None, out, out, flags, None) == 0
+    api.fake_drain()
+    n_pad = [_record(api, i)["n_pad"] for i in range(0, api.fake_records(), 2)]
+    assert len(n_pad) == 3 and n_pad[0] > 4096 and n_pad[1] > n_pad[0] and n_pad[2] == 4096
