@@ -162,12 +162,15 @@ int fail(fgs_ctx* c, int code, const char* fmt, ...)
     return code;
 }
 
+// (cudaGetLastError: an error reported here is not reported by the next call again)
 #define FGS_CUDA(ctx, expr)                                                                   \
     do {                                                                                      \
         cudaError_t e_ = (expr);                                                              \
-        if (e_ != cudaSuccess)                                                                \
+        if (e_ != cudaSuccess) {                                                              \
+            (void)cudaGetLastError();                                                         \
             return fail((ctx), e_ == cudaErrorMemoryAllocation ? FGS_ERR_NOMEM : FGS_ERR_CUDA, \
                         "%s: %s (%s:%d)", #expr, cudaGetErrorString(e_), __FILE__, __LINE__); \
+        }                                                                                     \
     } while (0)
 
 void free_ptr(void* p)
@@ -192,11 +195,15 @@ void drop_graph(fgs_ctx* c)
     c->batch.graph = nullptr;
 }
 
+// The ensure_* functions set a buffer set's capacity to 0 while they replace it, so that a
+// failed allocation leaves none (check_ready refuses to launch on those) and the next
+// call allocates again.
 // Pair buffers sized exactly for `cap` pairs (reallocated when it changes).
 int ensure_pairs(fgs_ctx* c, uint64_t cap)
 {
     if (cap == c->pair_cap) return FGS_OK;
     int r;
+    c->pair_cap = 0;
     const size_t n = (size_t)cap + 8;   // TMA reads an aligned superset of a slice
     if ((r = grow(c, (void**)&c->keys0, n * 8))) return r;
     if ((r = grow(c, (void**)&c->keys1, n * 8))) return r;
@@ -212,6 +219,7 @@ int ensure_nodes(fgs_ctx* c, size_t n_pad)
 {
     if (n_pad <= c->node_cap) return FGS_OK;
     int r;
+    c->node_cap = 0;
     if ((r = grow(c, (void**)&c->pbits, n_pad / 32 * 4))) return r;
     if ((r = grow(c, (void**)&c->selbits, n_pad / 32 * 4))) return r;
     if ((r = grow(c, (void**)&c->sel, n_pad * 4))) return r;
@@ -238,6 +246,7 @@ int ensure_ring(fgs_ctx* c, size_t pixels)
     }
     if (pixels > c->ring_cap) {
         FGS_CUDA(c, cudaStreamSynchronize(c->copy_stream));
+        c->ring_cap = 0;
         for (int i = 0; i < 2; ++i)
             if ((r = grow(c, (void**)&c->ring[i], pixels * 4 * 4))) return r;
         c->ring_busy[0] = c->ring_busy[1] = false;
@@ -250,6 +259,7 @@ int ensure_tiles(fgs_ctx* c, size_t tiles, size_t pixels)
 {
     int r;
     if (tiles > c->tile_cap) {
+        c->tile_cap = 0;
         if ((r = grow(c, (void**)&c->ranges, tiles * sizeof(uint2)))) return r;
         if ((r = grow(c, (void**)&c->tile_cnt, tiles * 4))) return r;
         if ((r = grow(c, (void**)&c->large, tiles * 4))) return r;
@@ -261,6 +271,7 @@ int ensure_tiles(fgs_ctx* c, size_t tiles, size_t pixels)
         c->tile_cap = tiles;
     }
     if (pixels > c->img_cap) {
+        c->img_cap = 0;
         if ((r = grow(c, (void**)&c->img, pixels * 4 * 4))) return r;
         if ((r = grow(c, (void**)&c->keep, pixels * sizeof(uint2)))) return r;
         c->img_cap = pixels;
@@ -351,6 +362,8 @@ int check_ready(fgs_ctx* c)
     if (!c) return FGS_ERR_ARG;
     if (!c->has_tree) return fail(c, FGS_ERR_STATE, "no tree loaded");
     if (!c->has_cam) return fail(c, FGS_ERR_STATE, "no camera set");
+    if (!c->node_cap || !c->pair_cap || !c->tile_cap || !c->img_cap)
+        return fail(c, FGS_ERR_STATE, "no frame buffers: an allocation failed");
     return FGS_OK;
 }
 
@@ -1172,6 +1185,7 @@ int fgs_backward(fgs_ctx* c, void* stream, const float* dL_drgb, const fgs_gauss
                            "grad mu", "grad log_scale", "grad quat", "grad logit", "grad sh"};
     if ((r = check_param_ptrs(c, ptrs, names, 11))) return r;
     if (c->gsplat_rows < c->tree.n) {
+        c->gsplat_rows = 0;
         if ((r = grow(c, (void**)&c->gsplat, (size_t)c->tree.n * 12 * sizeof(float)))) return r;
         c->gsplat_rows = c->tree.n;
     }
@@ -1198,16 +1212,9 @@ int fgs_batch_setup(fgs_ctx* c, const fgs_camera* views, int n_views, const int3
         if (!valid_camera(views + v)) return fail(c, FGS_ERR_ARG, "view %d: invalid camera", v);
     if ((uint64_t)n_views * c->tree.n_pad >= (1ull << 32))
         return fail(c, FGS_ERR_ARG, "views x nodes exceeds 2^32 selection entries");
-    DeviceGuard g(c->device);
-    auto& b = c->batch;
-    drop_graph(c);
-    b.V = n_views;
-    b.n_pad = c->tree.n_pad;
-    b.have_frame = false;
-    b.cams.assign(views, views + n_views);
-    b.tile_w.assign(n_views, c->params.tile_w);
-    b.tile_h.assign(n_views, c->params.tile_h);
-    b.warp_w.assign(n_views, c->params.blend_warp_w);
+    // everything is checked before the current set-up is touched
+    std::vector<int32_t> tile_w(n_views, c->params.tile_w), tile_h(n_views, c->params.tile_h);
+    std::vector<int32_t> warp_w(n_views, c->params.blend_warp_w);
     if (tile_shapes) {
         for (int v = 0; v < n_views; ++v) {
             const int tw = tile_shapes[3 * v], th = tile_shapes[3 * v + 1];
@@ -1215,11 +1222,25 @@ int fgs_batch_setup(fgs_ctx* c, const fgs_camera* views, int n_views, const int3
             if (!is_pow2(tw) || !is_pow2(th) || tw * th != 256 || tw < 8 || th < 4 ||
                 (ww != 8 && ww != 4) || th < 32 / ww)
                 return fail(c, FGS_ERR_ARG, "view %d: tile %dx%d / warp %d not supported", v, tw, th, ww);
-            b.tile_w[v] = tw;
-            b.tile_h[v] = th;
-            b.warp_w[v] = ww;
+            tile_w[v] = tw;
+            tile_h[v] = th;
+            warp_w[v] = ww;
         }
     }
+    const uint64_t sel_cap = sel_capacity ? sel_capacity : std::min<uint64_t>((uint64_t)n_views * c->tree.n_pad, 64ull << 20);
+    const uint64_t pair_cap = pair_capacity ? pair_capacity : (128ull << 20);
+    if (pair_cap > kMaxPairCap) return fail(c, FGS_ERR_ARG, "pair capacity too large");
+    DeviceGuard g(c->device);
+    auto& b = c->batch;
+    drop_graph(c);
+    // no views, and no capacity for the buffers being replaced, until all of it is there
+    b.V = 0;
+    b.have_frame = false;
+    b.n_pad = c->tree.n_pad;
+    b.cams.assign(views, views + n_views);
+    b.tile_w = tile_w;
+    b.tile_h = tile_h;
+    b.warp_w = warp_w;
     b.tile_base.assign(n_views + 1, 0);
     b.img_off.assign(n_views + 1, 0);
     for (int v = 0; v < n_views; ++v) {
@@ -1229,9 +1250,6 @@ int fgs_batch_setup(fgs_ctx* c, const fgs_camera* views, int n_views, const int3
         b.img_off[v + 1] = b.img_off[v] + (unsigned long long)views[v].width * views[v].height;
     }
     b.total_tiles = b.tile_base[n_views];
-    const uint64_t sel_cap = sel_capacity ? sel_capacity : std::min<uint64_t>((uint64_t)n_views * c->tree.n_pad, 64ull << 20);
-    const uint64_t pair_cap = pair_capacity ? pair_capacity : (128ull << 20);
-    if (pair_cap > kMaxPairCap) return fail(c, FGS_ERR_ARG, "pair capacity too large");
     const size_t n_words = c->tree.n_pad / 32;
     int r;
     if ((r = grow(c, (void**)&b.d_cams, sizeof(DevCamera) * n_views))) return r;
@@ -1242,12 +1260,14 @@ int fgs_batch_setup(fgs_ctx* c, const fgs_camera* views, int n_views, const int3
     if ((r = grow(c, (void**)&b.sel_cnt, 4 * batch_sel_tiles(n_words * n_views)))) return r;
     if ((r = grow(c, (void**)&b.lb_scan, 8 * tile_scan_lookback_entries(b.total_tiles)))) return r;
     if (sel_cap != b.sel_cap) {
+        b.sel_cap = 0;
         if ((r = grow(c, (void**)&b.sel, 4 * sel_cap))) return r;
         if ((r = grow(c, (void**)&b.splat, 4 * kSplatStride * sel_cap))) return r;
         if ((r = grow(c, (void**)&b.foot, sizeof(uint4) * sel_cap))) return r;
         b.sel_cap = sel_cap;
     }
     if (pair_cap != b.pair_cap) {
+        b.pair_cap = 0;
         const size_t n = pair_cap + 8;
         if ((r = grow(c, (void**)&b.items, 8 * n))) return r;
         if ((r = grow(c, (void**)&b.keys, 8 * n))) return r;
@@ -1257,12 +1277,11 @@ int fgs_batch_setup(fgs_ctx* c, const fgs_camera* views, int n_views, const int3
     if ((r = grow(c, (void**)&b.ranges, sizeof(uint2) * b.total_tiles))) return r;
     if ((r = grow(c, (void**)&b.tile_cnt, 4 * b.total_tiles))) return r;
     if ((r = grow(c, (void**)&b.large, 4 * b.total_tiles))) return r;
-    if (!b.st) {
-        if ((r = grow(c, (void**)&b.st, sizeof(FrameState)))) return r;
-        if ((r = grow(c, (void**)&b.heavy, 4 * kSplitTiles))) return r;
-    }
+    if (!b.st && (r = grow(c, (void**)&b.st, sizeof(FrameState)))) return r;
+    if (!b.heavy && (r = grow(c, (void**)&b.heavy, 4 * kSplitTiles))) return r;
     FGS_CUDA(c, cudaMemcpy(b.d_tile_base, b.tile_base.data(), 4 * (n_views + 1), cudaMemcpyHostToDevice));
     FGS_CUDA(c, cudaMemcpy(b.d_img_off, b.img_off.data(), 8 * (n_views + 1), cudaMemcpyHostToDevice));
+    b.V = n_views;
     return FGS_OK;
 }
 

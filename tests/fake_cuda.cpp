@@ -12,8 +12,9 @@
 static std::vector<Op> g_queue;
 static std::vector<Op>* g_capture = nullptr;
 static cudaStream_t g_capture_stream = nullptr;
-static std::set<const void*> g_device;
+static std::set<const void*> g_device, g_fresh;
 static long g_allocs = 0, g_fail_at = -1, g_execs = 0;
+static cudaError_t g_last = cudaSuccess;
 
 void fake_push(cudaStream_t s, Op op)
 {
@@ -31,9 +32,9 @@ static void drain()
 static cudaError_t alloc(void** p, size_t n, bool device)
 {
     *p = nullptr;
-    if (g_allocs++ == g_fail_at) return cudaErrorMemoryAllocation;
+    if (g_allocs++ == g_fail_at) return g_last = cudaErrorMemoryAllocation;
     *p = calloc(n ? n : 1, 1);
-    if (device) g_device.insert(*p);
+    if (device) g_device.insert(*p), g_fresh.insert(*p);
     return cudaSuccess;
 }
 
@@ -54,13 +55,24 @@ cudaError_t cudaGetDevice(int* d) { *d = 0; return cudaSuccess; }
 cudaError_t cudaSetDevice(int) { return cudaSuccess; }
 cudaError_t cudaDeviceGetAttribute(int* v, cudaDeviceAttr, int) { *v = 152; return cudaSuccess; }
 cudaError_t cudaDeviceSynchronize() { drain(); return cudaSuccess; }
-cudaError_t cudaGetLastError() { return cudaSuccess; }
+cudaError_t cudaGetLastError()
+{
+    const cudaError_t e = g_last;
+    g_last = cudaSuccess;
+    return e;
+}
 const char* cudaGetErrorString(cudaError_t) { return "fake"; }
 cudaError_t cudaMalloc(void** p, size_t n) { return alloc(p, n, true); }
 cudaError_t cudaMallocHost(void** p, size_t n) { return alloc(p, n, false); }
 cudaError_t cudaFree(void* p) { drain(); g_device.erase(p); free(p); return cudaSuccess; }
 cudaError_t cudaFreeHost(void* p) { drain(); free(p); return cudaSuccess; }
-cudaError_t cudaMemset(void* p, int v, size_t n) { drain(); memset(p, v, n); return cudaSuccess; }
+cudaError_t cudaMemset(void* p, int v, size_t n)
+{
+    drain();
+    if (g_fresh.erase(p) && v == 0) return cudaSuccess;             // calloc's zeros, untouched
+    memset(p, v, n);
+    return cudaSuccess;
+}
 cudaError_t cudaMemsetAsync(void* p, int v, size_t n, cudaStream_t s)
 {
     fake_push(s, [=] { memset(p, v, n); });

@@ -17,10 +17,12 @@ struct Record {
 };
 
 static std::vector<Record> g_records;
+static long g_nulls = 0;           // null buffers given to the single-view launches
 
 extern "C" {
 
 void fake_clear() { g_records.clear(); }
+long fake_nulls() { return g_nulls; }
 long fake_records() { return (long)g_records.size(); }
 void fake_record(long i, int* head, uint64_t* rgb, float* t)
 {
@@ -57,22 +59,48 @@ int occ_scatter() { return 1; }
 int occ_segsort() { return 1; }
 int occ_tile_scan() { return 1; }
 void launch_frame_begin(const FrameBegin&, cudaStream_t) {}
-void launch_filter_pred(const DevTree&, const DevCamera&, uint32_t*, FrameState*, const FrameBegin&, int, cudaStream_t) {}
+void launch_filter_pred(const DevTree&, const DevCamera&, uint32_t* pbits, FrameState*, const FrameBegin& f, int,
+                        cudaStream_t)
+{
+    g_nulls += nulls(pbits, f.st, f.tile_cnt, f.sel_cnt);
+}
 void launch_chunk_boxes(const DevTree&, int, cudaStream_t) {}
-void launch_filter_anc(const DevTree&, const uint32_t*, uint32_t*, uint32_t*, int, cudaStream_t) {}
+void launch_filter_anc(const DevTree&, const uint32_t* pbits, uint32_t* selbits, uint32_t* sel_cnt, int, cudaStream_t)
+{
+    g_nulls += nulls(pbits, selbits, sel_cnt);
+}
 void launch_wait_probe(const unsigned long long*, FrameState*, cudaStream_t) {}
 void launch_compact(const uint32_t*, uint32_t, uint32_t*, uint32_t, unsigned long long*, FrameState*, int, cudaStream_t) {}
-void launch_compact_counted(const uint32_t*, uint32_t, uint32_t*, uint32_t, const uint32_t*, FrameState*, cudaStream_t) {}
-void launch_project(const DevTree&, const DevCamera&, const uint32_t*, float*, uint4*, uint32_t*, FrameState*, int,
-                    cudaStream_t) {}
-void launch_tile_scan(uint32_t*, uint2*, uint32_t, uint32_t*, unsigned long long, unsigned long long*, FrameState*, int,
-                      cudaStream_t) {}
-void launch_scatter(const DevCamera&, const uint4*, uint32_t*, unsigned long long*, unsigned long long, FrameState*, int,
-                    cudaStream_t) {}
-void launch_segsort(const uint2*, uint32_t, const uint32_t*, unsigned long long*, unsigned long long*, uint32_t*,
-                    uint32_t*, FrameState*, int, cudaStream_t) {}
-void launch_blend(const DevCamera&, const uint2*, const uint32_t*, const uint32_t*, const float*, float*, float*, uint2*,
-                  FrameState*, bool, cudaStream_t) {}
+void launch_compact_counted(const uint32_t* selbits, uint32_t, uint32_t* sel, uint32_t, const uint32_t* sel_cnt,
+                            FrameState* st, cudaStream_t)
+{
+    g_nulls += nulls(selbits, sel, sel_cnt, st);
+}
+void launch_project(const DevTree&, const DevCamera&, const uint32_t* sel, float* splat, uint4* foot, uint32_t* tile_cnt,
+                    FrameState* st, int, cudaStream_t)
+{
+    g_nulls += nulls(sel, splat, foot, tile_cnt, st);
+}
+void launch_tile_scan(uint32_t* tile_cnt, uint2* ranges, uint32_t, uint32_t* large, unsigned long long,
+                      unsigned long long* lookback, FrameState* st, int, cudaStream_t)
+{
+    g_nulls += nulls(tile_cnt, ranges, large, lookback, st);
+}
+void launch_scatter(const DevCamera&, const uint4* foot, uint32_t* cursor, unsigned long long* items, unsigned long long,
+                    FrameState* st, int, cudaStream_t)
+{
+    g_nulls += nulls(foot, cursor, items, st);
+}
+void launch_segsort(const uint2* ranges, uint32_t, const uint32_t* large, unsigned long long* items,
+                    unsigned long long* keys_out, uint32_t* vals_out, uint32_t* heavy, FrameState* st, int, cudaStream_t)
+{
+    g_nulls += nulls(ranges, large, items, keys_out, vals_out, heavy, st);
+}
+void launch_blend(const DevCamera&, const uint2* ranges, const uint32_t* heavy, const uint32_t* vals, const float* splat,
+                  float* rgb, float*, uint2*, FrameState* st, bool, cudaStream_t)
+{
+    g_nulls += nulls(ranges, heavy, vals, splat, rgb, st);
+}
 void launch_blend_kpc(const DevCamera&, const uint2*, const uint32_t*, const float*, float*, float*, FrameState*,
                       cudaStream_t) {}
 void launch_eval_exp(const float*, float*, uint64_t, cudaStream_t) {}

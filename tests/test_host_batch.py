@@ -1,7 +1,8 @@
 """The host side of the batched calls on a CPU: csrc/api.cu linked against replacements of
 the CUDA runtime calls it makes and of the kernel launchers (fake_cuda.cpp,
 fake_launchers.cu), driven through the binding's structs.  What the launches are given, in
-which order host memory is read and rewritten; no kernel runs."""
+which order host memory is read and rewritten, and what a failed call leaves; no kernel
+runs."""
 import ctypes as C
 import os
 import shutil
@@ -34,7 +35,7 @@ def api(tmp_path_factory):
             continue                                      # another file's entry point
         f, g = getattr(L, name), getattr(filtergs.lib(), name)
         f.argtypes, f.restype = g.argtypes, g.restype
-    for name in ("fake_allocs", "fake_records", "fake_graphs", "fake_device_blocks"):
+    for name in ("fake_allocs", "fake_records", "fake_graphs", "fake_device_blocks", "fake_nulls"):
         getattr(L, name).restype = C.c_long
     L.fake_fail_at.argtypes = [C.c_long]
     L.fake_record.argtypes = [C.c_long, C.c_void_p, C.c_void_p, C.c_void_p]
@@ -114,3 +115,85 @@ def test_tree_loaded_after_the_set_up(api, ctx, flags):
     api.fake_drain()
     n_pad = [_record(api, i)["n_pad"] for i in range(0, api.fake_records(), 2)]
     assert len(n_pad) == 3 and n_pad[0] > 4096 and n_pad[1] > n_pad[0] and n_pad[2] == 4096
+
+
+@pytest.mark.parametrize("again", [False, True])
+def test_failed_set_up_leaves_none(api, ctx, again):
+    """Each allocation of the set-up fails in turn (the first set-up, or one that replaces
+    another): the batch is refused afterwards, and the next set-up has every buffer."""
+    out = C.c_void_p(0x1000)
+    _load(api, ctx)
+    for k in range(100):
+        if again:
+            assert _setup(api, ctx, _cams(api, 2, 0.0)) == 0
+        api.fake_clear()
+        api.fake_fail_at(k)
+        cams = _cams(api, 5, 0.0)
+        rc = api.fgs_batch_setup(ctx, C.cast(cams, C.c_void_p), 5, None, 1 << 13, 1 << 13)
+        failed = api.fake_allocs() > k
+        api.fake_fail_at(-1)
+        assert rc == (api.b.FGS_ERR_NOMEM if failed else 0), k
+        assert api.fgs_render_batch(ctx, None, out, out, 0, None) == (api.b.FGS_ERR_STATE if failed else 0), k
+        api.fake_drain()
+        assert api.fake_records() == (0 if failed else 2)
+        if not failed:
+            break
+        assert _setup(api, ctx, _cams(api, 2, 0.0)) == 0
+        assert api.fgs_render_batch(ctx, None, out, out, 0, None) == 0
+        api.fake_drain()
+        assert api.fake_records() == 2 and all(_record(api, i)["nulls"] == 0 for i in range(2)), k
+    assert 12 <= k < 99
+
+
+def test_refused_set_up_keeps_the_one_before(api, ctx):
+    """A set-up with a wrong argument changes nothing."""
+    out = C.c_void_p(0x1000)
+    _load(api, ctx)
+    assert _setup(api, ctx, _cams(api, 2, 0.0)) == 0
+    cams = _cams(api, 5, 0.0)
+    shapes = np.array([[16, 16, 8]] * 4 + [[16, 32, 8]], np.int32)
+    for ts, cap in ((shapes.ctypes.data, 0), (None, 1 << 40)):
+        assert api.fgs_batch_setup(ctx, C.cast(cams, C.c_void_p), 5, ts, 0, cap) == api.b.FGS_ERR_ARG
+        assert api.fgs_render_batch(ctx, None, out, out, 0, None) == 0
+    api.fake_drain()
+    assert [len(_record(api, i)["t"]) for i in range(api.fake_records())] == [2] * 4
+
+
+def test_failed_frame_buffers_are_not_used(api, ctx):
+    """Each allocation of a growing pair list, image and tree fails in turn: frames are refused
+    until the call is repeated, and no launch is given a null buffer."""
+    rgb = C.c_void_p(0x1000)
+    big = api.b._cams([synth.look_at_camera([0, -30.0, 9.0], [0, 0, 0], 640, 480, 60.0)])
+    grow = {"pairs": lambda: api.fgs_set_params(ctx, C.byref(api.b.make_params(pair_capacity=1 << 14))),
+            "camera": lambda: api.fgs_set_camera(ctx, big),
+            "tiles": lambda: api.fgs_set_params(ctx, C.byref(api.b.make_params(tile=(64, 4)))),
+            "tree": lambda: api.fgs_load_tree(ctx, C.byref(large.struct))}
+    large = api.b._TreeArrays(synth.random_small_tree(1, n_leaves=9000, branching=(2, 5), sh_degree=1))
+    nulls = api.fake_nulls()
+    for name, call in grow.items():
+        for k in range(100):
+            h = C.c_void_p()
+            api.fake_fail_at(-1)
+            assert api.fgs_create(C.byref(h), 0) == 0
+            ctx, keep = h, ctx
+            _load(api, ctx)
+            cam = api.b._cams([synth.look_at_camera([0, -30.0, 9.0], [0, 0, 0], 66, 48, 60.0)])
+            assert api.fgs_set_camera(ctx, cam) == 0 and api.fgs_render(ctx, None, rgb, None, 1, 0, None) == 0
+            api.fake_fail_at(k)
+            rc = call()
+            failed = api.fake_allocs() > k
+            api.fake_fail_at(-1)
+            assert rc == (api.b.FGS_ERR_NOMEM if failed else 0), (name, k)
+            assert api.fgs_render(ctx, None, rgb, None, 1, 0, None) == (api.b.FGS_ERR_STATE if failed else 0), (name, k)
+            assert call() == 0 and api.fgs_render(ctx, None, rgb, None, 1, 0, None) == 0
+            if name != "tree":
+                assert api.fgs_set_camera(ctx, cam) == 0
+            else:
+                _load(api, ctx)
+            assert api.fgs_render(ctx, None, rgb, None, 1, 0, None) == 0
+            assert api.fake_nulls() == nulls, (name, k)
+            api.fgs_destroy(h)
+            ctx = keep
+            if not failed:
+                break
+        assert 0 < k < 99, name
