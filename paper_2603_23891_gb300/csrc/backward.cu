@@ -385,8 +385,12 @@ __device__ __forceinline__ void blend_bwd_walk(const DevCamera& cam, uint32_t ti
                     const float p = exp_poly_neg(n, t);
                     return fm(cv.x, fm(p, __uint_as_float((t << 23) + (127u << 23))));
                 };
-                const f32x2 qd = fma2(dC2, dup2(cv.w), fma2(dC1, dup2(cv.z), mul2(dC0, dup2(cv.y))));
+                // dL/dC . colour; a pixel that does not apply the entry keeps D (0 times an
+                // infinite colour would not be 0)
+                f32x2 qd = fma2(dC2, dup2(cv.w), fma2(dC1, dup2(cv.z), mul2(dC0, dup2(cv.y))));
                 if constexpr (kTwo) {
+                    const float2 q = unpack2(qd);
+                    qd = pack2(h0 ? q.x : 0.0f, h1 ? q.y : 0.0f);
                     const float2 n = *reinterpret_cast<const float2*>(&W.n[at][park]);
                     const float r0 = alpha1(n.x), r1 = alpha1(n.y);
                     const f32x2 al = pack2(h0 ? fminf(r0, 0.99f) : 0.0f, h1 ? fminf(r1, 0.99f) : 0.0f);
@@ -400,7 +404,7 @@ __device__ __forceinline__ void blend_bwd_walk(const DevCamera& cam, uint32_t ti
                         *reinterpret_cast<f32x2*>(&W.w[at][park]) = w;
                         // a clamped alpha does not move
                         *reinterpret_cast<float2*>(&W.g[at][park]) =
-                            make_float2(r0 < 0.99f ? gp.x : 0.0f, r1 < 0.99f ? gp.y : 0.0f);
+                            make_float2(h0 && r0 < 0.99f ? gp.x : 0.0f, h1 && r1 < 0.99f ? gp.y : 0.0f);
                     }
                 } else {
                     const float r0 = alpha1(W.n[at][park]);
@@ -412,7 +416,7 @@ __device__ __forceinline__ void blend_bwd_walk(const DevCamera& cam, uint32_t ti
                         W.g[at][park] = r0 < 0.99f ? (t * q0 - iom * d) * al : 0.0f;
                     }
                     T = pack2(t, 0.0f);
-                    D = pack2(fmaf(w, q0, d), 0.0f);
+                    D = pack2(h0 ? fmaf(w, q0, d) : d, 0.0f);
                 }
             }
             __syncwarp();
