@@ -297,7 +297,7 @@ __device__ __forceinline__ void blend_bwd_walk(const DevCamera& cam, uint32_t ti
             const float4* g = reinterpret_cast<const float4*>(splat + (size_t)m * kSplatStride);
             const float4 g0 = __ldg(g), g1 = __ldg(g + 1), g2 = __ldg(g + 2);
             S.r0[tid] = g0;
-            S.r1[tid] = g1;
+            S.r1[tid] = staged_r1(g1);
             S.r2[tid] = g2;
             S.mask[tid] = (uint16_t)walk_mask(cam, tx0, ty0, g0.x, g0.y, g0.z, g0.w, g1.x, g1.y);
         }

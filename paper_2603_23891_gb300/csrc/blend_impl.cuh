@@ -71,6 +71,14 @@ __device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b)
     return r;
 }
 
+// A record's {C, lthr, alpha0, depth} as it is staged: no power below -87 passes the skip
+// test, where exp is 0 and the entry would change nothing (exp_poly_neg's range).
+__device__ __forceinline__ float4 staged_r1(float4 r)
+{
+    r.y = fmaxf(r.y, -87.0f);
+    return r;
+}
+
 // Leading zeros; all ones for 0.
 __device__ __forceinline__ uint32_t clz_or_ones(uint32_t v)
 {
@@ -264,7 +272,9 @@ __device__ __forceinline__ void blend_walk(const DevCamera& cam, uint32_t tile, 
 
     uint32_t mask = 0u;          // window: 16 bits a group of kLanes entries, the older in the upper half
     uint32_t par = 0u;           // the older group's half of the window slots: 0 or kLanes
-    bool careful = false;        // a colour or a coefficient is not finite (or huge)
+    // a colour or a coefficient is not finite (or huge), or an applied alpha may not be normal
+    // (an opacity that its logarithm, and so the threshold, does not describe)
+    bool careful = false;
     uint32_t c_steps = 0, c_evals = 0, c_hits = 0, c_active = 0, c_proc = 0, c_old = 0, c_new = 0;
 
     // the lane's next entry out of the window: its slot, and which pixels it applies to
@@ -304,14 +314,14 @@ __device__ __forceinline__ void blend_walk(const DevCamera& cam, uint32_t tile, 
         mask &= live;
     };
     // apply the window's entries, two a turn, until no lane has one left under `gate`;
-    // `care`: colours and powers may be infinite or NaN (0 times one is not 0)
+    // `care`: colours and powers may be infinite or NaN (0 times one is not 0), alpha subnormal
     auto apply = [&](uint32_t gate, auto care) {
         constexpr bool kCare = decltype(care)::value;
         // alpha for parked power n, 0 where the entry is not applied
         auto alpha1 = [&](float n, float a0, bool h) {
             uint32_t t;
             const float p = exp_poly_neg(n, t);
-            // alpha0 p 2^k: an applied alpha is normal, so 2^k can go into the exponent
+            // alpha0 p 2^k: a normal alpha takes 2^k into its exponent
             const float al = kCare ? fm(a0, fm(p, __uint_as_float((t << 23) + (127u << 23))))
                                    : __uint_as_float((t << 23) + __float_as_uint(fm(a0, p)));
             return h ? fminf(al, 0.99f) : 0.0f;
@@ -412,11 +422,13 @@ __device__ __forceinline__ void blend_walk(const DevCamera& cam, uint32_t tile, 
             const float4* g = reinterpret_cast<const float4*>(splat + (size_t)m * kSplatStride);
             const float4 g0 = __ldg(g), g1 = __ldg(g + 1), g2 = __ldg(g + 2);
             S.r0[tid] = g0;
-            S.r1[tid] = g1;
+            S.r1[tid] = staged_r1(g1);
             S.r2[tid] = g2;
-            S.mask[tid] = (uint16_t)walk_mask(cam, tx0, ty0, g0.x, g0.y, g0.z, g0.w, g1.x, g1.y);
-            odd = !(fabsf(g2.x) + fabsf(g2.y) + fabsf(g2.z) + fabsf(g0.x) + fabsf(g0.y) + fabsf(g0.z) + fabsf(g0.w) +
-                        fabsf(g1.x) <= 1.0e9f);
+            const uint32_t mask_tid = walk_mask(cam, tx0, ty0, g0.x, g0.y, g0.z, g0.w, g1.x, g1.y);
+            S.mask[tid] = (uint16_t)mask_tid;
+            odd = mask_tid && !(fabsf(g2.x) + fabsf(g2.y) + fabsf(g2.z) + fabsf(g0.x) + fabsf(g0.y) + fabsf(g0.z) +
+                                        fabsf(g0.w) + fabsf(g1.x) <= 1.0e9f &&
+                                g1.y >= -20.0f && g1.z >= 1.0e-20f);
         }
         const bool last = s0 + kC >= e;
         if (s0 + kC + tid < e) m = __ldg(vals + s0 + kC + tid);
@@ -598,7 +610,7 @@ __device__ __forceinline__ void blend_walk_kpc(const DevCamera& cam, uint32_t ti
             const float4* g = reinterpret_cast<const float4*>(splat + (size_t)m * kSplatStride);
             const float4 g0 = __ldg(g), g1 = __ldg(g + 1);
             S.r0[tid] = g0;
-            S.r1[tid] = g1;
+            S.r1[tid] = staged_r1(g1);
             my_mask = walk_mask(cam, tx0, ty0, g0.x, g0.y, g0.z, g0.w, g1.x, g1.y);
             S.mask[tid] = (uint16_t)my_mask;
 #pragma unroll
