@@ -177,14 +177,6 @@ struct BwdSmem {
     BwdWarp w[blendk::kWalkWarps];
 };
 
-// 1 / x for x in [0.01, 1]: the approximate reciprocal and one Newton step.
-__device__ __forceinline__ float rcp1(float x)
-{
-    float r;
-    asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
-    return fmaf(r, fmaf(-x, r, 1.0f), r);
-}
-
 // Gradient walk of a tile (kLanes = 8) or its half `part` (kLanes = 16), laid out as the
 // forward's walk (blend_walk): lanes, blocks, chunks, lists and the test are the same,
 // the chunks and the lists' groups of kLanes entries taken from the last to the first.

@@ -151,6 +151,15 @@ __device__ __forceinline__ float exp_cw(float x)
     return exp_nonpos(x);
 }
 
+// 1 / x for x in [1/128, 1]: the approximate reciprocal and one Newton step with fused
+// multiply-adds, correctly rounded for every x there (as __frcp_rn, without its branch).
+__device__ __forceinline__ float rcp1(float x)
+{
+    float r;
+    asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return fmaf(r, fmaf(-x, r, 1.0f), r);
+}
+
 // Screen-space view of one node: camera-space centre, frustum test and the
 // 2D covariance J W Sigma W^T J^T + 0.3 I (EWA), larger eigenvalue.
 struct NodeView {
