@@ -754,7 +754,7 @@ __device__ __forceinline__ void walk_grid(uint32_t bid, uint32_t n_ctas, uint32_
     } else {
         const uint32_t tile = bid - n_half;
         const uint2 rg = ranges[tile];
-        if (rg.y - rg.x > split_pairs(st->n_pairs)) return;
+        if (rg.y - rg.x > st->split) return;
         whole(tile, rg);
     }
 }

@@ -86,7 +86,8 @@ struct FrameState {
     uint32_t tickets[16];      // dynamic tile counters (one per kernel use)
     int32_t status;            // latched error (0 = ok)
     uint32_t status_info;
-    uint32_t reserved0;
+    uint32_t n_used;                      // tiles with pairs
+    uint32_t split;                       // pairs above which the blend splits a tile (the sort's split_pairs)
     unsigned long long blend_entries;     // test steps of the list walk (counting frames only)
     unsigned long long blend_evals;       // pixel-Gaussian evaluations (lanes not yet stopped)
     unsigned long long blend_hits;        // evaluations that reached the alpha / T update
@@ -319,9 +320,17 @@ __device__ __forceinline__ void ewa_cov2d(const DevCamera& cam, float vz, float 
 // 168 / 133 / 113 us where one tile holds 3,473 of 1.08M pairs, 148 / 152 / 131 us for
 // 2,299 of 1.44M, 111 / 113 / 111 us for 1,834 of 1.12M.  By the definition there are
 // fewer than kSplitTiles of them; in a small frame most tiles with pairs are.
-__device__ __forceinline__ uint32_t split_pairs(unsigned long long n_pairs)
+// Above 3/5 of the resident CTAs in tiles with pairs, a tile is split only if it also holds a
+// quarter more than their mean: whole tiles of even load then fill one wave, their halves
+// more than one (evenly covered frames, 803 pairs in each of 836 tiles: blend 82 us with all
+// of them split, 66 so; 1,086 in 576: 84, 78; below, the halves are faster: 1,236 in 493:
+// 80, 86; one wave of halves: 1,307 in 448: 60).
+__device__ __forceinline__ uint32_t split_pairs(const FrameState* st)
 {
-    return (uint32_t)(n_pairs / kSplitTiles);
+    const uint32_t n_pairs = (uint32_t)st->n_pairs, used = st->n_used;     // (the scan's count saturates at 2^32 - 1)
+    const uint32_t share = n_pairs / kSplitTiles;
+    if (used <= kSplitTiles * 3 / 5) return share;
+    return max(share, (uint32_t)__fdiv_rn(__fmul_rn(1.25f, (float)n_pairs), (float)used));
 }
 inline int split_slots(int n_tiles) { return n_tiles < (int)kSplitTiles ? n_tiles : (int)kSplitTiles; }
 
@@ -435,6 +444,7 @@ __device__ __forceinline__ void frame_begin(const FrameBegin& f, int tid, int n_
         st->epoch = st->epoch + 1;
         st->M = 0;
         st->n_pairs = 0;
+        st->n_used = 0;
         st->blend_entries = 0;
         st->blend_evals = 0;
         st->blend_hits = 0;

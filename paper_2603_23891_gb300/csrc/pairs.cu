@@ -784,7 +784,7 @@ __global__ void __launch_bounds__(kScanThreads) tile_scan_kernel(uint32_t* __res
         if (incl == 0xFFFFFFFFu) off = 0xFFFFFFFFu;          // saturated: clamps to the capacity below
         // each tile's range [first, last) clamped to the capacity, its scatter cursor,
         // and which tiles the block sort takes
-        uint32_t big = 0u;
+        uint32_t big = 0u, used = 0u;
 #pragma unroll
         for (int i = 0; i < kScanItems; ++i) {
             const uint32_t t = t0 + i;
@@ -796,11 +796,12 @@ __global__ void __launch_bounds__(kScanThreads) tile_scan_kernel(uint32_t* __res
                 tile_cnt[t] = a;
             }
             if (t < n_tiles && e - a > (uint32_t)kSegSmall) big |= 1u << i;
+            used += t < n_tiles && e > a;
             off = end;
         }
         // the block's list entries by one reservation (one a warp and tile in turn took
         // eight round trips, half of the kernel: 8.4 -> 6 us on 8,160 tiles)
-        uint32_t bi = __popc(big);
+        uint32_t bi = __popc(big) | used << 16;                // (and the tiles with pairs, in the upper half)
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
             const uint32_t u = __shfl_up_sync(0xffffffffu, bi, o);
@@ -815,9 +816,12 @@ __global__ void __launch_bounds__(kScanThreads) tile_scan_kernel(uint32_t* __res
             if (w < (int)warp) boff += tw;
             btotal += tw;
         }
-        if (tid == 0 && btotal) s_prefix = atomicAdd(&st->tickets[kTicketLarge], btotal);
+        if (tid == 0 && btotal) {
+            atomicAdd(&st->n_used, btotal >> 16);
+            s_prefix = atomicAdd(&st->tickets[kTicketLarge], btotal & 0xFFFFu);
+        }
         __syncthreads();
-        uint32_t slot = s_prefix + boff + bi - __popc(big);
+        uint32_t slot = s_prefix + ((boff + bi) & 0xFFFFu) - __popc(big);
 #pragma unroll
         for (int i = 0; i < kScanItems; ++i)
             if ((big >> i) & 1u) large[slot++] = t0 + i;
@@ -962,7 +966,8 @@ __global__ void __launch_bounds__(kSegThreads, 4) segsort_kernel(const uint2* __
     // large buckets first: one block each; a block's first bucket is its index,
     // later ones come from a ticket counter
     const uint32_t n_large = st->tickets[kTicketLarge];
-    const uint32_t split = split_pairs(st->n_pairs);
+    const uint32_t split = split_pairs(st);
+    if (blockIdx.x == 0 && threadIdx.x == 0) st->split = split;
     bool first = true;
     for (;;) {
         if (threadIdx.x == 0)
