@@ -24,7 +24,7 @@
 //    instead of up to four: 49 -> 34 us for 1.13M pairs of 1M blobs at 1080p, 75 ->
 //    45 us for a city frame with buckets above kSegSmem; issue and barrier bound),
 //    and the runs of equal ones, which keep the scatter's order, are ordered
-//    where they lie; a bucket with a run longer than kTieRun is sorted by every bit.
+//    where they lie; a bucket whose leading bits are crowded is sorted by every bit.
 //    The sorted bucket is written as keys
 //    (tile << 32 | depth bits) and values (rank).
 #include "pairs_impl.cuh"
@@ -318,12 +318,18 @@ __device__ __forceinline__ void block_min_max(uint32_t lo, uint32_t hi, RadixSme
 // binary32 values, so 65,536 steps between its nearest and farthest put one to a few
 // Gaussians in each).  A run of equal sorted bits keeps the scatter's order; it is put
 // in (depth, rank) order where it lies by the thread holding its first element, by
-// insertion, if it is at most kTieRun long; a longer one sends the bucket to the next
-// slower sort.
+// insertion, if it is at most kTieRun long.  Depths that crowd together (a wall seen
+// head-on behind one near Gaussian) would leave longer runs; such a bucket is sorted by
+// all bits: the first pass's digit counts show them before anything has been moved, a
+// run's elements having the same digit.  (667K pairs of a flat scene, 920 tiles: 45 us;
+// found after the two passes and sorted by the network 90, by all bits always 31.)
 constexpr uint32_t kTieRun = 32;
 constexpr uint32_t kCoarseBits = 16;
+// The most items of one digit that do not count as crowded: twice the even share, and 12 (a
+// run of 16 takes its thread about as long as two more passes take the block).
+__device__ __forceinline__ uint32_t crowd_limit(uint32_t n) { return 12u + n / 128u; }
 
-__device__ __forceinline__ uint32_t coarse_shift(uint32_t bl) { return bl > kCoarseBits ? bl - kCoarseBits : 0u; }
+__device__ __forceinline__ uint32_t coarse_shift(uint32_t bl, uint32_t bits = kCoarseBits) { return bl > bits ? bl - bits : 0u; }
 
 // Order the run that starts at i (the element before it has other leading bits);
 // false, changing nothing, for a run longer than kTieRun.  Only this thread writes the
@@ -336,6 +342,18 @@ __device__ __forceinline__ bool sort_run(uint32_t* keys, uint32_t* vals, uint32_
     while (j < n && (keys[j] - base) >> s0 == k) {
         if (j - i >= kTieRun) return false;
         ++j;
+    }
+    if (s0 == 0u) {                                        // equal depths: by rank
+        for (uint32_t a = i + 1; a < j; ++a) {
+            const uint32_t v = vals[a];
+            uint32_t b = a;
+            while (b > i && vals[b - 1] > v) {
+                vals[b] = vals[b - 1];
+                --b;
+            }
+            vals[b] = v;
+        }
+        return true;
     }
     for (uint32_t a = i + 1; a < j; ++a) {
         const uint32_t x = keys[a], v = vals[a];
@@ -373,16 +391,17 @@ __device__ __forceinline__ bool sort_run64(unsigned long long* items, uint32_t b
     return true;
 }
 
-// A block sorts n <= 256 I items of one tile by depth (its leading bits if coarse)
+// A block sorts n <= 256 I items of one tile by depth (its leading bits if those do)
 // with a stable LSD radix sort, items held in registers and exchanged through shared
 // memory (skeys / svals) after every pass.  Item i of the input order is item it, lane
 // L of warp w with i = (w I + it) 32 + L.  Then each run of equal sorted bits is put
-// in order where it lies.  If a run is longer than kTieRun, false is returned and
-// nothing is written; otherwise the sorted pairs are written and true is returned.
+// in order where it lies.  If a run is longer than kTieRun (depths equal to the last
+// bit), false is returned and nothing is written; otherwise the sorted pairs are written
+// and true is returned.
 template <int I>
 __device__ bool block_radix_bucket(const unsigned long long* items, uint32_t n, uint32_t tile,
                                    unsigned long long* keys_out, uint32_t* vals_out, uint32_t* skeys,
-                                   uint32_t* svals, RadixSmem& R, bool coarse)
+                                   uint32_t* svals, RadixSmem& R)
 {
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     uint32_t key[I], val[I];
@@ -400,12 +419,17 @@ __device__ bool block_radix_bucket(const unsigned long long* items, uint32_t n, 
     }
     block_min_max(lo, hi, R);
     const uint32_t base = R.lo, bl = 32u - (uint32_t)__clz((int)(R.hi - R.lo));
-    const uint32_t s0 = coarse ? coarse_shift(bl) : 0u;
+    uint32_t s0 = coarse_shift(bl);
     for (uint32_t shift = s0; shift < bl; shift += 8) {
         uint32_t d[I], rank[I];
 #pragma unroll
         for (int it = 0; it < I; ++it) d[it] = ((key[it] - base) >> shift) & 0xFFu;
         rank_chunk<I>(d, n, R, rank);
+        if (s0 && shift == s0 && __syncthreads_or(R.dcnt[tid] > crowd_limit(n))) {
+            s0 = 0u;                                       // crowded depths: by all bits
+            shift = 0u - 8u;
+            continue;
+        }
         R.dbase[tid] = block_excl_scan(R.dcnt[tid], R.tmp);
         __syncthreads();
 #pragma unroll
@@ -455,15 +479,19 @@ __device__ bool block_radix_bucket(const unsigned long long* items, uint32_t n, 
 // A block sorts a bucket of any size by (depth, rank) with stable LSD radix passes
 // over 8-bit digits of the 64-bit items, each pass a histogram sweep and a scatter
 // sweep over chunks of 256 I items, between the bucket (a) and the tile's slots of the
-// key output (b) as scratch.  First only the leading bits of the depths (two passes),
-// and each run of equal ones put in order where it lies; if a run is longer than
-// kTieRun the sort is repeated over every byte in which the items differ (rank bytes
-// first; the input order does not matter, (depth, rank) being unique).  The sorted
-// pairs are written to keys_out (which is b) and vals_out.
+// key output (b) as scratch.  First by the leading bits of the depths (two passes; three
+// from kManyItems on, where 65,536 steps would leave long runs), or by all of them if
+// a digit of the first pass is crowded, and each run of equal ones put in order where it
+// lies; after a run longer than kTieRun by all bits of the depths, and if there still is
+// one (equal depths) by every byte in which the items differ (rank bytes first; the
+// input order does not matter, (depth, rank) being unique).  The sorted pairs are
+// written to keys_out (which is b) and vals_out.
+constexpr uint32_t kManyItems = 8192;
 constexpr int kRadixGlobalItems = 8;
-// One pass over bits [shift, shift + 8) of the items less `base`.
-__device__ void radix_global_pass(const unsigned long long* src, unsigned long long* dst, uint32_t n,
-                                  unsigned long long base, uint32_t shift, RadixSmem& R)
+// One pass over bits [shift, shift + 8) of the items less `base`.  Returns false, moving
+// nothing, if more than `most` items have the same digit.
+__device__ bool radix_global_pass(const unsigned long long* src, unsigned long long* dst, uint32_t n,
+                                  unsigned long long base, uint32_t shift, uint32_t most, RadixSmem& R)
 {
     constexpr int I = kRadixGlobalItems;
     constexpr uint32_t kChunk = 256u * I;
@@ -473,7 +501,9 @@ __device__ void radix_global_pass(const unsigned long long* src, unsigned long l
     __syncthreads();
     for (uint32_t i = tid; i < n; i += kSegThreads) atomicAdd(&R.dcnt[(uint32_t)((src[i] - base) >> shift) & 0xFFu], 1u);
     __syncthreads();
-    R.dbase[tid] = block_excl_scan(R.dcnt[tid], R.tmp);
+    const uint32_t count = R.dcnt[tid];
+    if (__syncthreads_or(count > most)) return false;
+    R.dbase[tid] = block_excl_scan(count, R.tmp);
     __syncthreads();
     // stable scatter, chunk by chunk in order
     for (uint32_t c0 = 0; c0 < n; c0 += kChunk) {
@@ -495,6 +525,7 @@ __device__ void radix_global_pass(const unsigned long long* src, unsigned long l
         R.dbase[tid] += R.dcnt[tid];
         __syncthreads();
     }
+    return true;
 }
 
 __device__ void block_radix_global(unsigned long long* a, unsigned long long* b, uint32_t n, uint32_t tile,
@@ -508,25 +539,42 @@ __device__ void block_radix_global(unsigned long long* a, unsigned long long* b,
         hi = max(hi, d);
     }
     block_min_max(lo, hi, R);
-    const uint32_t base = R.lo, bl = 32u - (uint32_t)__clz((int)(R.hi - R.lo)), s0 = coarse_shift(bl);
+    const uint32_t base = R.lo, bl = 32u - (uint32_t)__clz((int)(R.hi - R.lo));
+    uint32_t s0 = coarse_shift(bl, n < kManyItems ? kCoarseBits : kCoarseBits + 8u);
     unsigned long long* src = a;
     unsigned long long* dst = b;
-    auto pass = [&](unsigned long long from, uint32_t shift) {
-        radix_global_pass(src, dst, n, from, shift, R);
+    auto pass = [&](unsigned long long from, uint32_t shift, uint32_t most) {
+        if (!radix_global_pass(src, dst, n, from, shift, most, R)) return false;
         unsigned long long* t = src;
         src = dst;
         dst = t;
+        return true;
     };
-    for (uint32_t shift = s0; shift < bl; shift += 8) pass((unsigned long long)base << 32, 32u + shift);
-    // each run in order where it lies; a run longer than kTieRun: the full sort instead
-    bool long_run = false;
-    for (uint32_t i = tid; i + 1 < n; i += kSegThreads) {
-        const uint32_t k = ((uint32_t)(src[i] >> 32) - base) >> s0;
-        if (((uint32_t)(src[i + 1] >> 32) - base) >> s0 == k &&
-            (i == 0 || ((uint32_t)(src[i - 1] >> 32) - base) >> s0 != k))
-            long_run |= !sort_run64(src, base, s0, i, n);
+    // by bits [s0, bl) of the depths, then each run of equal ones in order; whether a run
+    // is too long
+    auto by_depth = [&]() {
+        const unsigned long long from = (unsigned long long)base << 32;
+        for (uint32_t shift = s0; shift < bl; shift += 8)
+            // (the first pass moves nothing when it finds the digits crowded: by all bits)
+            if (!pass(from, 32u + shift, s0 && shift == s0 ? crowd_limit(n) : n)) {
+                s0 = 0u;
+                shift = 0u - 8u;
+            }
+        bool long_run = false;
+        for (uint32_t i = tid; i + 1 < n; i += kSegThreads) {
+            const uint32_t k = ((uint32_t)(src[i] >> 32) - base) >> s0;
+            if (((uint32_t)(src[i + 1] >> 32) - base) >> s0 == k &&
+                (i == 0 || ((uint32_t)(src[i - 1] >> 32) - base) >> s0 != k))
+                long_run |= !sort_run64(src, base, s0, i, n);
+        }
+        return __syncthreads_or(long_run) != 0;
+    };
+    bool long_run = by_depth();
+    if (long_run && s0) {
+        s0 = 0u;
+        long_run = by_depth();
     }
-    if (__syncthreads_or(long_run)) {
+    if (long_run) {
         unsigned long long vor = 0ull, vand = ~0ull;
         for (uint32_t i = tid; i < n; i += kSegThreads) {
             vor |= src[i];
@@ -535,7 +583,7 @@ __device__ void block_radix_global(unsigned long long* a, unsigned long long* b,
         block_or_and(vor, vand, R);
         const unsigned long long diff = R.vor & ~R.vand;
         for (uint32_t shift = 0; shift < 64; shift += 8)
-            if (((diff >> shift) & 0xFFull) != 0ull) pass(0ull, shift);
+            if (((diff >> shift) & 0xFFull) != 0ull) pass(0ull, shift, n);
     }
     // src holds the sorted items; a slot of keys_out (= b) is read and then
     // rewritten by the same thread
@@ -545,11 +593,11 @@ __device__ void block_radix_global(unsigned long long* a, unsigned long long* b,
 
 // A warp sorts n <= 32 I items of one tile by (depth, rank), items in registers
 // (item it of lane L is element 32 it + L): stable LSD radix passes over the leading
-// bits of the depths, each ranking the digits with one ballot per digit bit and the
-// warp's 256 counters (hist), the items exchanged through the warp's buffer buf (32 I
-// slots); then each run of equal leading bits in order where it lies, and the pairs
-// written.  Returns false, writing nothing, if a run is longer than kTieRun (the
-// caller sorts the bucket by the bitonic network instead).
+// (or, if those are crowded, all) bits of the depths, each ranking the digits with one
+// ballot per digit bit and the warp's 256 counters (hist), the items exchanged through
+// the warp's buffer buf (32 I slots); then each run of equal sorted bits in order where
+// it lies, and the pairs written.  Returns false, writing nothing, if a run is longer
+// than kTieRun (the caller sorts the bucket by the bitonic network instead).
 template <int I>
 __device__ bool warp_radix_small(const unsigned long long* items, uint32_t n, uint32_t tile,
                                  unsigned long long* keys_out, uint32_t* vals_out, unsigned long long* buf,
@@ -569,7 +617,7 @@ __device__ bool warp_radix_small(const unsigned long long* items, uint32_t n, ui
     }
     const uint32_t base = __reduce_min_sync(0xffffffffu, lo);
     const uint32_t bl = 32u - (uint32_t)__clz((int)(__reduce_max_sync(0xffffffffu, hi) - base));
-    const uint32_t s0 = coarse_shift(bl);
+    uint32_t s0 = coarse_shift(bl);
     for (uint32_t shift = s0; shift < bl; shift += 8) {
 #pragma unroll
         for (int j = 0; j < 8; ++j) hist[lane * 8 + j] = 0u;
@@ -593,11 +641,18 @@ __device__ bool warp_radix_small(const unsigned long long* items, uint32_t n, ui
             rank[it] = base + __popc(peers & lt);
         }
         // exclusive scan of the 256 counters, 8 consecutive ones a lane
-        uint32_t c[8], sum = 0u;
+        uint32_t c[8], sum = 0u, top = 0u;
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
             c[j] = hist[lane * 8 + j];
             sum += c[j];
+            top = max(top, c[j]);
+        }
+        if (s0 && shift == s0 && __any_sync(0xffffffffu, top > crowd_limit(n))) {
+            s0 = 0u;                                       // crowded depths: by all bits
+            shift = 0u - 8u;
+            __syncwarp();
+            continue;
         }
         uint32_t incl = sum;
 #pragma unroll
@@ -984,13 +1039,10 @@ __global__ void __launch_bounds__(kSegThreads, 4) segsort_kernel(const uint2* __
         if (threadIdx.x == 0) list_heavy(n, split, t, heavy, st);
         if (n <= (uint32_t)kSegSmem) {
             uint32_t* sk = reinterpret_cast<uint32_t*>(s_items);
-            bool done = false;
-            // by the leading bits of the depth; by all of them; by the network
-            for (int coarse = 1; coarse >= 0 && !done; --coarse) {
-                if (n <= 512u) done = block_radix_bucket<2>(it, n, t, keys_out + r.x, vals_out + r.x, sk, sk + kSegSmem, s_radix, coarse);
-                else if (n <= 1024u) done = block_radix_bucket<4>(it, n, t, keys_out + r.x, vals_out + r.x, sk, sk + kSegSmem, s_radix, coarse);
-                else done = block_radix_bucket<8>(it, n, t, keys_out + r.x, vals_out + r.x, sk, sk + kSegSmem, s_radix, coarse);
-            }
+            bool done;
+            if (n <= 512u) done = block_radix_bucket<2>(it, n, t, keys_out + r.x, vals_out + r.x, sk, sk + kSegSmem, s_radix);
+            else if (n <= 1024u) done = block_radix_bucket<4>(it, n, t, keys_out + r.x, vals_out + r.x, sk, sk + kSegSmem, s_radix);
+            else done = block_radix_bucket<8>(it, n, t, keys_out + r.x, vals_out + r.x, sk, sk + kSegSmem, s_radix);
             if (!done) block_bitonic_any(s_items, it, n, t, keys_out + r.x, vals_out + r.x);
         } else {
             block_radix_global(it, keys_out + r.x, n, t, keys_out + r.x, vals_out + r.x, s_radix);
