@@ -198,16 +198,19 @@ __device__ __forceinline__ void project_walk(const DevTree& t, const uint32_t* _
         if (m >= M) f.z = 0u;
         const uint32_t emit = __ballot_sync(0xffffffffu, f.z > 0u);
         emitting += (uint32_t)__popc(emit);
-        // the SH rows of the emitting lanes: 16 bytes a lane and step, row by row
+        // the SH rows of the emitting lanes (in a small view of a large scene often none): 16
+        // bytes a lane and step, row by row
+        if (emit) {
 #pragma unroll
-        for (int i = 0; i < kQ; ++i) {
-            const uint32_t idx = (uint32_t)i * 32u + lane, r = idx / kQ, k = idx - r * kQ;
-            const uint32_t nr = __shfl_sync(0xffffffffu, n, r);
-            if ((emit >> r) & 1u)
-                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
-                                 (uint32_t)__cvta_generic_to_shared(rows + r * kStride + k)),
-                             "l"(t.sh + (size_t)nr * t.sh_stride + 4 * k)
-                             : "memory");
+            for (int i = 0; i < kQ; ++i) {
+                const uint32_t idx = (uint32_t)i * 32u + lane, r = idx / kQ, k = idx - r * kQ;
+                const uint32_t nr = __shfl_sync(0xffffffffu, n, r);
+                if ((emit >> r) & 1u)
+                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                                     (uint32_t)__cvta_generic_to_shared(rows + r * kStride + k)),
+                                 "l"(t.sh + (size_t)nr * t.sh_stride + 4 * k)
+                                 : "memory");
+            }
         }
         // direction to the colour; then the next entries' attributes
         float dx = at.q0.x - cam->campos[0], dy = at.q0.y - cam->campos[1], dz = at.q0.z - cam->campos[2];
