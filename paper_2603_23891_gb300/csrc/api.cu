@@ -133,7 +133,7 @@ struct fgs_ctx {
         float* splat = nullptr;
         uint4* foot = nullptr;
         unsigned long long *items = nullptr, *keys = nullptr, *lb_scan = nullptr;
-        uint32_t* sel_cnt = nullptr;              // selected entries per kBatchSelTileWords words
+        uint32_t* sel_cnt = nullptr;              // selected entries per counted tile
         uint32_t* vals = nullptr;
         uint2* ranges = nullptr;
         uint32_t *tile_cnt = nullptr, *large = nullptr, *heavy = nullptr;

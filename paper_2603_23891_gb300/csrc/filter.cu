@@ -340,9 +340,9 @@ __global__ void __launch_bounds__(256) compact_kernel(const uint32_t* __restrict
 // tile, kW words per thread, takes the tile's first slot as the sum of the counts of
 // the tiles before it, so no block waits on another (no look-back chain); then
 // popcounts, a block scan and a warp-cooperative bit expansion of each warp's words
-// (coalesced stores of ascending ids).  kW = 1 for one view; 4 for a batch, whose sums
-// over many more tiles would otherwise grow with their square (8 views of 12.5M nodes:
-// 45 us with the look-back kernel, 25 with this one).
+// (coalesced stores of ascending ids).  kW = 1 for one view; 4 or 16 for a batch
+// (batch_sel_shift), whose sums over many more tiles would otherwise grow with their square
+// (8 views of 12.5M nodes: 45 us with the look-back kernel, 27 with this one).
 template <int kW>
 __global__ void __launch_bounds__(256) compact_counted_kernel(const uint32_t* __restrict__ selbits,
                                                               uint32_t n_words, uint32_t* __restrict__ sel,
@@ -426,9 +426,9 @@ void launch_compact_counted(const uint32_t* selbits, uint32_t n_words, uint32_t*
 void launch_compact_counted_batch(const uint32_t* selbits, uint32_t n_words, uint32_t* sel, uint32_t cap,
                                   const uint32_t* sel_cnt, FrameState* st, cudaStream_t s)
 {
-    const int n_tiles = (int)((n_words + kBatchSelTileWords - 1) / kBatchSelTileWords);
-    launch_pdl(compact_counted_kernel<kBatchSelTileWords / 256>, n_tiles < 1 ? 1 : n_tiles, 256, 0, s, selbits, n_words,
-               sel, cap, sel_cnt, st);
+    const unsigned n_tiles = (unsigned)batch_sel_tiles(n_words);
+    const auto kernel = batch_sel_shift(n_words) == 10u ? compact_counted_kernel<4> : compact_counted_kernel<16>;
+    launch_pdl(kernel, n_tiles < 1 ? 1u : n_tiles, 256, 0, s, selbits, n_words, sel, cap, sel_cnt, st);
 }
 
 // One warp looks back from tile 1 at tile 0 with a tag whose low four bits
