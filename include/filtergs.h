@@ -332,10 +332,11 @@ int fgs_compact_selection_noalloc(const uint32_t* selbits, uint64_t n_words, uin
 
 /* Batched multi-view form (next form beside §3.2-§3.3's single view: many
  * views of uneven resolution per call).  Set-up for n_views (1..64) cameras
- * (host array): tile_shapes (may be NULL = the context's tile and blend warp
- * shape) holds {tile_w, tile_h, blend_warp_w} per view; sel_capacity / pair_capacity bound the selected
- * entries and Gaussian-tile pairs of the whole batch (0 = defaults: views x
- * nodes up to 64 Mi entries, 128 Mi pairs).  Allocates the batch buffers.
+ * (host array): tile_shapes (may be NULL = the context's tile shape) holds
+ * {tile_w, tile_h, blend_warp_w} per view (the last checked, without effect, as
+ * in fgs_params); sel_capacity / pair_capacity bound the selected entries and
+ * Gaussian-tile pairs of the whole batch (0 = defaults: views x nodes up to
+ * 64 Mi entries, 128 Mi pairs).  Allocates the batch buffers.
  * The batch keeps the context's tau_R, background and shrink mode as they are
  * at each fgs_render_batch call.  A tree loaded later is rendered with the same
  * set-up if it is no larger (node count rounded up to 4096); for a larger one

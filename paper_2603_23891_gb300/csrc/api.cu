@@ -121,7 +121,7 @@ struct fgs_ctx {
         int V = 0;
         uint32_t n_pad = 0;                       // nodes a view the buffers hold (the tree's at set-up)
         std::vector<fgs_camera> cams;
-        std::vector<int32_t> tile_w, tile_h, warp_w;
+        std::vector<int32_t> tile_w, tile_h;
         std::vector<uint32_t> tile_base;          // V + 1
         std::vector<unsigned long long> img_off;  // V + 1 (pixels)
         uint32_t total_tiles = 0;
@@ -312,11 +312,10 @@ DevCamera make_devcam(const fgs_ctx* c, bool force_shrink_off)
     d.tau = c->tau;
     d.ln_tau = c->ln_tau;
     std::memcpy(d.bg, c->params.bg, sizeof d.bg);
-    d.warp_shift = c->params.blend_warp_w == 4 ? 2 : 3;
     return d;
 }
 
-DevCamera make_devcam_for(const fgs_ctx* c, const fgs_camera& cam, int tile_w, int tile_h, int warp_w)
+DevCamera make_devcam_for(const fgs_ctx* c, const fgs_camera& cam, int tile_w, int tile_h)
 {
     DevCamera d{};
     std::memcpy(d.R, cam.R, sizeof d.R);
@@ -341,7 +340,6 @@ DevCamera make_devcam_for(const fgs_ctx* c, const fgs_camera& cam, int tile_w, i
     d.tau = c->tau;
     d.ln_tau = c->ln_tau;
     std::memcpy(d.bg, c->params.bg, sizeof d.bg);
-    d.warp_shift = warp_w == 4 ? 2 : 3;
     return d;
 }
 
@@ -1214,7 +1212,6 @@ int fgs_batch_setup(fgs_ctx* c, const fgs_camera* views, int n_views, const int3
         return fail(c, FGS_ERR_ARG, "views x nodes exceeds 2^32 selection entries");
     // everything is checked before the current set-up is touched
     std::vector<int32_t> tile_w(n_views, c->params.tile_w), tile_h(n_views, c->params.tile_h);
-    std::vector<int32_t> warp_w(n_views, c->params.blend_warp_w);
     if (tile_shapes) {
         for (int v = 0; v < n_views; ++v) {
             const int tw = tile_shapes[3 * v], th = tile_shapes[3 * v + 1];
@@ -1224,7 +1221,6 @@ int fgs_batch_setup(fgs_ctx* c, const fgs_camera* views, int n_views, const int3
                 return fail(c, FGS_ERR_ARG, "view %d: tile %dx%d / warp %d not supported", v, tw, th, ww);
             tile_w[v] = tw;
             tile_h[v] = th;
-            warp_w[v] = ww;
         }
     }
     const uint64_t sel_cap = sel_capacity ? sel_capacity : std::min<uint64_t>((uint64_t)n_views * c->tree.n_pad, 64ull << 20);
@@ -1240,7 +1236,6 @@ int fgs_batch_setup(fgs_ctx* c, const fgs_camera* views, int n_views, const int3
     b.cams.assign(views, views + n_views);
     b.tile_w = tile_w;
     b.tile_h = tile_h;
-    b.warp_w = warp_w;
     b.tile_base.assign(n_views + 1, 0);
     b.img_off.assign(n_views + 1, 0);
     for (int v = 0; v < n_views; ++v) {
@@ -1336,7 +1331,7 @@ int fgs_render_batch(fgs_ctx* c, void* stream, float* rgb_out, float* T_out, uin
     DeviceGuard g(c->device);
     cudaStream_t s = (cudaStream_t)stream;
     DevCamera cams[kMaxBatchViews];
-    for (int v = 0; v < b.V; ++v) cams[v] = make_devcam_for(c, b.cams[v], b.tile_w[v], b.tile_h[v], b.warp_w[v]);
+    for (int v = 0; v < b.V; ++v) cams[v] = make_devcam_for(c, b.cams[v], b.tile_w[v], b.tile_h[v]);
     launch_batch_cameras(cams, b.V, b.d_cams, s);
     const int launches = 9;
     if (flags & FGS_BATCH_GRAPH) {

@@ -62,7 +62,6 @@ struct DevCamera {
     int32_t shrink;
     float tau, ln_tau;
     float bg[3];
-    int32_t warp_shift;        // blend warps cover (1 << warp_shift) x (32 >> warp_shift) pixels
 };
 
 // Tree on the device (SoA; arrays padded to a multiple of 128 nodes).

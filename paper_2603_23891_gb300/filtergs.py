@@ -577,10 +577,14 @@ class Renderer:
 
         Greedy: all classes start at candidates[0]; each class in turn keeps the
         candidate with the lowest median batch time (CUDA events, graph replay).
+        Candidates of one tile shape differ in nothing that is rendered (the warp
+        width is without effect): the first of them is timed for all.
         Leaves the batch set up with the choice; returns (choice, ms)."""
         torch = _torch()
         classes = sorted({(c.width, c.height) for c in cams})
         choice = {cls: candidates[0] for cls in classes}
+        shapes = {tuple(c[:2]): c for c in reversed(candidates)}           # the first of each shape
+        others = [c for c in candidates[1:] if shapes[tuple(c[:2])] is c]
 
         def timed(ch):
             shapes = [ch[(c.width, c.height)] for c in cams]
@@ -603,7 +607,7 @@ class Renderer:
 
         best = timed(choice)
         for cls in classes:
-            for cand in candidates[1:]:
+            for cand in others:
                 trial = dict(choice)
                 trial[cls] = cand
                 t = timed(trial)
