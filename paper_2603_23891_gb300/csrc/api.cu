@@ -76,7 +76,6 @@ struct fgs_ctx {
     uint64_t pair_cap = 0;
     unsigned long long* keys0 = nullptr;
     unsigned long long* keys1 = nullptr;
-    uint32_t* vals0 = nullptr;
     uint32_t* vals1 = nullptr;
     float* kpc = nullptr;
     // tile-sized buffers
@@ -204,10 +203,9 @@ int ensure_pairs(fgs_ctx* c, uint64_t cap)
     if (cap == c->pair_cap) return FGS_OK;
     int r;
     c->pair_cap = 0;
-    const size_t n = (size_t)cap + 8;   // TMA reads an aligned superset of a slice
+    const size_t n = (size_t)cap;
     if ((r = grow(c, (void**)&c->keys0, n * 8))) return r;
     if ((r = grow(c, (void**)&c->keys1, n * 8))) return r;
-    if ((r = grow(c, (void**)&c->vals0, n * 4))) return r;
     if ((r = grow(c, (void**)&c->vals1, n * 4))) return r;
     if ((r = grow(c, (void**)&c->kpc, n * 4))) return r;
     c->pair_cap = cap;
@@ -482,7 +480,7 @@ int fgs_destroy(fgs_ctx* c)
     cudaDeviceSynchronize();
     void* bufs[] = {c->child_start, c->children, c->frontier0, c->frontier1, c->d_counter,
                     c->tree_mem, c->pbits, c->selbits, c->sel, c->splat, c->lb_compact, c->sel_cnt, c->foot,
-                    c->keys0, c->keys1, c->vals0, c->vals1, c->kpc, c->ranges, c->tile_cnt, c->large, c->lb_scan,
+                    c->keys0, c->keys1, c->vals1, c->kpc, c->ranges, c->tile_cnt, c->large, c->lb_scan,
                     c->G, c->img, c->keep, c->st, c->gsplat, c->heavy};
     for (void* p : bufs) free_ptr(p);
     for (float* p : c->ring) free_ptr(p);
@@ -623,14 +621,12 @@ int fgs_load_tree(fgs_ctx* c, const fgs_tree* t)
     DeviceGuard g(c->device);
     const size_t n_pad = align_up(N, kFilterTile);
     const uint32_t sh_stride = (uint32_t)align_up((size_t)K * 3, 4);
-    const size_t sz_mu = 3 * n_pad * 4, sz_cov = 6 * n_pad * 4, sz_op = n_pad * 4;
+    const size_t sz_mu = 3 * n_pad * 4, sz_cov = 6 * n_pad * 4;
     const size_t sz_sh = n_pad * sh_stride * 4, sz_leaf = n_pad / 32 * 4;
     const size_t sz_ap = (size_t)std::max<uint32_t>(D, 1) * n_pad * 4;
     size_t off = 0;
     const size_t o_mu = off; off = align_up(off + sz_mu, 256);
     const size_t o_cov = off; off = align_up(off + sz_cov, 256);
-    const size_t o_op = off; off = align_up(off + sz_op, 256);
-    const size_t o_lop = off; off = align_up(off + sz_op, 256);
     const size_t o_sh = off; off = align_up(off + sz_sh, 256);
     const size_t o_leaf = off; off = align_up(off + sz_leaf, 256);
     const size_t o_ap = off; off = align_up(off + sz_ap, 256);
@@ -651,8 +647,6 @@ int fgs_load_tree(fgs_ctx* c, const fgs_tree* t)
         FGS_CUDA(c, cudaMemcpy(base + o_mu + q * n_pad * 4, t->mu + q * N, N * 4, cudaMemcpyHostToDevice));
     for (int q = 0; q < 6; ++q)
         FGS_CUDA(c, cudaMemcpy(base + o_cov + q * n_pad * 4, t->cov + q * N, N * 4, cudaMemcpyHostToDevice));
-    FGS_CUDA(c, cudaMemcpy(base + o_op, t->opacity, N * 4, cudaMemcpyHostToDevice));
-    FGS_CUDA(c, cudaMemcpy(base + o_lop, t->ln_opacity, N * 4, cudaMemcpyHostToDevice));
     if (sh_stride == (uint32_t)K * 3) {
         FGS_CUDA(c, cudaMemcpy(base + o_sh, t->sh, N * sh_stride * 4, cudaMemcpyHostToDevice));
     } else {
@@ -692,8 +686,6 @@ int fgs_load_tree(fgs_ctx* c, const fgs_tree* t)
     dt.sh_stride = sh_stride;
     dt.mu = (const float*)(base + o_mu);
     dt.cov = (const float*)(base + o_cov);
-    dt.opacity = (const float*)(base + o_op);
-    dt.ln_opacity = (const float*)(base + o_lop);
     dt.sh = (const float*)(base + o_sh);
     dt.leaf_bits = (const uint32_t*)(base + o_leaf);
     dt.ap = (const uint32_t*)(base + o_ap);
@@ -1263,7 +1255,7 @@ int fgs_batch_setup(fgs_ctx* c, const fgs_camera* views, int n_views, const int3
     }
     if (pair_cap != b.pair_cap) {
         b.pair_cap = 0;
-        const size_t n = pair_cap + 8;
+        const size_t n = pair_cap;
         if ((r = grow(c, (void**)&b.items, 8 * n))) return r;
         if ((r = grow(c, (void**)&b.keys, 8 * n))) return r;
         if ((r = grow(c, (void**)&b.vals, 4 * n))) return r;

@@ -103,7 +103,7 @@ __device__ __forceinline__ float clamp_logit(float l)
 // (coefficients [n][K3] -> rows of sh_stride floats; vec: sh_stride == K3 and the source
 // 16-byte aligned, so one flat copy by 16-byte loads, four in flight a thread), the
 // boxes (a warp a chunk, from the parameters), the attributes (a thread a node).
-// Bound: HBM, 4 (11 + K3) bytes read and 4 (23 + sh_stride) written a node.  1.25M nodes
+// Bound: HBM, 4 (11 + K3) bytes read and 4 (21 + sh_stride) written a node.  1.25M nodes
 // of degree 3: 135 us as three launches with 4-byte SH copies.
 template <int kDeg>
 __global__ void __launch_bounds__(256) prep_kernel(DevTree t, ParamPtrs p, bool vec)
@@ -135,8 +135,6 @@ __global__ void __launch_bounds__(256) prep_kernel(DevTree t, ParamPtrs p, bool 
     chunk_boxes(p.mu, p.n, p.n, t.n_pad >> 7, const_cast<float4*>(t.cbox), tid, nt);
     float* mu = const_cast<float*>(t.mu);
     float* cov = const_cast<float*>(t.cov);
-    float* op = const_cast<float*>(t.opacity);
-    float* lop = const_cast<float*>(t.ln_opacity);
     const size_t np = t.n_pad, N = p.n;
     for (uint32_t n = tid; n < p.n; n += nt) {
 #pragma unroll
@@ -147,8 +145,6 @@ __global__ void __launch_bounds__(256) prep_kernel(DevTree t, ParamPtrs p, bool 
         for (int k = 0; k < 6; ++k) cov[k * np + n] = c6[k];
         const float den = fa(1.0f, exp_cw(-clamp_logit(p.logit[n])));
         const float a0 = fd(1.0f, den), la0 = -ln_cw(den);
-        op[n] = a0;
-        lop[n] = la0;
         float4* attr = const_cast<float4*>(t.attr) + 3 * (size_t)n;
         attr[0] = make_float4(p.mu[n], p.mu[N + n], p.mu[2 * N + n], a0);
         attr[1] = make_float4(c6[0], c6[1], c6[2], c6[3]);

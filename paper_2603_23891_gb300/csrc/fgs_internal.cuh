@@ -73,8 +73,6 @@ struct DevTree {
     uint32_t sh_stride;        // floats per node in sh (K*3 rounded up to 4)
     const float* mu;           // [3][n_pad]
     const float* cov;          // [6][n_pad]
-    const float* opacity;      // [n_pad]
-    const float* ln_opacity;   // [n_pad]
     const float* sh;           // [n_pad][sh_stride]
     const uint32_t* leaf_bits; // [n_pad/32]
     const uint32_t* ap;        // [depth][n_pad]
