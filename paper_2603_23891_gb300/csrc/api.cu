@@ -86,7 +86,8 @@ struct fgs_ctx {
     unsigned long long* lb_scan = nullptr;   // the tile scan's look-back entries
     uint32_t* heavy = nullptr;      // tiles the blend splits (kSplitTiles)
     float* G = nullptr;
-    float* G_host = nullptr;        // pinned, tile_cap
+    float* G_host = nullptr;        // pinned, G_host_cap (a calibration's)
+    size_t G_host_cap = 0;
     // image staging for host outputs: rgb planes + T
     size_t img_cap = 0;
     float* img = nullptr;
@@ -263,9 +264,6 @@ int ensure_tiles(fgs_ctx* c, size_t tiles, size_t pixels)
         if ((r = grow(c, (void**)&c->large, tiles * 4))) return r;
         if ((r = grow(c, (void**)&c->lb_scan, tile_scan_lookback_entries(tiles) * 8))) return r;
         if ((r = grow(c, (void**)&c->G, tiles * 4))) return r;
-        if (c->G_host) cudaFreeHost(c->G_host);
-        c->G_host = nullptr;
-        FGS_CUDA(c, cudaMallocHost((void**)&c->G_host, tiles * 4));
         c->tile_cap = tiles;
     }
     if (pixels > c->img_cap) {
@@ -1016,6 +1014,14 @@ int kpc_view(fgs_ctx* c, void* stream, bool force_3sigma, double* gbar_out, floa
     DeviceGuard g(c->device);
     cudaStream_t s = (cudaStream_t)stream;
     const DevCamera dc = make_devcam(c, force_3sigma);
+    const size_t tiles = (size_t)dc.tiles_x * dc.tiles_y;
+    if (tiles > c->G_host_cap) {
+        c->G_host_cap = 0;
+        if (c->G_host) FGS_CUDA(c, cudaFreeHost(c->G_host));
+        c->G_host = nullptr;
+        FGS_CUDA(c, cudaMallocHost((void**)&c->G_host, c->tile_cap * 4));
+        c->G_host_cap = c->tile_cap;
+    }
     enqueue_front(c, dc, s, nullptr);
     launch_blend_kpc(dc, c->ranges, c->vals1, c->splat, c->kpc, c->G, c->st, s);
     FGS_CUDA(c, cudaGetLastError());
@@ -1024,7 +1030,6 @@ int kpc_view(fgs_ctx* c, void* stream, bool force_3sigma, double* gbar_out, floa
     c->frame_kept = false;
     // the state and G with one wait (and G through pinned memory): two waits and two
     // copies into pageable memory took 40 us of a 1080p view's 320
-    const size_t tiles = (size_t)dc.tiles_x * dc.tiles_y;
     FGS_CUDA(c, cudaMemcpyAsync(c->G_host, c->G, tiles * 4, cudaMemcpyDeviceToHost, s));
     if ((r = read_state(c, s))) return r;
     if ((r = latched_status(c))) {

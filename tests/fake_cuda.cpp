@@ -12,7 +12,8 @@
 static std::vector<Op> g_queue;
 static std::vector<Op>* g_capture = nullptr;
 static cudaStream_t g_capture_stream = nullptr;
-static std::set<const void*> g_device, g_fresh;
+static std::set<const void*> g_fresh;
+static long g_pinned = 0;            // pinned blocks
 static long g_allocs = 0, g_fail_at = -1, g_execs = 0;
 static cudaError_t g_last = cudaSuccess;
 
@@ -34,7 +35,7 @@ static cudaError_t alloc(void** p, size_t n, bool device)
     *p = nullptr;
     if (g_allocs++ == g_fail_at) return g_last = cudaErrorMemoryAllocation;
     *p = calloc(n ? n : 1, 1);
-    if (device) g_device.insert(*p), g_fresh.insert(*p);
+    if (device) g_fresh.insert(*p);
     return cudaSuccess;
 }
 
@@ -44,7 +45,7 @@ void fake_fail_at(long n) { g_allocs = 0, g_fail_at = n; }      // the n-th allo
 long fake_allocs() { return g_allocs; }
 void fake_drain() { drain(); }
 long fake_graphs() { return g_execs; }
-long fake_device_blocks() { return (long)g_device.size(); }
+long fake_pinned() { return g_pinned; }
 
 // ---- the runtime
 void** __cudaRegisterFatBinary(void*) { static void* h; return &h; }
@@ -63,9 +64,14 @@ cudaError_t cudaGetLastError()
 }
 const char* cudaGetErrorString(cudaError_t) { return "fake"; }
 cudaError_t cudaMalloc(void** p, size_t n) { return alloc(p, n, true); }
-cudaError_t cudaMallocHost(void** p, size_t n) { return alloc(p, n, false); }
-cudaError_t cudaFree(void* p) { drain(); g_device.erase(p); free(p); return cudaSuccess; }
-cudaError_t cudaFreeHost(void* p) { drain(); free(p); return cudaSuccess; }
+cudaError_t cudaMallocHost(void** p, size_t n)
+{
+    const cudaError_t e = alloc(p, n, false);
+    g_pinned += e == cudaSuccess;
+    return e;
+}
+cudaError_t cudaFree(void* p) { drain(); g_fresh.erase(p); free(p); return cudaSuccess; }
+cudaError_t cudaFreeHost(void* p) { drain(); free(p); --g_pinned; return cudaSuccess; }
 cudaError_t cudaMemset(void* p, int v, size_t n)
 {
     drain();

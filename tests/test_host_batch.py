@@ -35,7 +35,7 @@ def api(tmp_path_factory):
             continue                                      # another file's entry point
         f, g = getattr(L, name), getattr(filtergs.lib(), name)
         f.argtypes, f.restype = g.argtypes, g.restype
-    for name in ("fake_allocs", "fake_records", "fake_graphs", "fake_device_blocks", "fake_nulls"):
+    for name in ("fake_allocs", "fake_records", "fake_graphs", "fake_pinned", "fake_nulls"):
         getattr(L, name).restype = C.c_long
     L.fake_fail_at.argtypes = [C.c_long]
     L.fake_record.argtypes = [C.c_long, C.c_void_p, C.c_void_p, C.c_void_p]
@@ -197,3 +197,23 @@ def test_failed_frame_buffers_are_not_used(api, ctx):
             if not failed:
                 break
         assert 0 < k < 99, name
+
+
+def test_a_frame_needs_no_pinned_memory(api, ctx):
+    """The calibration's pinned buffer is allocated by the first calibration, not by a camera
+    of more tiles, and a failure leaves frames as they were."""
+    rgb, gbar = C.c_void_p(0x1000), C.c_double()
+    _load(api, ctx)
+    small, large = (api.b._cams([synth.look_at_camera([0, -30.0, 9.0], [0, 0, 0], w, 48, 60.0)]) for w in (64, 640))
+    pinned = api.fake_pinned()
+    for cam in (small, large):
+        assert api.fgs_set_camera(ctx, cam) == 0 and api.fgs_render(ctx, None, rgb, None, 1, 0, None) == 0
+    assert api.fake_pinned() == pinned
+    api.fake_fail_at(0)
+    assert api.fgs_calibrate_view(ctx, None, C.byref(gbar), None, 0, None, 0) == api.b.FGS_ERR_NOMEM
+    api.fake_fail_at(-1)
+    assert api.fgs_render(ctx, None, rgb, None, 1, 0, None) == 0
+    for cam in (small, large):
+        assert api.fgs_set_camera(ctx, cam) == 0
+        assert api.fgs_calibrate_view(ctx, None, C.byref(gbar), None, 0, None, 0) == 0
+    assert api.fake_pinned() == pinned + 1
