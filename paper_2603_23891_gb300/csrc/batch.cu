@@ -160,9 +160,9 @@ __global__ void __launch_bounds__(256, 3) bpred_kernel(DevTree t, const DevCamer
 // cost a few loads and stores for all 4 together.  For the others the path of each node
 // is read once for all views (and the next such word's paths are prefetched), and the
 // ancestors' bits of two views that have a P bit in the word in one batch of independent
-// loads.  The survivors of every compaction tile are counted.  Bound: latency; a word at
-// a time over every view, an ancestor's bit looked up before the next, took 238 us for 8
-// views of 12.5M nodes; one view a turn 214, two 157, 4 words instead of 8 at a time 133.
+// loads.  The survivors of every compaction tile are counted.  Bound: latency of the
+// paths' and bits' loads (8 views of 12.5M nodes: 133 us; 238 with a word at a time over
+// every view, an ancestor's bit looked up before the next).
 __global__ void __launch_bounds__(256, 5) banc_kernel(DevTree t, int V, const uint32_t* __restrict__ pbits,
                                                       uint32_t* __restrict__ selbits, uint32_t* __restrict__ sel_cnt,
                                                       uint32_t sel_shift)

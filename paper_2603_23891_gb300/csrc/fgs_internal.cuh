@@ -30,13 +30,17 @@ constexpr int kSelTileWords = 256;        // words per counted tile (the Ancesto
 // (45) us, 2^25 104 / 37 (318), 2^27 1200 / 153 (1238); below, small dense batches need the
 // blocks.
 inline uint32_t batch_sel_shift(size_t words) { return words <= (1u << 22) ? 10u : 12u; }
+// Counters enough for every number of words up to this one.
+inline size_t batch_sel_counters(size_t words) { return (words + 1023) >> 10; }
 inline size_t batch_sel_tiles(size_t words)
 {
     const uint32_t shift = batch_sel_shift(words);
     return (words + (1u << shift) - 1) >> shift;
 }
 constexpr int kAncCacheWords = 4096;      // P-bit words of the lowest node ids kept in shared memory
-constexpr uint32_t kSplitTiles = 912;      // fewer tiles than that of a blend are split (6 an SM)
+// fewer tiles than that of a blend are split: the plain forward's resident CTAs, 6 x 152 (the
+// keeping form and the backward fit 5 an SM and share the list)
+constexpr uint32_t kSplitTiles = 912;
 constexpr int kProjectThreads = 128;      // threads per projection block
 constexpr int kProjectBlocks = 6;         // projection blocks an SM (registers; 160 KB of staged SH rows)
 constexpr int kProjThreads = 256;         // Gaussians per scatter tile

@@ -165,7 +165,7 @@ void launch_filter_pred(const DevTree& t, const DevCamera& cam, uint32_t* pbits,
 }
 
 // ---------------------------------------------------------------------------
-// Ancestor filter + compaction (persistent, dynamic tiles, decoupled look-back)
+// Ancestor filter
 // ---------------------------------------------------------------------------
 
 // Ancestor filter (§3.2): sel(n) = P(n) and no node of AP(n) has P.  One node per

@@ -5,6 +5,7 @@
 #include "fake_cuda.h"
 
 #include <cstdlib>
+#include <map>
 #include <cstring>
 #include <set>
 #include <vector>
@@ -13,6 +14,7 @@ static std::vector<Op> g_queue;
 static std::vector<Op>* g_capture = nullptr;
 static cudaStream_t g_capture_stream = nullptr;
 static std::set<const void*> g_fresh;
+static std::map<const void*, size_t> g_size;        // device blocks
 static long g_pinned = 0;            // pinned blocks
 static long g_allocs = 0, g_fail_at = -1, g_execs = 0;
 static cudaError_t g_last = cudaSuccess;
@@ -30,12 +32,18 @@ static void drain()
     for (auto& op : q) op();
 }
 
+size_t fake_size(const void* p)
+{
+    const auto i = g_size.find(p);
+    return i == g_size.end() ? 0 : i->second;
+}
+
 static cudaError_t alloc(void** p, size_t n, bool device)
 {
     *p = nullptr;
     if (g_allocs++ == g_fail_at) return g_last = cudaErrorMemoryAllocation;
     *p = calloc(n ? n : 1, 1);
-    if (device) g_fresh.insert(*p);
+    if (device) g_fresh.insert(*p), g_size[*p] = n;
     return cudaSuccess;
 }
 
@@ -70,7 +78,7 @@ cudaError_t cudaMallocHost(void** p, size_t n)
     g_pinned += e == cudaSuccess;
     return e;
 }
-cudaError_t cudaFree(void* p) { drain(); g_fresh.erase(p); free(p); return cudaSuccess; }
+cudaError_t cudaFree(void* p) { drain(); g_fresh.erase(p); g_size.erase(p); free(p); return cudaSuccess; }
 cudaError_t cudaFreeHost(void* p) { drain(); free(p); --g_pinned; return cudaSuccess; }
 cudaError_t cudaMemset(void* p, int v, size_t n)
 {

@@ -12,7 +12,7 @@ struct Record {
     int views;
     uint32_t n_pad;
     const void* rgb;
-    int null_args;                 // null buffers among the launch's
+    int null_args;                 // null (or too small) buffers among the launch's
     float t[64][3];                // the cameras' translations
 };
 
@@ -117,9 +117,12 @@ void launch_batch_front(const DevTree& t, const DevCamera* cams, int V, uint32_t
                         uint32_t* vals, unsigned long long, uint32_t* sel_cnt, unsigned long long* lb_scan,
                         uint2* ranges, FrameState* st, int, cudaStream_t s)
 {
+    const size_t words = (size_t)t.n_pad / 32 * V;
     record(0, cams, V, t.n_pad, nullptr,
            nulls(cams, tile_base, pbits, selbits, sel, splat, foot, tile_cnt, large, heavy, items, keys, vals, sel_cnt,
-                 lb_scan, ranges, st),
+                 lb_scan, ranges, st) +
+               (fake_size(pbits) < 4 * words) + (fake_size(selbits) < 4 * words) +
+               (fake_size(sel_cnt) < 4 * batch_sel_tiles(words)),
            s);
 }
 void launch_batch_blend(const DevCamera* cams, int V, uint32_t, const uint32_t* tile_base,

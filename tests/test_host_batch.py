@@ -217,3 +217,29 @@ def test_a_frame_needs_no_pinned_memory(api, ctx):
         assert api.fgs_set_camera(ctx, cam) == 0
         assert api.fgs_calibrate_view(ctx, None, C.byref(gbar), None, 0, None, 0) == 0
     assert api.fake_pinned() == pinned + 1
+
+
+def _flat_tree(api, n):
+    """A root and n - 1 leaves."""
+    from types import SimpleNamespace
+    parent = np.zeros(n, np.int32)
+    parent[0] = -1
+    ap = np.zeros((1, n), np.uint32)
+    ap[0, 0] = 0xFFFFFFFF
+    leaf = np.ones(n, np.uint8)
+    leaf[0] = 0
+    return api.b._TreeArrays(SimpleNamespace(
+        mu=np.zeros((3, n)), cov=np.ones((6, n)), opacity=np.full(n, 0.5), ln_opacity=np.full(n, np.log(0.5)),
+        sh=np.zeros((n, 1, 3)), sh_degree=0, parent=parent, is_leaf=leaf, ap=ap))
+
+
+@pytest.mark.parametrize("first,then", [(2101248, 2097152), (2097152, 2093056), (2101248, 4096)])
+def test_smaller_tree_with_the_same_set_up(api, ctx, first, then):
+    """64 views on both sides of 2^22 words of selection bits, where the counted tiles' width
+    changes: the set-up's bit arrays and counters hold every smaller tree's."""
+    assert api.fgs_load_tree(ctx, C.byref(_flat_tree(api, first).struct)) == 0
+    assert _setup(api, ctx, _cams(api, 64, 0.0)) == 0
+    assert api.fgs_load_tree(ctx, C.byref(_flat_tree(api, then).struct)) == 0
+    assert api.fgs_render_batch(ctx, None, C.c_void_p(0x1000), None, 0, None) == 0
+    api.fake_drain()
+    assert [_record(api, i)["nulls"] for i in range(api.fake_records())] == [0, 0]
