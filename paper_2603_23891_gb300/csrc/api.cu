@@ -133,7 +133,7 @@ struct fgs_ctx {
         float* splat = nullptr;
         uint4* foot = nullptr;
         unsigned long long *items = nullptr, *keys = nullptr, *lb_scan = nullptr;
-        uint32_t* sel_cnt = nullptr;              // selected entries per counted tile
+        uint32_t* sel_cnt = nullptr;              // selected entries per kBatchSelTileWords words
         uint32_t* vals = nullptr;
         uint2* ranges = nullptr;
         uint32_t *tile_cnt = nullptr, *large = nullptr, *heavy = nullptr;
@@ -1249,7 +1249,7 @@ int fgs_batch_setup(fgs_ctx* c, const fgs_camera* views, int n_views, const int3
     if ((r = grow(c, (void**)&b.d_img_off, 8 * (n_views + 1)))) return r;
     if ((r = grow(c, (void**)&b.pbits, 4 * n_words * n_views))) return r;
     if ((r = grow(c, (void**)&b.selbits, 4 * n_words * n_views))) return r;
-    if ((r = grow(c, (void**)&b.sel_cnt, 4 * batch_sel_counters(n_words * n_views)))) return r;
+    if ((r = grow(c, (void**)&b.sel_cnt, 4 * batch_sel_tiles(n_words * n_views)))) return r;
     if ((r = grow(c, (void**)&b.lb_scan, 8 * tile_scan_lookback_entries(b.total_tiles)))) return r;
     if (sel_cap != b.sel_cap) {
         b.sel_cap = 0;

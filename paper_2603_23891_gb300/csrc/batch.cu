@@ -164,8 +164,7 @@ __global__ void __launch_bounds__(256, 3) bpred_kernel(DevTree t, const DevCamer
 // paths' and bits' loads (8 views of 12.5M nodes: 133 us; 238 with a word at a time over
 // every view, an ancestor's bit looked up before the next).
 __global__ void __launch_bounds__(256, 5) banc_kernel(DevTree t, int V, const uint32_t* __restrict__ pbits,
-                                                      uint32_t* __restrict__ selbits, uint32_t* __restrict__ sel_cnt,
-                                                      uint32_t sel_shift)
+                                                      uint32_t* __restrict__ selbits, uint32_t* __restrict__ sel_cnt)
 {
     grid_dep_wait();
     const uint32_t lane = threadIdx.x & 31;
@@ -236,7 +235,7 @@ __global__ void __launch_bounds__(256, 5) banc_kernel(DevTree t, int V, const ui
                         const uint32_t b = lane ? b1 : b0;
                         const size_t at = (size_t)(vb + (lane ? v1 : v0)) * n_words + w;
                         selbits[at] = b;
-                        if (b) atomicAdd(sel_cnt + (at >> sel_shift), (uint32_t)__popc(b));
+                        if (b) atomicAdd(sel_cnt + at / kBatchSelTileWords, (uint32_t)__popc(b));
                     }
                 }
             }
@@ -333,8 +332,7 @@ void launch_batch_front(const DevTree& t, const DevCamera* cams, int V, uint32_t
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, bpred_kernel, 256, 0);
     launch_pdl(bpred_kernel, sms * (occ > 0 ? occ : 1), 256, 0, s, t, cams, V, pbits, begin);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, banc_kernel, 256, 0);
-    launch_pdl(banc_kernel, sms * (occ > 0 ? occ : 1), 256, 0, s, t, V, pbits, selbits, sel_cnt,
-               batch_sel_shift(all_words));
+    launch_pdl(banc_kernel, sms * (occ > 0 ? occ : 1), 256, 0, s, t, V, pbits, selbits, sel_cnt);
     launch_compact_counted_batch(selbits, all_words, sel, sel_cap, sel_cnt, st, s);
     const auto bproject = t.sh_degree == 0   ? bproject_kernel<0>
                           : t.sh_degree == 1 ? bproject_kernel<1>

@@ -23,20 +23,8 @@ constexpr int kSegSmem = 2048;            // pairs of a tile sorted by one block
 constexpr int kFilterTile = 4096;         // node arrays are padded to a multiple of this
 constexpr int kCompactWords = 1024;       // 32-bit selection words per compaction tile (32K nodes)
 constexpr int kSelTileWords = 256;        // words per counted tile (the Ancestor filter's sel_cnt)
-// The same in the batched form (its logarithm): 1024, and 4096 above 2^22 words.  A tile's
-// first slot is the sum of the counts before it, so the sums' work grows with the square
-// of the number of tiles; this keeps them within 2^15 up to the limit of 2^27 words.  One
-// word in 128 selected, 1024 / 4096 words a tile (look-back kernel): 2^22 words 11.7 / 9.7
-// (45) us, 2^25 104 / 37 (318), 2^27 1200 / 153 (1238); below, small dense batches need the
-// blocks.
-inline uint32_t batch_sel_shift(size_t words) { return words <= (1u << 22) ? 10u : 12u; }
-// Counters enough for every number of words up to this one.
-inline size_t batch_sel_counters(size_t words) { return (words + 1023) >> 10; }
-inline size_t batch_sel_tiles(size_t words)
-{
-    const uint32_t shift = batch_sel_shift(words);
-    return (words + (1u << shift) - 1) >> shift;
-}
+constexpr int kBatchSelTileWords = 1024;  // the same in the batched form
+inline size_t batch_sel_tiles(size_t words) { return (words + kBatchSelTileWords - 1) / kBatchSelTileWords; }
 constexpr int kAncCacheWords = 4096;      // P-bit words of the lowest node ids kept in shared memory
 // fewer tiles than that of a blend are split: the plain forward's resident CTAs, 6 x 152 (the
 // keeping form and the backward fit 5 an SM and share the list)
@@ -521,7 +509,7 @@ void launch_compact(const uint32_t* selbits, uint32_t n_words, uint32_t* sel, ui
 // The same result from the Ancestor filter's per-tile counts (one block a tile).
 void launch_compact_counted(const uint32_t* selbits, uint32_t n_words, uint32_t* sel, uint32_t cap,
                             const uint32_t* sel_cnt, FrameState* st, cudaStream_t s);
-// The same for a batch: sel_cnt per 2^batch_sel_shift(n_words) words.
+// The same for a batch: sel_cnt per kBatchSelTileWords words.
 void launch_compact_counted_batch(const uint32_t* selbits, uint32_t n_words, uint32_t* sel, uint32_t cap,
                                   const uint32_t* sel_cnt, FrameState* st, cudaStream_t s);
 // Projection (splat records, footprints) and the per-tile pair counts

@@ -336,14 +336,16 @@ __global__ void __launch_bounds__(256) compact_kernel(const uint32_t* __restrict
 }
 
 // Compaction of the frame's selection bits when the Ancestor filter has also
-// counted the selected nodes of every tile of 256 kW words (sel_cnt): one block per
-// tile, kW words per thread, takes the tile's first slot as the sum of the counts of
-// the tiles before it, so no block waits on another (no look-back chain); then
+// counted the selected nodes of every 256 kCnt words (sel_cnt): one block per
+// tile of 256 kW words, kW words per thread, takes the tile's first slot as the sum of
+// the counts before it, so no block waits on another (no look-back chain); then
 // popcounts, a block scan and a warp-cooperative bit expansion of each warp's words
-// (coalesced stores of ascending ids).  kW = 1 for one view; 4 or 16 for a batch
-// (batch_sel_shift), whose sums over many more tiles would otherwise grow with their square
-// (8 views of 12.5M nodes: 45 us with the look-back kernel, 27 with this one).
-template <int kW>
+// (coalesced stores of ascending ids).  kW = kCnt = 1 for one view; 4 for a batch, whose
+// sums over many more tiles would otherwise grow with their square (8 views of 12.5M
+// nodes: 45 us with the look-back kernel, 27 with this one), and from there on kW = 16
+// (batch_wide): a quarter of the sums for the same counts.  (Counts of 4096 words instead:
+// the Ancestor filter's increments meet, 32 views 356 -> 440 us.)
+template <int kW, int kCnt>
 __global__ void __launch_bounds__(256) compact_counted_kernel(const uint32_t* __restrict__ selbits,
                                                               uint32_t n_words, uint32_t* __restrict__ sel,
                                                               uint32_t cap, const uint32_t* __restrict__ sel_cnt,
@@ -365,7 +367,7 @@ __global__ void __launch_bounds__(256) compact_counted_kernel(const uint32_t* __
         wv[k] = w < n_words ? selbits[w] : 0u;               // issued before the prefix loads
     }
     uint32_t part = 0;
-    for (uint32_t j = tid; j < tile; j += 256u) part += sel_cnt[j];
+    for (uint32_t j = tid; j < tile * (kW / kCnt); j += 256u) part += sel_cnt[j];
     part = warp_sum_u32(part);
     if (lane == 0) s_warp_tot[warp] = part;
     __syncthreads();
@@ -419,15 +421,22 @@ void launch_compact_counted(const uint32_t* selbits, uint32_t n_words, uint32_t*
                             const uint32_t* sel_cnt, FrameState* st, cudaStream_t s)
 {
     const int n_tiles = (int)((n_words + kSelTileWords - 1) / kSelTileWords);
-    launch_pdl(compact_counted_kernel<kSelTileWords / 256>, n_tiles < 1 ? 1 : n_tiles, 256, 0, s, selbits, n_words, sel,
+    launch_pdl(compact_counted_kernel<kSelTileWords / 256, kSelTileWords / 256>, n_tiles < 1 ? 1 : n_tiles, 256, 0, s, selbits, n_words, sel,
                cap, sel_cnt, st);
 }
+
+// Words from which a block takes 4096 of them: below, the sums are the smaller part and dense
+// selections need the blocks.  One word in 128 selected, 1024 / 4096 words a block (look-back
+// kernel): 2^25 words 104 / 46 (309) us, 2^26 324 / 161 (613), 2^27 1148 / 663 (1217).
+static bool batch_wide(uint32_t n_words) { return n_words > (1u << 25); }
 
 void launch_compact_counted_batch(const uint32_t* selbits, uint32_t n_words, uint32_t* sel, uint32_t cap,
                                   const uint32_t* sel_cnt, FrameState* st, cudaStream_t s)
 {
-    const unsigned n_tiles = (unsigned)batch_sel_tiles(n_words);
-    const auto kernel = batch_sel_shift(n_words) == 10u ? compact_counted_kernel<4> : compact_counted_kernel<16>;
+    constexpr int kCnt = kBatchSelTileWords / 256;
+    const uint32_t tile = batch_wide(n_words) ? 4096u : (uint32_t)kBatchSelTileWords;
+    const uint32_t n_tiles = (uint32_t)(((uint64_t)n_words + tile - 1) / tile);
+    const auto kernel = batch_wide(n_words) ? compact_counted_kernel<16, kCnt> : compact_counted_kernel<4, kCnt>;
     launch_pdl(kernel, n_tiles < 1 ? 1u : n_tiles, 256, 0, s, selbits, n_words, sel, cap, sel_cnt, st);
 }
 

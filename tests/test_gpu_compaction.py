@@ -19,8 +19,9 @@ using namespace fgs;
 #define OK(x) do { if ((x) != cudaSuccess) { std::printf("cuda error, line %d\n", __LINE__); return 1; } } while (0)
 int main()
 {
-    const uint32_t sizes[] = {1, 31, 255, 1023, 1024, 1025, 40000, (1u << 22) - 1, 1u << 22, (1u << 22) + 1, (1u << 22) + 4097};
-    const uint32_t max_words = (1u << 22) + 4097, max_cap = 10u << 20;
+    const uint32_t sizes[] = {1, 31, 255, 1023, 1024, 1025, 40000, 1u << 22, (1u << 25) - 1, 1u << 25, (1u << 25) + 1,
+                              (1u << 25) + 1025, (1u << 25) + 4097};
+    const uint32_t max_words = (1u << 25) + 4097, max_cap = 20u << 20;
     uint32_t *d_bits, *d_sel, *d_cnt;
     FrameState* st;
     OK(cudaMalloc(&d_bits, 4ull * max_words));
@@ -34,8 +35,8 @@ int main()
             for (int full = 0; full < 2; ++full) {
                 std::vector<uint32_t> bits(n), want, cnt(batch_sel_tiles(n));
                 for (uint32_t w = 0; w < n; ++w) {
-                    bits[w] = dense ? (n > 1000000 ? next() & next() & next() & next() : next()) : next() % 97 == 0 ? next() : 0;
-                    cnt[w >> batch_sel_shift(n)] += (uint32_t)__builtin_popcount(bits[w]);
+                    bits[w] = dense ? (n > 1000000 ? next() & next() & next() & next() & next() & next() : next()) : next() % 997 == 0 ? next() : 0;
+                    cnt[w / kBatchSelTileWords] += (uint32_t)__builtin_popcount(bits[w]);
                     for (int b = 0; b < 32; ++b)
                         if (bits[w] >> b & 1) want.push_back(32 * w + b);
                 }

@@ -235,8 +235,8 @@ def _flat_tree(api, n):
 
 @pytest.mark.parametrize("first,then", [(2101248, 2097152), (2097152, 2093056), (2101248, 4096)])
 def test_smaller_tree_with_the_same_set_up(api, ctx, first, then):
-    """64 views on both sides of 2^22 words of selection bits, where the counted tiles' width
-    changes: the set-up's bit arrays and counters hold every smaller tree's."""
+    """A set-up's bit arrays and counters hold every smaller tree's, 64 views of 2^22 words and
+    fewer."""
     assert api.fgs_load_tree(ctx, C.byref(_flat_tree(api, first).struct)) == 0
     assert _setup(api, ctx, _cams(api, 64, 0.0)) == 0
     assert api.fgs_load_tree(ctx, C.byref(_flat_tree(api, then).struct)) == 0
