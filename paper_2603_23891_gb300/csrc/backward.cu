@@ -619,7 +619,7 @@ struct GradPtrs {
 // lanes of a quarter-warp hit different banks.  Bound: the latency of the rows (8 blocks
 // of 2 warps an SM, by shared memory and registers), so the next group's rows are copied
 // and its other inputs prefetched while this one is computed (537K Gaussians of degree 3:
-// 73 -> 58 us; accumulating 264K: 36 -> 24).
+// 73 -> 54 us; accumulating 264K: 36 -> 33).
 __device__ __forceinline__ void cp_async4(float* smem, const float* gmem)
 {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(smem)), "l"(gmem)

@@ -421,8 +421,9 @@ void launch_compact_counted(const uint32_t* selbits, uint32_t n_words, uint32_t*
                             const uint32_t* sel_cnt, FrameState* st, cudaStream_t s)
 {
     const int n_tiles = (int)((n_words + kSelTileWords - 1) / kSelTileWords);
-    launch_pdl(compact_counted_kernel<kSelTileWords / 256, kSelTileWords / 256>, n_tiles < 1 ? 1 : n_tiles, 256, 0, s, selbits, n_words, sel,
-               cap, sel_cnt, st);
+    constexpr int kW = kSelTileWords / 256;
+    launch_pdl(compact_counted_kernel<kW, kW>, n_tiles < 1 ? 1 : n_tiles, 256, 0, s, selbits, n_words, sel, cap, sel_cnt,
+               st);
 }
 
 // Words from which a block takes 4096 of them: below, the sums are the smaller part and dense

@@ -21,8 +21,9 @@
 //    radix passes in shared memory, and a larger bucket in chunks between the
 //    bucket and the tile's slots of the key output.  The radix passes cover the
 //    leading 16 bits of the depths' offsets from the bucket's nearest (two passes
-//    instead of up to four: 49 -> 34 us for 1.13M pairs of 1M blobs at 1080p, 75 ->
-//    45 us for a city frame with buckets above kSegSmem; issue and barrier bound),
+//    instead of up to four: 49 -> 34 us for 1.13M pairs of 1M blobs at 1080p, 31 with
+//    four blocks an SM, 75 -> 45 us for a city frame with buckets above kSegSmem; issue
+//    and barrier bound),
 //    and the runs of equal ones, which keep the scatter's order, are ordered
 //    where they lie; a bucket whose leading bits are crowded is sorted by every bit.
 //    The sorted bucket is written as keys
@@ -1006,7 +1007,8 @@ __device__ __forceinline__ void list_heavy(uint32_t n, uint32_t split, uint32_t 
 }
 
 // Four blocks an SM (64 registers, a few words spilled): 1.13M pairs in 30.1 us, against 33.5
-// with three and 31.3 with five; 7M pairs 139, 157 and 149.
+// with three and 31.3 with five (31.4 since crowded depths are looked for); 7M pairs 139, 157
+// and 149.
 __global__ void __launch_bounds__(kSegThreads, 4) segsort_kernel(const uint2* __restrict__ ranges,
                                                               uint32_t n_tiles,
                                                               const uint32_t* __restrict__ large,

@@ -172,8 +172,7 @@ struct Rows {
 // asynchronously, whole rows by consecutive lanes (a lane's own 16-byte loads touch half
 // of each sector and wait where they are used), while the warp counts its pairs and the
 // next 32 entries' attributes are on their way.  537K Gaussians of degree 3 (450K emitting,
-// 1.13M pairs): 44 -> 37 us, 157 MB; 8 views, 7.5M entries: 258 us, 1.9 GB, at HBM's rate
-// before and after.
+// 1.13M pairs): 44 -> 37 us, 157 MB; 8 views, 7.5M entries: 258 -> 252 us, 1.45 GB of DRAM.
 template <int kDeg, class View>
 __device__ __forceinline__ void project_walk(const DevTree& t, const uint32_t* __restrict__ sel, Rows<kDeg>& S,
                                              float* __restrict__ splat, uint4* __restrict__ foot,
