@@ -608,7 +608,8 @@ struct GradPtrs {
 // Chain rule for selected Gaussian m (node sel[m]): splat gradient -> mean,
 // log-scale, quaternion, logit, SH.  Each node appears once in the selection,
 // so plain stores do, and loads and stores when accumulating (reductions in global memory
-// flush subnormal numbers; two accumulating views of 375K nodes 410 us with them, 418 so).
+// flush subnormal numbers; two accumulating views of 375K nodes 408 us with them, 418 so,
+// of degree 2 402 and 406, 437 with one old value in flight at a time).
 //
 // Each warp takes 32 consecutive selected Gaussians per iteration, one per
 // lane.  Their SH rows (3 K floats each, contiguous per node) are staged in
@@ -629,14 +630,6 @@ __device__ __forceinline__ void cp_async16(float* smem, const float* gmem)
 {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(smem)), "l"(gmem)
                  : "memory");
-}
-
-// A gradient stored, or added to what is there (each node appears once).  By load and
-// store: reductions in global memory flush subnormal numbers.
-template <bool kAdd>
-__device__ __forceinline__ void put(float* p, float v)
-{
-    *p = kAdd ? *p + v : v;
 }
 
 __device__ __forceinline__ void prefetch_l2(const float* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
@@ -873,10 +866,29 @@ __global__ void __launch_bounds__(kPbWarps * 32, 16 / kPbWarps) project_bwd_kern
                 }
             }
         } else {
-            for (int i = 0; i < K3; ++i) {
-                const uint32_t idx = (uint32_t)i * 32u + lane, r = idx / K3, k = idx - r * K3;
-                const uint32_t nr = __shfl_sync(0xffffffffu, n, r);
-                if (base + r < M) put<kAccumulate>(gr.sh + (size_t)nr * K3 + k, rows[r * RS + k]);
+            constexpr int kB = K3 % 9 == 0 ? 9 : K3 % 6 == 0 ? 6 : 3;
+            auto at = [&](int i, uint32_t& r, uint32_t& k) {
+                const uint32_t idx = (uint32_t)i * 32u + lane;
+                r = idx / K3;
+                k = idx - r * K3;
+                return gr.sh + (size_t)__shfl_sync(0xffffffffu, n, r) * K3 + k;
+            };
+#pragma unroll 1
+            for (int i0 = 0; i0 < K3; i0 += kB) {
+                uint32_t r, k;
+                float held[kB] = {};
+                if (kAccumulate)
+#pragma unroll
+                    for (int j = 0; j < kB; ++j) {
+                        const float* p = at(i0 + j, r, k);
+                        if (base + r < M) held[j] = *p;
+                    }
+#pragma unroll
+                for (int j = 0; j < kB; ++j) {
+                    float* p = at(i0 + j, r, k);
+                    const float g = rows[r * RS + k];
+                    if (base + r < M) *p = kAccumulate ? held[j] + g : g;
+                }
             }
         }
         __syncwarp();
